@@ -145,8 +145,8 @@ struct DecodeParams {
   const uint8_t *wstream;  // bf16 weight chunks in WeightSchedule<D> order, block after block
   uint32_t layer_bytes;    // WeightSchedule<D>::kLayerBytes
   const float *lparams;  // [n_layers][LayerParamLayout::stride(D)]
-  const float *emb;      // [T][D - d_spe]
-  const float *spe;      // [T][d_spe]
+  const float4 *xtab;    // [D / 4][Tp] columns 4c .. 4c + 3 of the row's token: its embedding in the first
+                         // D - d_spe columns (scaled by h_t), then its positional encoding
   const float *w_d1;     // [D]
   float b_d1;
   const float *w_out;    // [T][n]

@@ -45,7 +45,7 @@ struct aecct_handle {
   uint32_t layer_bytes = 0;
   int n_chunks = 0;
   ChunkDesc chunks[32] = {};  // WeightSchedule<d> order
-  float *lparams = nullptr, *emb = nullptr, *spe = nullptr, *w_d1 = nullptr, *w_out = nullptr, *b_out = nullptr;
+  float *lparams = nullptr, *xtab = nullptr, *w_d1 = nullptr, *w_out = nullptr, *b_out = nullptr;
   uint32_t *hbits = nullptr, *mask_info[2] = {nullptr, nullptr};
   int hwords = 0;
   uint16_t *mask_list[2] = {nullptr, nullptr};
@@ -798,12 +798,20 @@ int aecct_create(const aecct_model_desc *desc, aecct_handle **out) {
       return AECCT_ERR_UNSUPPORTED;
     }
   }
+  // embedding and positional encoding in one table, [D / 4][Tp][4]: row by row of a codeword (a padding
+  // row stays 0), so that the rows of a warp are next to each other
   const int de = D - d.d_spe;
+  std::vector<float> xtab((size_t)D * h->Tp, 0.0f);
+  for (int row = 0; row < h->Tp; ++row) {
+    const size_t t = perm[row];
+    if (t == 0xFFFFu) continue;
+    for (int c = 0; c < D; ++c)
+      xtab[((size_t)(c / 4) * h->Tp + row) * 4 + c % 4] = c < de ? d.emb[t * de + c] : d.spe[t * d.d_spe + (c - de)];
+  }
   if ((rc = dev_upload(h, &h->wstream, gpu_unpack ? nullptr : reinterpret_cast<const uint8_t *>(ws.data()),
                       (size_t)d.n_layers * off)) ||
       (rc = dev_upload(h, &h->lparams, lpv.data(), lpv.size())) ||
-      (rc = dev_upload(h, &h->emb, d.emb, (size_t)T * de)) ||
-      (rc = dev_upload(h, &h->spe, d.spe, (size_t)T * d.d_spe)) ||
+      (rc = dev_upload(h, &h->xtab, xtab.data(), xtab.size())) ||
       (rc = dev_upload(h, &h->w_d1, d.w_d1, (size_t)D)) ||
       (rc = dev_upload(h, &h->w_out, d.w_out, (size_t)T * n)) ||
       (rc = dev_upload(h, &h->b_out, d.b_out, (size_t)n)) ||
@@ -857,7 +865,7 @@ static DecodeParams decode_params(const aecct_handle *h, int64_t B, const float 
   p.n_clusters = static_cast<int>(p.n_groups < h->max_clusters ? p.n_groups : h->max_clusters);
   p.y = y_dev, p.bits = bits_dev, p.syn = syn_dev, p.logits = logits_dev;
   p.wstream = h->wstream, p.layer_bytes = h->layer_bytes;
-  p.lparams = h->lparams, p.emb = h->emb, p.spe = h->spe, p.w_d1 = h->w_d1, p.b_d1 = h->b_d1;
+  p.lparams = h->lparams, p.xtab = reinterpret_cast<const float4 *>(h->xtab), p.w_d1 = h->w_d1, p.b_d1 = h->b_d1;
   p.w_out = h->w_out, p.b_out = h->b_out, p.hbits = h->hbits, p.hwords = h->hwords;
   p.perm = h->perm, p.pos = h->pos;
   p.plan_blob = reinterpret_cast<const uint4 *>(h->plan_blob), p.plan_bytes = h->plan_bytes;
