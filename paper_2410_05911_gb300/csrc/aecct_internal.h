@@ -17,7 +17,6 @@ constexpr int kOutBitsBytes = 4096;      // decoded bits of the codewords one CT
 constexpr int kMaxTasks = 16;            // attention tasks per warp (task mode)
 constexpr int kQSlots = 8;               // d = 128 tasks run off their quadrant (2 KB Q/A slots in W2)
 constexpr int kMaxGroups = 32;           // 32-row query groups per CTA (task mode)
-constexpr int kTaskCache = 64;           // attention scores per task kept in TMEM (task mode)
 constexpr int kRowCache = 64;            // attention scores per (row, head) kept in TMEM (row mode)
 
 // One weight chunk of a block: rows [n0, n0 + nrows) and K columns [k0, k0 + kcols) of the
@@ -228,13 +227,18 @@ struct SmemLayout {
   static constexpr uint32_t kOffMisc = kOffBar + 256;  // tmem base, abort flag, peer bases, copy count
   static constexpr uint32_t kTotal = kOffMisc + 256;
   // QKV / FFN1 accumulators in [0, 4D) (x parked in [3D, 4D) during attention).  Attention
-  // scores are cached in TMEM between the two softmax passes: task mode from kTaskCacheCol
-  // (4 warps per lane quadrant x kTaskCache columns: [256, 512) for d <= 64, the dead K and V
-  // accumulator columns [128, 384) for d = 128); row mode kRowCache columns per column slice
+  // scores are cached in TMEM between the two softmax passes.  Task mode: kTaskCache columns for each
+  // of the 4 warps of a lane quadrant, in whatever is dead or free then: d = 128 the K and V
+  // accumulators [128, 384) (Q and A stay in [0, 128)); d <= 64 (Q, K, V in shared memory) 96 keys a
+  // warp, so that a word of up to 96 tokens never recomputes a score: d = 64 [0, 192) and [256, 448)
+  // around the parked residual, d = 32 [128, 512).  Row mode: kRowCache columns per column slice
   // from kRowCacheCol, each thread in its own row's lane (d = 128: [128, 384); d <= 64:
   // [256, 512)).
   static constexpr uint32_t kTmemCols = 512u;
-  static constexpr uint32_t kTaskCacheCol = (D == 128) ? 128u : 256u;
+  static constexpr int kTaskCache = D == 128 ? 64 : 96;
+  __host__ __device__ static constexpr uint32_t task_cache_col(uint32_t slice) {
+    return D == 128 ? 128u + 64u * slice : D == 32 ? 128u + 96u * slice : slice < 2u ? 96u * slice : 64u + 96u * slice;
+  }
   static constexpr uint32_t kRowCacheCol = (D == 128) ? 128u : 256u;
 };
 

@@ -604,7 +604,15 @@ int aecct_create(const aecct_model_desc *desc, aecct_handle **out) {
         puinfo[gi * 2 + ring] = static_cast<uint32_t>((start << 8) | uni.size());
         ucount[gi * 2 + ring] = static_cast<int>(uni.size());
         for (int u : uni) pulist.push_back(static_cast<uint8_t>(pos[u]));
-        while (pulist.size() % 16) pulist.push_back(0);
+        // the last 16-key block is filled up with keys that no lane holds: where its rows are
+        // consecutive, the rows that follow, so that the kernel's fixed-offset path takes the block
+        // (every row of the CTA is written, whether it holds a token or not), else the last row again
+        if (pulist.size() % 16) {
+          const size_t b0 = pulist.size() / 16 * 16;
+          bool run = grps[gi].cwrow0 + pulist[b0] + 16 <= kRows;
+          for (size_t i = b0 + 1; i < pulist.size(); ++i) run = run && pulist[i] == pulist[i - 1] + 1;
+          while (pulist.size() % 16) pulist.push_back(static_cast<uint8_t>(pulist.back() + (run ? 1 : 0)));
+        }
         for (int ln = 0; ln < grps[gi].lanes; ++ln) {
           std::vector<uint8_t> mine(T, 0);
           for (uint16_t u : nb[ring][perm[off0 + ln]]) mine[u] = 1;

@@ -446,13 +446,51 @@ __device__ __forceinline__ bool contiguous(const uint4 &w) {
   return w.x == pat && w.y == pat + 0x04040404u && w.z == pat + 0x08080808u && w.w == pat + 0x0C0C0C0Cu;
 }
 
-// One HPSA head for a query group (task mode).  Every lane walks the group's union key list in
-// ascending token order; the loads are warp-uniform (shared-memory broadcasts).  A lane only
-// folds in the keys of its own set (membership bit), so for each query the max, the sum l and
-// the weighted sum num see exactly its keys, in ascending order, as in the canonical definition.
-// Keys go two at a time through f32x2 instructions: the two lanes of a pair are independent
-// computations, and the folds into l and num stay sequential in key order.
+// The same head where a V row of the CTA is not finite (parameters near the end of the fp32 range): a
+// lane folds in its own keys only, so that an infinity stays with the queries that attend to it.  q
+// comes in and A goes out in `qa`.
 template <int DH, uint32_t STRIDE>
+static __device__ __noinline__ void hpsa_task_any(float *qa, const uint4 mask, int cnt, const uint4 *ul,
+                                                  const uint8_t *rows, uint32_t kslot, float scale) {
+  const uint8_t *row = reinterpret_cast<const uint8_t *>(ul);
+  auto member = [&](int k) {
+    const uint32_t word = k < 64 ? (k < 32 ? mask.x : mask.y) : (k < 96 ? mask.z : mask.w);
+    return ((word >> (k & 31)) & 1u) != 0u;
+  };
+  auto score = [&](int k) {
+    const float *kk = reinterpret_cast<const float *>(rows + row[k] * STRIDE + kslot);
+    float d0 = 0.0f, d1 = 0.0f;
+    for (int i = 0; i < DH; i += 2) d0 = __fmaf_rn(qa[i], kk[i], d0), d1 = __fmaf_rn(qa[i + 1], kk[i + 1], d1);
+    return __fmul_rn(__fadd_rn(d0, d1), scale);
+  };
+  float mx = -INFINITY, lsum = 0.0f, num[DH];
+  for (int i = 0; i < DH; ++i) num[i] = 0.0f;
+  for (int k = 0; k < cnt; ++k)
+    if (member(k)) mx = fmaxf(mx, score(k));
+  for (int k = 0; k < cnt; ++k) {
+    if (!member(k)) continue;
+    const float pr = exp2_series(__fsub_rn(score(k), mx));
+    const float *vv = reinterpret_cast<const float *>(rows + row[k] * STRIDE + kslot) + DH;
+    lsum = __fadd_rn(lsum, pr);
+    for (int i = 0; i < DH; ++i) num[i] = __fmaf_rn(pr, vv[i], num[i]);
+  }
+  const float inv = __fdiv_rn(1.0f, lsum);
+  for (int i = 0; i < DH; ++i) qa[i] = __fmul_rn(num[i], inv);
+}
+
+// One HPSA head for a query group (task mode).  Every lane walks the group's union key list in
+// ascending token order; the loads are warp-uniform (shared-memory broadcasts).  A key that is not
+// in the lane's own set (membership bit) gets the score -inf and so, exactly, the probability 0:
+// it changes neither the maximum nor l nor num (x + 0 and fma(0, v, x) are x for finite v), and for
+// each query the max, the sum l and the weighted sum num see its keys in ascending order, as in
+// the canonical definition, without a branch per key.  V has to be finite (the caller checks).
+// Keys go U at a time; the two lanes of a paired instruction are independent computations, and the
+// folds into l and num stay sequential in key order.
+// Bound by issue slots, FMA pipe and shared-memory loads at 50 to 70% each.  With a divergent branch
+// around every maximum and fold, a key step of three warps a scheduler took 93.8 cycles at d_h = 16
+// (63 keys) and 64 at d_h = 4 (15 keys), now 79 and 48; U = 2 in place of 4 at d_h = 16: 82.
+// BCH(63,36) 546.8 -> 496.6 ms for 262,144 words, Polar(64,32) 46.7 -> 45.5 ms for 65,536.
+template <int DH, uint32_t STRIDE, int CACHE>
 __device__ __forceinline__ void hpsa_task(const float *q, const uint4 mask, int cnt, const uint4 *ul,
                                           const uint8_t *rows, uint32_t kslot, float scale, uint32_t tcache,
                                           float *A) {
@@ -468,74 +506,62 @@ __device__ __forceinline__ void hpsa_task(const float *q, const uint4 mask, int 
     }
     return __fadd_rn(d.x, d.y);
   };
-  auto dot2 = [&](const float4 *ka, const float4 *kb) -> float2 { return make_float2(dot(ka), dot(kb)); };
   const float2 sc = make_float2(scale, scale);
-  constexpr int U = (DH >= 16) ? 2 : 4;  // keys per step (registers: U x d_h fp32 of K or V)
+  constexpr int U = DH >= 8 ? 4 : 8;  // keys per step (registers: U x d_h fp32 of K or V)
   // membership bits of a 16-key block (jb is a multiple of 16)
   auto segment = [&](int jb) -> uint32_t {
     const uint32_t word = jb < 64 ? (jb < 32 ? mask.x : mask.y) : (jb < 96 ? mask.z : mask.w);
     return word >> (jb & 16);
   };
-  // pass 1: maximum score over the lane's keys.  The scores sigma = fl(dot * scale) of the first
-  // kTaskCache keys also go to this warp's TMEM columns, so that pass 2 reads them back
-  // instead of reloading K and recomputing the dot products (same values, bit for bit).
+  // the scores of keys k0 .. k0 + U - 1 of a block (sigma = fl(dot * scale), -inf outside the lane's
+  // set); CONTIG: the block's keys are consecutive rows (addresses at fixed offsets from the first);
+  // DENSE: every lane holds all of the block's keys (no membership tests)
+  auto scores = [&](auto contig_tag, auto dense_tag, const uint4 &w, uint32_t seg, int k0, float *sg) {
+    constexpr bool CONTIG = decltype(contig_tag)::value, DENSE = decltype(dense_tag)::value;
+    float4 kk[U][DH / 4];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const float4 *kp = CONTIG ? kptr(static_cast<int>(w.x & 0xFFu) + k0 + k) : kptr(byte_at(w, k0 + k));
+#pragma unroll
+      for (int i = 0; i < DH / 4; ++i) kk[k][i] = kp[i];
+    }
+#pragma unroll
+    for (int k = 0; k < U; k += 2) {
+      const float2 v = mul2(make_float2(dot(kk[k]), dot(kk[k + 1])), sc);
+      sg[k] = (DENSE || ((seg >> (k0 + k)) & 1u)) ? v.x : -INFINITY;
+      sg[k + 1] = (DENSE || ((seg >> (k0 + k + 1)) & 1u)) ? v.y : -INFINITY;
+    }
+  };
+  // pass 1: maximum score over the lane's keys.  The scores of the first CACHE keys also go to
+  // this warp's TMEM columns, so that pass 2 reads them back instead of reloading K and recomputing
+  // the dot products (same values, bit for bit).
   float mx = -INFINITY;
+#pragma unroll 1
   for (int jb = 0; jb < cnt; jb += 16) {
     const uint4 w = ul[jb >> 4];
     const uint32_t seg = segment(jb);
-    const int nk = min(16, cnt - jb);
+    const int nk = cnt - jb;
     float sgs[16];
-    // the 16 keys of a full segment; DENSE: every lane holds all of them (no membership tests);
-    // CONTIG: the keys are 16 consecutive rows (addresses at fixed offsets from the first)
-    const bool contig = nk == 16 && contiguous(w);
-    auto full_segment = [&](auto dense_tag, auto contig_tag) {
-      constexpr bool DENSE = decltype(dense_tag)::value, CONTIG = decltype(contig_tag)::value;
+    auto block = [&](auto contig_tag, auto dense_tag) {
 #pragma unroll
       for (int k0 = 0; k0 < 16; k0 += U) {
-        float4 kk[U][DH / 4];
+        if (k0 == 0 || decltype(dense_tag)::value || k0 < nk) {
+          scores(contig_tag, dense_tag, w, seg, k0, sgs + k0);
 #pragma unroll
-        for (int k = 0; k < U; ++k) {
-          const float4 *kp = CONTIG ? kptr(static_cast<int>(w.x & 0xFFu) + k0 + k) : kptr(byte_at(w, k0 + k));
+          for (int k = 0; k < U; ++k) mx = fmaxf(mx, sgs[k0 + k]);
+        } else {
 #pragma unroll
-          for (int i = 0; i < DH / 4; ++i) kk[k][i] = kp[i];
-        }
-#pragma unroll
-        for (int k = 0; k < U; k += 2) {
-          const float2 sg = mul2(dot2(kk[k], kk[k + 1]), sc);
-          sgs[k0 + k] = sg.x, sgs[k0 + k + 1] = sg.y;
-          if (DENSE || ((seg >> (k0 + k)) & 1u)) mx = fmaxf(mx, sg.x);
-          if (DENSE || ((seg >> (k0 + k + 1)) & 1u)) mx = fmaxf(mx, sg.y);
+          for (int k = 0; k < U; ++k) sgs[k0 + k] = -INFINITY;
         }
       }
     };
-    if (nk == 16) {
-      const bool dense = __all_sync(0xffffffffu, (seg & 0xFFFFu) == 0xFFFFu);
-      if (contig) {
-        if (dense) full_segment(std::true_type{}, std::true_type{});
-        else full_segment(std::false_type{}, std::true_type{});
-      } else {
-        if (dense) full_segment(std::true_type{}, std::false_type{});
-        else full_segment(std::false_type{}, std::false_type{});
-      }
+    if (contiguous(w)) {
+      if (nk >= 16 && __all_sync(0xffffffffu, (seg & 0xFFFFu) == 0xFFFFu)) block(std::true_type{}, std::true_type{});
+      else block(std::true_type{}, std::false_type{});
     } else {
-#pragma unroll
-      for (int k = 0; k < 16; k += 2) {
-        if (k < nk) {
-          const int k1 = (k + 1 < nk) ? k + 1 : k;
-          float4 ka[DH / 4], kb[DH / 4];
-          const float4 *pa = kptr(byte_at(w, k)), *pb = kptr(byte_at(w, k1));
-#pragma unroll
-          for (int i = 0; i < DH / 4; ++i) ka[i] = pa[i], kb[i] = pb[i];
-          const float2 sg = mul2(dot2(ka, kb), sc);
-          sgs[k] = sg.x, sgs[k + 1] = sg.y;
-          if (((seg >> k) & 1u)) mx = fmaxf(mx, sg.x);
-          if (k1 != k && ((seg >> k1) & 1u)) mx = fmaxf(mx, sg.y);
-        } else {
-          sgs[k] = 0.0f, sgs[k + 1] = 0.0f;
-        }
-      }
+      block(std::false_type{}, std::false_type{});
     }
-    if (jb < kTaskCache) tmem_st<16>(tcache + jb, sgs);
+    if (jb < CACHE) tmem_st<16>(tcache + jb, sgs);
   }
   tmem_wait_st();
   // pass 2: p = 2^(sigma - m), l += p, num += p v, in key order
@@ -543,10 +569,6 @@ __device__ __forceinline__ void hpsa_task(const float *q, const uint4 mask, int 
   float num[DH];
 #pragma unroll
   for (int i = 0; i < DH; ++i) num[i] = 0.0f;
-  // sigma - m for a pair of dot products (scalar: a product followed by a subtraction)
-  auto shifted = [&](float2 d) {
-    return make_float2(__fsub_rn(__fmul_rn(d.x, scale), mx), __fsub_rn(__fmul_rn(d.y, scale), mx));
-  };
   auto fold = [&](float pr, const float4 *vv) {
     lsum = __fadd_rn(lsum, pr);
     const float2 pp = make_float2(pr, pr);
@@ -557,26 +579,23 @@ __device__ __forceinline__ void hpsa_task(const float *q, const uint4 mask, int 
       num[4 * i] = lo.x, num[4 * i + 1] = lo.y, num[4 * i + 2] = hi.x, num[4 * i + 3] = hi.y;
     }
   };
+#pragma unroll 1
   for (int jb = 0; jb < cnt; jb += 16) {
     const uint4 w = ul[jb >> 4];
-    const uint32_t seg = segment(jb);
-    const int nk = min(16, cnt - jb);
-    if (jb < kTaskCache) {
+    const int nk = cnt - jb;
+    if (jb < CACHE) {
       float sgs[16];
       tmem_ld<16>(tcache + jb, sgs);
       tmem_wait_ld();
-      // DENSE: a full segment held by every lane (no membership or range tests); CONTIG: a full
-      // segment of 16 consecutive rows
-      auto cached_segment = [&](auto dense_tag, auto contig_tag) {
-        constexpr bool DENSE = decltype(dense_tag)::value, CONTIG = decltype(contig_tag)::value;
+      auto block = [&](auto contig_tag) {
+        constexpr bool CONTIG = decltype(contig_tag)::value;
 #pragma unroll
         for (int k0 = 0; k0 < 16; k0 += U) {
-          if (DENSE || CONTIG || k0 < nk) {
+          if (k0 == 0 || k0 < nk) {
             float4 vv[U][DH / 4];
 #pragma unroll
             for (int k = 0; k < U; ++k) {
-              const float4 *kp = CONTIG ? kptr(static_cast<int>(w.x & 0xFFu) + k0 + k)
-                                        : kptr(byte_at(w, DENSE ? k0 + k : min(k0 + k, nk - 1)));
+              const float4 *kp = CONTIG ? kptr(static_cast<int>(w.x & 0xFFu) + k0 + k) : kptr(byte_at(w, k0 + k));
 #pragma unroll
               for (int i = 0; i < DH / 4; ++i) vv[k][i] = kp[DH / 4 + i];
             }
@@ -586,53 +605,29 @@ __device__ __forceinline__ void hpsa_task(const float *q, const uint4 mask, int 
               // sigma - m for two keys: one paired add of -m (the cached scores are not products)
               pr[k / 2] = exp2_series2(add2(make_float2(sgs[k0 + k], sgs[k0 + k + 1]), make_float2(-mx, -mx)));
 #pragma unroll
-            for (int k = 0; k < U; k += 2) {
-              if (DENSE || ((CONTIG || k0 + k < nk) && ((seg >> (k0 + k)) & 1u))) fold(pr[k / 2].x, vv[k]);
-              if (DENSE || ((CONTIG || k0 + k + 1 < nk) && ((seg >> (k0 + k + 1)) & 1u)))
-                fold(pr[k / 2].y, vv[k + 1]);
-            }
+            for (int k = 0; k < U; k += 2) fold(pr[k / 2].x, vv[k]), fold(pr[k / 2].y, vv[k + 1]);
           }
         }
       };
-      const bool dense = nk == 16 && __all_sync(0xffffffffu, (seg & 0xFFFFu) == 0xFFFFu);
-      if (nk == 16 && contiguous(w)) {
-        if (dense) cached_segment(std::true_type{}, std::true_type{});
-        else cached_segment(std::false_type{}, std::true_type{});
-      } else {
-        if (dense) cached_segment(std::true_type{}, std::false_type{});
-        else cached_segment(std::false_type{}, std::false_type{});
-      }
-    } else if (nk == 16) {
+      if (contiguous(w)) block(std::true_type{});
+      else block(std::false_type{});
+    } else {
+      const uint32_t seg = segment(jb);
 #pragma unroll
       for (int k0 = 0; k0 < 16; k0 += U) {
-        float4 kk[U][DH / 4], vv[U][DH / 4];
+        if (k0 < nk) {
+          float sg[U];
+          scores(std::false_type{}, std::false_type{}, w, seg, k0, sg);
 #pragma unroll
-        for (int k = 0; k < U; ++k) {
-          const float4 *kp = kptr(byte_at(w, k0 + k));
+          for (int k = 0; k < U; k += 2) {
+            const float2 pr = exp2_series2(add2(make_float2(sg[k], sg[k + 1]), make_float2(-mx, -mx)));
+            float4 va[DH / 4], vb[DH / 4];
+            const float4 *pa = kptr(byte_at(w, k0 + k)), *pb = kptr(byte_at(w, k0 + k + 1));
 #pragma unroll
-          for (int i = 0; i < DH / 4; ++i) kk[k][i] = kp[i];
-#pragma unroll
-          for (int i = 0; i < DH / 4; ++i) vv[k][i] = kp[DH / 4 + i];
+            for (int i = 0; i < DH / 4; ++i) va[i] = pa[DH / 4 + i], vb[i] = pb[DH / 4 + i];
+            fold(pr.x, va), fold(pr.y, vb);
+          }
         }
-        float2 pr[U / 2];
-#pragma unroll
-        for (int k = 0; k < U; k += 2) pr[k / 2] = exp2_series2(shifted(dot2(kk[k], kk[k + 1])));
-#pragma unroll
-        for (int k = 0; k < U; k += 2) {
-          if (((seg >> (k0 + k)) & 1u)) fold(pr[k / 2].x, vv[k]);
-          if (((seg >> (k0 + k + 1)) & 1u)) fold(pr[k / 2].y, vv[k + 1]);
-        }
-      }
-    } else {
-      for (int k = 0; k < nk; k += 2) {
-        const int k1 = (k + 1 < nk) ? k + 1 : k;
-        float4 ka[DH / 4], kb[DH / 4], va[DH / 4], vb[DH / 4];
-        const float4 *pa = kptr(byte_at(w, k)), *pb = kptr(byte_at(w, k1));
-#pragma unroll
-        for (int i = 0; i < DH / 4; ++i) ka[i] = pa[i], kb[i] = pb[i], va[i] = pa[DH / 4 + i], vb[i] = pb[DH / 4 + i];
-        const float2 pr = exp2_series2(shifted(dot2(ka, kb)));
-        if (((seg >> k) & 1u)) fold(pr.x, va);
-        if (k1 != k && ((seg >> k1) & 1u)) fold(pr.y, vb);
       }
     }
   }
@@ -1060,6 +1055,8 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
   uint32_t *s_issued = reinterpret_cast<uint32_t *>(smem + L::kOffMisc + 136);  // [10] weight copies / phases armed
   // staged attention: warps past their reads of a buffer set in the current head round ([2] sets)
   uint32_t *s_headdone = reinterpret_cast<uint32_t *>(smem + L::kOffMisc + 176);
+  // warp tasks: 1 when a V row of the current block is not finite
+  volatile uint32_t *s_vbad = reinterpret_cast<volatile uint32_t *>(smem + L::kOffMisc + 184);
   // staged attention: the barriers of the K and V buffers (buffer set 0; set 1 when two heads fit)
   const uint32_t bar_sk = bar_fin + 32, bar_sv = bar_fin + 40;  // + 16: set 1
 
@@ -1081,6 +1078,7 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
     *s_abort = 0;
     for (int i = 0; i < 10; ++i) s_issued[i] = 0;
     s_headdone[0] = s_headdone[1] = 0;
+    *s_vbad = 0;
     // base of the K/V area of every CTA of the cluster as a shared::cluster address, and generic
     // base of its z area: this CTA's own through its plain shared-memory window, the others
     // through the distributed shared window
@@ -1393,6 +1391,12 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
           }
           dequant<DH>(ka, fk, bk, ka);
           dequant<DH>(va, fv, bv, va);
+          if constexpr (TASKS) {
+            float2 c = make_float2(0.0f, 0.0f);  // 0 * v summed: NaN if a value is not finite
+#pragma unroll
+            for (int i = 0; i < DH; i += 2) c = fma2(make_float2(va[i], va[i + 1]), make_float2(0.0f, 0.0f), c);
+            if (!(__fadd_rn(c.x, c.y) == 0.0f)) *s_vbad = 1;
+          }
           if constexpr (STAGED) {
             // K and V of this row and head, head-major in region U ([head][K, V][128 rows][64 B],
             // 16-byte piece f of row r at f ^ ((r >> 1) & 3)): the layout of the cluster's scratch
@@ -1443,16 +1447,15 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
         }
         if constexpr (TASKS) {
           // ---------------- S5: HPSA (Sec. 4.2), task mode: warp tasks over query groups
+          tc_fence_before();  // the score cache reuses accumulator columns that other warps have read
           named_bar_sync(5, kEpiThreads);  // every Q, K, V row of this CTA is in shared memory
-          // this warp's score cache: its lane quadrant, kTaskCache columns from kTaskCacheCol
-          static_assert(L::kQInSmem ? (L::kTaskCacheCol >= 4u * D && L::kTaskCacheCol + 4u * kTaskCache <= L::kTmemCols)
-                                    : (L::kTaskCacheCol >= 1u * D && L::kTaskCacheCol + 4u * kTaskCache <= 3u * D),
-                        "TMEM: the cache clears Q/A, the live accumulators and the parked residual");
+          tc_fence_after();
+          // this warp's score cache: its lane quadrant, kTaskCache columns (SmemLayout).
           // d = 128: a task's 32 rows are this warp's TMEM lane quadrant (the plan keeps every task on
           // a warp of its group's quadrant); Q comes from the QKV accumulators of this thread's row
           // and the output goes back over them
-          const uint32_t tcache = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + L::kTaskCacheCol +
-                                  static_cast<uint32_t>(warp >> 2) * kTaskCache;
+          const uint32_t tcache = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + L::task_cache_col(warp >> 2);
+          const bool vbad = *s_vbad != 0;
           for (int k = 0; k < kMaxTasks; ++k) {
             const uint32_t task = reinterpret_cast<const uint16_t *>(splan + p.off_task)[warp * kMaxTasks + k];
             if (task == 0xFFFFu) break;
@@ -1490,10 +1493,20 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
               if (cap) capture_acc(l, 0, qa, e * DH, DH);
               dequant<DH>(qa, fq, bq, q);
             }
-            hpsa_task<DH, L::kKvStride>(q, mk, static_cast<int>(ui & 255u),
-                                        reinterpret_cast<const uint4 *>(splan + p.off_ulist) + (ui >> 8),
-                                        smem + L::kOffU + gi.z * L::kKvStride,
-                                        e * L::kSlot + (L::kQInSmem ? 4 * DH : 0), p.att_scale, tcache, a);
+            const uint4 *ul = reinterpret_cast<const uint4 *>(splan + p.off_ulist) + (ui >> 8);
+            const uint8_t *krows = smem + L::kOffU + gi.z * L::kKvStride;
+            const uint32_t kslot = e * L::kSlot + (L::kQInSmem ? 4 * DH : 0);
+            if (!vbad) {
+              hpsa_task<DH, L::kKvStride, L::kTaskCache>(q, mk, static_cast<int>(ui & 255u), ul, krows, kslot,
+                                                         p.att_scale, tcache, a);
+            } else {
+              float qa[DH];
+#pragma unroll
+              for (int i = 0; i < DH; ++i) qa[i] = q[i];
+              hpsa_task_any<DH, L::kKvStride>(qa, mk, static_cast<int>(ui & 255u), ul, krows, kslot, p.att_scale);
+#pragma unroll
+              for (int i = 0; i < DH; ++i) a[i] = qa[i];
+            }
             if constexpr (L::kQInSmem) {
               if (act) {
                 // A of (row, head e) replaces Q of (row, head e): this task was its only reader
@@ -1517,6 +1530,7 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
             tc_fence_before();  // the TMEM stores are ordered before the barrier for the row owners
           }
           named_bar_sync(5, kEpiThreads);  // A complete; Q, K, V no longer read
+          if (tid == 0) *s_vbad = 0;  // the next block's V come after further barriers
           // Quant(A) -> O operand, by row slices
           // columns [sl XS, sl XS + XS) are heads 2 sl and 2 sl + 1, in their Q slots (shared memory)
           // or over their Q accumulators (TMEM, d = 128)

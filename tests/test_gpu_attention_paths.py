@@ -1,0 +1,84 @@
+"""The attention paths that the decoder picks by itself against the per-row walk (attention_mode 1),
+bit for bit, at the sizes where a path can go wrong: key lists that end inside, at and past a 16-key
+block and the score cache, lists whose rows are not consecutive, more words than a group holds."""
+import numpy as np
+import pytest
+
+from paper_2410_05911_gb300 import aecct as A
+from paper_2410_05911_gb300 import inputs as I
+
+torch = pytest.importorskip("torch")
+
+
+def random_code(n, m, weight, seed):
+    """A code whose variables join `weight` random checks each (every check at least one variable)."""
+    rng = np.random.Generator(np.random.PCG64(seed))
+    H = np.zeros((m, n), np.uint8)
+    for j in range(n):
+        H[rng.permutation(m)[:weight], j] = 1
+    H[np.arange(m), np.arange(m) % n] = 1
+    return I.LinearCode(f"random({n},{n - m})", n, n - m, H, np.zeros((1, n), np.uint8))
+
+
+def both(model, B, seed, mode=0):
+    rng = np.random.Generator(np.random.PCG64(seed))
+    y = torch.from_numpy(rng.standard_normal((B, model.n)).astype(np.float32)).cuda()
+    got = []
+    for attention in (mode, 1):
+        dec = A.Decoder(model, attention_mode=attention)
+        got.append([t.clone() for t in dec.decode(y)] + [dec.query()["attention_mode"]])
+        torch.cuda.synchronize()
+        assert dec.synchronize() == A.AECCT_OK
+        dec.close()
+    return got
+
+
+def same(got):
+    a, b = got
+    assert torch.equal(a[2].view(torch.int32), b[2].view(torch.int32)), "logits"
+    assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1])
+
+
+# (n, m, column weight): union lists below, at and above 16, 64 and 96 keys, up to 128 tokens
+TASKS = [(7, 3, 2), (18, 14, 2), (17, 15, 3), (33, 31, 1), (64, 32, 4), (65, 31, 3), (96, 32, 3), (97, 31, 2),
+         (110, 18, 3), (120, 8, 2)]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d", [32, 64, 128])
+@pytest.mark.parametrize("n,m,weight", TASKS, ids=lambda v: str(v))
+def test_warp_tasks_equal_per_row_walk(n, m, weight, d):
+    if d == 128 and (n + 31) // 32 * 32 + m > 128:
+        pytest.skip("warp tasks at d = 128 hold one padded word in 128 rows")
+    for mask_mode in (0, 1):
+        model = I.random_model(random_code(n, m, weight, n + d), d, 2, seed=n, spe_noise=True)
+        model.mask_mode = mask_mode
+        got = both(model, 5, seed=m, mode=2)
+        assert got[0][3] == 2 and got[1][3] == 1
+        same(got)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d", [32, 64, 128])
+def test_warp_tasks_keep_an_infinite_value_with_its_queries(d):
+    # one token's embedding so large that its V overflows: the rows that do not attend to it keep the
+    # finite attention outputs (recorded O operand) that the per-row walk gives them
+    code = random_code(40, 20, 2, 3)
+    model = I.random_model(code, d, 1, seed=5, spe_noise=True)
+    model.emb[7] = 1.0e38
+    model.w_scale[0, 2] = 1.0e4
+    rng = np.random.Generator(np.random.PCG64(2))
+    y = torch.from_numpy(np.clip(rng.standard_normal((3, code.n)), -2, 2).astype(np.float32)).cuda()
+    caps = []
+    for mode in (2, 1):
+        dec = A.Decoder(model, attention_mode=mode)
+        cap = dec.set_capture(3)
+        dec.decode(y)
+        torch.cuda.synchronize()
+        caps.append({k: cap[k].cpu().numpy() for k in ("alpha", "acc")})
+        dec.close()
+    finite = np.isfinite(caps[1]["alpha"][:, 0, 1])
+    assert finite.any() and not finite.all()
+    assert (np.isfinite(caps[0]["alpha"][:, 0, 1]) == finite).all()
+    assert (caps[0]["alpha"][:, 0, 1][finite] == caps[1]["alpha"][:, 0, 1][finite]).all()
+    assert (caps[0]["acc"][:, 0, 1][finite] == caps[1]["acc"][:, 0, 1][finite]).all()
