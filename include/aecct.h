@@ -69,8 +69,9 @@ typedef struct aecct_handle aecct_handle; /* opaque */
  *                 3 = per-row neighbour lists over per-head staged rows (d = 128, at most 640
  *                 token rows per group and 256 keys per row): head by head, the group's K and V
  *                 rows are gathered from every CTA of the cluster into local shared memory, and
- *                 the 4 threads of a row share its keys.  The default for d = 128 when a group
- *                 spans more than one CTA.  Every mode computes the same results bit for bit.
+ *                 4 lanes of a warp share a row's keys.  The default for d = 64 (where it cannot be
+ *                 asked for) and d = 128 when a group spans more than one CTA.  Every mode computes
+ *                 the same results bit for bit.
  *   mask_mode     0 = HPSA (Sec. 4.2): heads [0, h_first) first ring, the rest second ring;
  *                 1 = the ECCT code-aware mask (Sec. 3) for every head: the union of the first
  *                 and second rings (which contains each node itself).  Other values are rejected.

@@ -156,7 +156,8 @@ struct DecodeParams {
   const uint16_t *pos;          // [T] token -> row offset within its codeword
   // HPSA neighbour lists, 0 = first ring, 1 = second ring.  mask_info[mk][t] = (start << 11) | count:
   // the count row offsets of token t's neighbours (ascending token order) begin at mask_list[mk][start]
-  // and continue 8 per 16-byte entry (a list is padded to whole entries).
+  // and continue 8 per 16-byte entry (a list is padded to whole entries).  Staged attention: byte
+  // offsets in place of row offsets, row offset * 4 d_h + kv_piece(row offset).
   const uint32_t *mask_info[2];
   const uint4 *mask_list[2];
   // Task-mode attention plan (one CTA per group of codewords, d <= 64).  A task is one head for
@@ -184,9 +185,9 @@ struct DecodeParams {
   int32_t *cap_acc;
   float *cap_alpha;
   uint8_t *cap_syn;
-  // staged attention (d = 128): K and V of every row, per cluster, in global memory (L2), read back
-  // head by head with bulk copies: [cluster][8 heads][K, V][C * 128 rows][16 floats], 16-byte
-  // piece f of row rho at f ^ ((rho >> 1) & 3)
+  // staged attention (d >= 64): K and V of every row, per cluster, in global memory (L2), read back
+  // head by head with bulk copies: [cluster][8 heads][K, V][C * 128 rows][d_h floats], the 16-byte
+  // pieces of a row in the order of kv_piece
   float *kv_scratch;
   // control
   int *err;  // device word, bit 0 = a bounded wait timed out
@@ -198,6 +199,13 @@ struct DecodeParams {
 // K are adjacent (lbo = 128), 8-row groups are kdim/8 * 128 bytes apart (sbo).
 __host__ __device__ constexpr inline uint32_t core_off(uint32_t r, uint32_t c, uint32_t kdim) {
   return (r >> 3) * (kdim >> 3) * 128u + (c >> 3) * 128u + (r & 7u) * 16u + (c & 7u) * 2u;
+}
+
+// Staged attention: the 16-byte pieces of a K or V row of one head (4 at d_h = 16, 2 at d_h = 8) are
+// stored with piece f at byte 16 f ^ kv_piece(row offset within its word), which spreads lanes that
+// read the same piece of different rows over the banks (8 groups of 16 bytes).
+__host__ __device__ constexpr inline uint32_t kv_piece(int dh, uint32_t off) {
+  return dh == 16 ? ((off >> 1) & 3u) << 4 : ((off >> 2) & 1u) << 4;
 }
 
 // Shared-memory map.  Region U holds, per block, first the attention operands and then the FFN2
@@ -243,7 +251,7 @@ struct SmemLayout {
 };
 
 // decoder_kernel.cuh.  ATT: 0 = per-row neighbour lists, 1 = warp tasks, 2 = per-row lists over
-// per-head staged rows (d = 128); ACT: 0 = ReLU, 1 = GELU; LIN: 0 = AAP linears, 1 = full-precision
+// per-head staged rows (d >= 64); ACT: 0 = ReLU, 1 = GELU; LIN: 0 = AAP linears, 1 = full-precision
 // (bf16) linears.  Instantiated in decoder_kernel.cu (0, 0), decoder_kernel_gelu.cu (1, 0),
 // decoder_kernel_fp.cu (0, 1) and decoder_kernel_fp_gelu.cu (1, 1).
 template <int D, int ATT, int ACT, int LIN>

@@ -237,6 +237,9 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
 __device__ __forceinline__ void st_shared_v4(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
   asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
+__device__ __forceinline__ void st_shared_u32(uint32_t addr, uint32_t a) {
+  asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(a) : "memory");
+}
 __device__ __forceinline__ void st_shared_v2(uint32_t addr, uint32_t a, uint32_t b) {
   asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
 }
@@ -245,15 +248,22 @@ __device__ __forceinline__ float4 ld_shared_f4(uint32_t addr) {
   asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr) : "memory");
   return v;
 }
+__device__ __forceinline__ float2 ld_shared_f2(uint32_t addr) {
+  float2 v;
+  asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "r"(addr) : "memory");
+  return v;
+}
 __device__ __forceinline__ void st_shared_f4(uint32_t addr, float a, float b, float c, float d) {
   asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(a), "f"(b), "f"(c), "f"(d) : "memory");
 }
 
 // write the codes of LEN consecutive columns [c0, c0 + LEN) of row r into a K-major operand tile
-// (c0 is a multiple of 8, or of 4 when LEN == 4)
+// (c0 is a multiple of 8, or of LEN when that is 2 or 4)
 template <int LEN>
 __device__ __forceinline__ void store_codes(uint32_t tile, int r, int c0, int kdim, const float *q) {
-  if constexpr (LEN == 4) {
+  if constexpr (LEN == 2) {
+    st_shared_u32(tile + core_off(r, c0, kdim), pack_bf16x2(q[0], q[1]));
+  } else if constexpr (LEN == 4) {
     st_shared_v2(tile + core_off(r, c0, kdim), pack_bf16x2(q[0], q[1]), pack_bf16x2(q[2], q[3]));
   } else {
     static_assert(LEN % 8 == 0, "code run");
@@ -272,7 +282,9 @@ __device__ __forceinline__ uint32_t pack_bf16x2_rn(float a, float b) {
 }
 template <int LEN>
 __device__ __forceinline__ void store_bf16(uint32_t tile, int r, int c0, int kdim, const float *v) {
-  if constexpr (LEN == 4) {
+  if constexpr (LEN == 2) {
+    st_shared_u32(tile + core_off(r, c0, kdim), pack_bf16x2_rn(v[0], v[1]));
+  } else if constexpr (LEN == 4) {
     st_shared_v2(tile + core_off(r, c0, kdim), pack_bf16x2_rn(v[0], v[1]), pack_bf16x2_rn(v[2], v[3]));
   } else {
     static_assert(LEN % 8 == 0, "bf16 run");
@@ -1024,7 +1036,7 @@ template <int D, int ATT, int ACT, int LIN>
 __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid_constant__ DecodeParams p) {
   // ATT: 0 = per-row neighbour lists, 1 = warp tasks, 2 = per-row lists over per-head staged rows
   constexpr bool TASKS = ATT == 1, STAGED = ATT == 2;
-  static_assert(!STAGED || D == 128, "staged attention is built for d = 128");
+  static_assert(!STAGED || D == 64 || D == 128, "staged attention is built for d = 64 and 128");
   using L = SmemLayout<D, TASKS>;
   using LP = LayerParamLayout;
   constexpr int DH = D / kHeads;  // head width
@@ -1057,8 +1069,7 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
   uint32_t *s_headdone = reinterpret_cast<uint32_t *>(smem + L::kOffMisc + 176);
   // warp tasks: 1 when a V row of the current block is not finite
   volatile uint32_t *s_vbad = reinterpret_cast<volatile uint32_t *>(smem + L::kOffMisc + 184);
-  // staged attention: the barriers of the K and V buffers (buffer set 0; set 1 when two heads fit)
-  const uint32_t bar_sk = bar_fin + 32, bar_sv = bar_fin + 40;  // + 16: set 1
+  const uint32_t bar_skv = bar_fin + 32;  // staged attention: the barriers of the two sets of K and V buffers
 
   if (tid == 0) {
     for (int s = 0; s < S; ++s) {
@@ -1072,8 +1083,8 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
     mbar_init(bar_zr, p.C);
     mbar_init(bar_zf, p.C);
     mbar_init(bar_fin, 1);
-    if constexpr (D == 128)  // region U, the two operand-tile halves (d = 128 weight schedule), the
-                             // staged K/V buffers, FFN1's first half
+    if constexpr (D == 128 || STAGED)  // region U, the two operand-tile halves (d = 128 weight schedule),
+                                       // the staged K/V buffers, FFN1's first half
       for (int i = 0; i < 8; ++i) mbar_init(bar_fin + 8 + 8 * i, 1);
     *s_abort = 0;
     for (int i = 0; i < 10; ++i) s_issued[i] = 0;
@@ -1155,9 +1166,9 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
     // between the group start and S10).  Word g's rows are [g T, g T + T).
     float *rowmax_s = reinterpret_cast<float *>(smem + L::kOffZ);
     float *wordmax_s = reinterpret_cast<float *>(smem + L::kOffBitWords);
-    auto word_alpha = [&](float a_row) -> float {
-      if (p.alpha_mode == 0) return a_row;
-      if (sl == 0) rowmax_s[r] = a_row;
+    // (`publish`: the thread that holds row `row`'s absmax; `gw`: the word of its own row)
+    auto word_max = [&](float a_row, bool publish, int row, int gw) -> float {
+      if (publish) rowmax_s[row] = a_row;
       named_bar_sync(5, kEpiThreads);
       if (warp < p.G) {
         float a = 0.0f;
@@ -1167,9 +1178,9 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
         if (lane == 0) wordmax_s[warp] = a;
       }
       named_bar_sync(5, kEpiThreads);
-      const int gw = (static_cast<int>(crank) * kRows + r) / p.Tp;
       return gw < p.G ? wordmax_s[gw] : a_row;
     };
+    auto word_alpha = [&](float a_row) -> float { return p.alpha_mode == 0 ? a_row : word_max(a_row, sl == 0, r, g); };
     auto row_sum = [&](float v) -> float {
       *red.slot(sl, r) = v;
       named_bar_sync(qbar, 128);
@@ -1398,16 +1409,16 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
             if (!(__fadd_rn(c.x, c.y) == 0.0f)) *s_vbad = 1;
           }
           if constexpr (STAGED) {
-            // K and V of this row and head, head-major in region U ([head][K, V][128 rows][64 B],
-            // 16-byte piece f of row r at f ^ ((r >> 1) & 3)): the layout of the cluster's scratch
-            // in global memory, where bulk copies take them next
-            const uint32_t kd = kvl + ((static_cast<uint32_t>(e) * 2u) * kRows + r) * 64u;
-            const uint32_t vd = kd + kRows * 64u;
+            // K and V of this row and head, head-major in region U ([head][K, V][128 rows][d_h],
+            // 16-byte pieces in the order of kv_piece): the layout of the cluster's scratch in global
+            // memory, where bulk copies take them next
+            const uint32_t kd = kvl + ((static_cast<uint32_t>(e) * 2u) * kRows + r) * (4u * DH);
+            const uint32_t vd = kd + kRows * (4u * DH);
 #pragma unroll
             for (int f = 0; f < DH / 4; ++f) {
-              const uint32_t g = static_cast<uint32_t>((f ^ ((r >> 1) & 3)) << 4);
-              st_shared_f4(kd + g, ka[4 * f], ka[4 * f + 1], ka[4 * f + 2], ka[4 * f + 3]);
-              st_shared_f4(vd + g, va[4 * f], va[4 * f + 1], va[4 * f + 2], va[4 * f + 3]);
+              const uint32_t g16 = static_cast<uint32_t>(f << 4) ^ kv_piece(DH, static_cast<uint32_t>(rho - g * Tp));
+              st_shared_f4(kd + g16, ka[4 * f], ka[4 * f + 1], ka[4 * f + 2], ka[4 * f + 3]);
+              st_shared_f4(vd + g16, va[4 * f], va[4 * f + 1], va[4 * f + 2], va[4 * f + 3]);
             }
           } else {
             // head slot of this row: (K | V), or (Q | K | V) in task mode at d <= 64
@@ -1660,18 +1671,26 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
             }
           }
         } else {
-          // ---------------- S5: HPSA (Sec. 4.2), per-row lists over per-head staged rows (d = 128).
-          // Every CTA of the cluster has left the K and V rows of its token rows in the cluster's
-          // scratch in global memory (L2).  Head by head, one bulk copy brings the K rows of the
-          // head for every row of the group into a K buffer and another the V rows into a V buffer;
-          // two sets of buffers (region U and the operand tile, idle here) let the next head's rows
-          // arrive while this head computes.  The row's 4 threads share the head: each takes 4 keys of every 16-key block for the scores
-          // and their exponentials (the row's TMEM lane, columns from kSc), and then folds every
-          // key, in ascending order, into 4 of the 16 features of num.  The arithmetic is the
-          // canonical one, key for key and feature for feature.
+          // ---------------- S5: HPSA (Sec. 4.2), per-row lists over per-head staged rows (d >= 64).
+          // Every CTA of the cluster leaves the K and V rows of its token rows in the cluster's scratch
+          // in global memory (L2).  Head by head, one bulk copy brings the K rows of the head for every
+          // row of the group into a K buffer and another the V rows into a V buffer; two sets of buffers
+          // (region U and the operand tile, idle here) let the next head's rows arrive while this head
+          // computes.  A warp takes 8 rows of its lane quadrant, four adjacent lanes a row: lane part s
+          // takes keys s, s + 4, s + 8, ... of the row's list for the scores and their exponentials, and
+          // then folds every key, in ascending order, into a quarter of the features of num.  The maximum
+          // and the exponentials pass between the four lanes by shuffles, so that a warp meets no other
+          // warp until the last head.  The arithmetic is the canonical one, key for key and feature for
+          // feature.  Bound by the shared-memory reads of scattered K rows and V pieces (bank conflicts).
+          // With a row's four threads in the four warps of its quadrant instead, which met in three named
+          // barriers and two TMEM exchanges a head, LDPC(128,64) took 379.9 ms for 131,072 words (now
+          // 330.8) and LDPC(384,192) 164.5 ms for 16,384 (146.9).  LDPC(128,64) at d = 64, whose rows
+          // read keys through distributed shared memory before: 21.57 ms for 10,007 words (17.25).
+          //
           // this CTA's K and V rows, from region U to the cluster's scratch in global memory: 16 bulk
-          // copies (one per head and kind, 8 KB each) by thread 0, complete before the cluster
-          // learns that they are there
+          // copies (one per head and kind) by thread 0, complete before the cluster learns that they are
+          // there
+          constexpr uint32_t kRowBytes = 4u * DH;
           fence_proxy_async_smem();  // this thread's K / V stores, before the bulk copies read them
           named_bar_sync(5, kEpiThreads);
           if (tid == 0 && !*s_abort) {
@@ -1679,60 +1698,49 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
             for (int ek = 0; ek < 2 * kHeads; ++ek)
               bulk_s2g(p.kv_scratch + (static_cast<size_t>(cluster_id) * 2 * kHeads + ek) * R * DH +
                            static_cast<size_t>(crank) * kRows * DH,
-                       kvl + static_cast<uint32_t>(ek) * kRows * 64u, kRows * 64u);
+                       kvl + static_cast<uint32_t>(ek) * kRows * kRowBytes, kRows * kRowBytes);
             bulk_commit_group();
             bulk_wait_group_0();
             fence_proxy_async_global();
           }
           cluster_arrive(bar_kvr);
           cluster_wait(bar_kvr, kvr_ph);
-          static_assert(L::kOffU == 0 && L::kOffAop == L::kRegionU &&
-                            L::kRegionU + L::kAopBytes >= 4u * kStagedMaxRows * 64u,
+          static_assert(L::kOffU == 0 && L::kOffAop == L::kRegionU && 16u * kRows * kRowBytes <= L::kRegionU &&
+                            L::kRegionU + L::kAopBytes >= 4u * kStagedMaxRows * kRowBytes,
                         "two sets of K and V buffers span region U and the operand tile");
-          constexpr uint32_t kSc = 128;  // the dead K and V accumulator columns [128, 384)
-          // row rho of the group: 64 bytes at rho * 64, 16-byte piece f at f ^ ((rho >> 1) & 3)
-          const int nrows = p.G * Tp;  // <= 640 (checked at create)
-          const int rowbase = g * Tp;
-          const uint32_t fetch_bytes = static_cast<uint32_t>(nrows) * 64u;
-          // two sets of K and V buffers in region U (its K and V went to the scratch: idle here) and
-          // the operand tile, [K0 | V0 | K1 | V1]: head e uses set e & 1 and the next-but-one head is
-          // fetched after head e, so each head needs one CTA barrier
+          // row rho of the group: kRowBytes at rho * kRowBytes, its 16-byte pieces in the order of kv_piece
+          const uint32_t fetch_bytes = static_cast<uint32_t>(p.G * Tp) * kRowBytes;  // <= 640 rows (checked at create)
+          // [K0 | V0 | K1 | V1]: head e uses set e & 1, and the next-but-one head is fetched after head e
           const float *kvs = p.kv_scratch + static_cast<size_t>(cluster_id) * kHeads * 2 * (p.C * kRows) * DH;
           auto buf_of = [&](int e, int kind) -> uint32_t {
             return sb + L::kOffU + (static_cast<uint32_t>(e & 1) * 2u + kind) * fetch_bytes;
           };
-          auto bar_of = [&](int e, int kind) -> uint32_t { return (kind ? bar_sv : bar_sk) + ((e & 1) ? 16u : 0u); };
-          // phase parity of head e's barrier: one completion per two heads, 4 a block
-          auto par_of = [&](int e) -> uint32_t { return static_cast<uint32_t>((e >> 1) & 1); };
-          // thread 0: the bulk copy of head e's K (kind 0) or V (kind 1) rows (nothing once a wait
-          // gave up, so that the teardown knows every copy in flight)
-          auto fetch = [&](int e, int kind) {
+          // one thread: the bulk copies of head e's K and V rows (nothing once a wait gave up, so that the
+          // teardown knows every copy in flight); a set's barrier completes 4 times a block
+          auto fetch = [&](int e) {
             if (*s_abort) return;
-            const uint32_t bar = bar_of(e, kind);
-            mbar_arrive_expect_tx(bar, fetch_bytes);
-            bulk_g2s(buf_of(e, kind), kvs + (static_cast<size_t>(e) * 2 + kind) * (p.C * kRows) * DH, fetch_bytes,
-                     bar);
-            ++s_issued[6 + kind + ((e & 1) ? 2 : 0)];
+            const uint32_t bar = bar_skv + ((e & 1) ? 8u : 0u);
+            mbar_arrive_expect_tx(bar, 2u * fetch_bytes);
+#pragma unroll 1
+            for (int kind = 0; kind < 2; ++kind)
+              bulk_g2s(buf_of(e, kind), kvs + (static_cast<size_t>(e) * 2 + kind) * (p.C * kRows) * DH, fetch_bytes, bar);
+            ++s_issued[6 + (e & 1)];
           };
-          if (tid == 0) fetch(0, 0), fetch(0, 1), fetch(1, 0), fetch(1, 1);
-          auto dot16 = [&](const float *q, const float4 *kk) -> float {
-            float2 d2 = make_float2(0.0f, 0.0f);
-#pragma unroll
-            for (int i = 0; i < DH / 4; ++i) {
-              d2 = fma2(make_float2(q[4 * i], q[4 * i + 1]), make_float2(kk[i].x, kk[i].y), d2);
-              d2 = fma2(make_float2(q[4 * i + 2], q[4 * i + 3]), make_float2(kk[i].z, kk[i].w), d2);
-            }
-            return __fadd_rn(d2.x, d2.y);
-          };
+          if (tid == 0) fetch(0), fetch(1);
+          // this lane's row (row ar of the quadrant: its Q, token and word come from lane ar) and part s
+          const int ar = 8 * sl + (lane >> 2), s = lane & 3, r2 = 32 * qd + ar;
+          const int t2 = __shfl_sync(0xffffffffu, t, ar), g2 = __shfl_sync(0xffffffffu, g, ar);
+          const bool row2 = __shfl_sync(0xffffffffu, row_cw ? 1 : 0, ar) != 0;
+          const uint32_t word_off = row2 ? static_cast<uint32_t>(g2 * Tp) * kRowBytes : 0u;
+          constexpr int VF = DH / 4;  // features of a lane
+          float av[kHeads * VF];
+#pragma unroll 1
           for (int e = 0; e < kHeads; ++e) {
-            // each barrier completes 4 times a block: an even number
-            const uint32_t ph = par_of(e);
-            const uint32_t kbuf = buf_of(e, 0), vbuf = buf_of(e, 1);
             const int mk = (e < p.h_first) ? 0 : 1;
-            const uint32_t info = row_cw ? __ldg(p.mask_info[mk] + t) : 0u;
+            const uint32_t info = row2 ? __ldg(p.mask_info[mk] + t2) : 0u;
             const int cnt = static_cast<int>(info & 2047u);
             const uint4 *lst = p.mask_list[mk] + (info >> 11);
-            const int nmax = __reduce_max_sync(0xffffffffu, cnt);  // the same for the 4 warps of the quadrant
+            const int nmax = __reduce_max_sync(0xffffffffu, cnt);
             float q[DH];
             {
               float qa[DH], bq[DH];
@@ -1740,128 +1748,157 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
               tmem_ld<DH>(tl + e * DH, qa);
               tmem_wait_ld();
               if (cap && sl == (e & 3)) capture_acc(l, 0, qa, e * DH, DH);
+              dequant<DH>(qa, fq, bq, q);
 #pragma unroll
-              for (int i = 0; i < DH; ++i) q[i] = __fadd_rn(__fmul_rn(qa[i], fq), bq[i]);
+              for (int i = 0; i < DH; ++i) q[i] = __shfl_sync(0xffffffffu, q[i], ar);
             }
-            wait_bar_warp(ctl, bar_of(e, 0), ph, false);  // this head's K rows have landed
-            // pass 1: sigma of keys [b + 4 sl, b + 4 sl + 4) of every 16-key block b, and their maximum
-            float mx = -INFINITY;
-            for (int b = 0; b < nmax; b += 16) {
-              const int k0 = b + 4 * sl;
-              if (k0 < nmax) {
-                const uint4 w = (k0 < cnt) ? __ldg(lst + (k0 >> 3)) : make_uint4(0u, 0u, 0u, 0u);
-                const uint32_t lo = (k0 & 4) ? w.z : w.x, hi = (k0 & 4) ? w.w : w.y;
-                const int idx[4] = {static_cast<int>(lo & 0xFFFFu), static_cast<int>(lo >> 16),
-                                    static_cast<int>(hi & 0xFFFFu), static_cast<int>(hi >> 16)};
-                float sg[4];
+            const uint32_t kbuf = buf_of(e, 0) + word_off, vbuf = buf_of(e, 1) + word_off;
+            // the 16 list entries of block b (zeros past the row's list: the word's first row)
+            auto entries = [&](int b, uint4 *w) {
+              w[0] = b < cnt ? __ldg(lst + (b >> 3)) : make_uint4(0u, 0u, 0u, 0u);
+              w[1] = b + 8 < cnt ? __ldg(lst + (b >> 3) + 1) : make_uint4(0u, 0u, 0u, 0u);
+            };
+            // sigma of this lane's keys b + 4 i + s, -inf past the row's list
+            auto score4 = [&](int b, const uint4 *w, float *sg) {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                  const int rho = rowbase + idx[i];  // a key past the row's count reads a valid row (offset 0)
-                  const uint32_t rb = kbuf + static_cast<uint32_t>(rho) * 64u;
-                  float4 kk[DH / 4];
+              for (int i = 0; i < 4; ++i) {
+                if (b + 4 * i < nmax) {
+                  const uint4 &wi = w[i >> 1];
+                  const uint32_t pair = (i & 1) ? ((s & 2) ? wi.w : wi.z) : ((s & 2) ? wi.y : wi.x);
+                  const uint32_t kr = kbuf + ((s & 1) ? pair >> 16 : pair & 0xFFFFu);
+                  float2 d2 = make_float2(0.0f, 0.0f);
 #pragma unroll
-                  for (int f = 0; f < DH / 4; ++f)
-                    kk[f] = ld_shared_f4(rb + static_cast<uint32_t>((f ^ ((rho >> 1) & 3)) << 4));
-                  sg[i] = __fmul_rn(dot16(q, kk), p.att_scale);
-                  if (k0 + i < cnt) mx = fmaxf(mx, sg[i]);
+                  for (int f = 0; f < DH / 4; ++f) {
+                    const float4 kk = ld_shared_f4(kr ^ static_cast<uint32_t>(f << 4));
+                    d2 = fma2(make_float2(q[4 * f], q[4 * f + 1]), make_float2(kk.x, kk.y), d2);
+                    d2 = fma2(make_float2(q[4 * f + 2], q[4 * f + 3]), make_float2(kk.z, kk.w), d2);
+                  }
+                  const float sc = __fmul_rn(__fadd_rn(d2.x, d2.y), p.att_scale);
+                  sg[i] = b + 4 * i + s < cnt ? sc : -INFINITY;
+                } else {
+                  sg[i] = -INFINITY;
                 }
-                tmem_st4(tl + kSc + k0, sg[0], sg[1], sg[2], sg[3]);
               }
-            }
-            tmem_wait_st();
-            tc_fence_before();
-            mx = row_max(mx);
-            tc_fence_after();
-            // pass 2: p = 2^(sigma - m) of the same keys, written over their scores
-            for (int b = 0; b < nmax; b += 16) {
-              const int k0 = b + 4 * sl;
-              if (k0 < nmax) {
-                float sg[4];
-                tmem_ld<4>(tl + kSc + k0, sg);
+            };
+            float mx = -INFINITY, lsum = 0.0f, num[VF];
+#pragma unroll
+            for (int f = 0; f < VF; ++f) num[f] = 0.0f;
+            // the exponentials of this lane's four scores, then l = sum p and num = sum p v over the block's
+            // keys in ascending order: key 4 i + u has its p in lane part u
+            auto fold16 = [&](int b, const uint4 *w, const float *sg) {
+              const float2 p01 = exp2_series2(add2(make_float2(sg[0], sg[1]), make_float2(-mx, -mx)));
+              const float2 p23 = exp2_series2(add2(make_float2(sg[2], sg[3]), make_float2(-mx, -mx)));
+              const float pr[4] = {p01.x, p01.y, p23.x, p23.y};
+#pragma unroll
+              for (int i = 0; i < 4; ++i) {
+                if (b + 4 * i < nmax) {
+                  float vv[4][VF], pk[4];
+#pragma unroll
+                  for (int u = 0; u < 4; ++u) {
+                    const int kk = 4 * i + u;
+                    const uint32_t va = vbuf + (static_cast<uint32_t>(idx_at(w[kk >> 3], kk & 7)) ^
+                                                static_cast<uint32_t>(s * 4 * VF));
+                    if constexpr (VF == 4) {
+                      const float4 x4 = ld_shared_f4(va);
+                      vv[u][0] = x4.x, vv[u][1] = x4.y, vv[u][2] = x4.z, vv[u][3] = x4.w;
+                    } else {
+                      const float2 x2 = ld_shared_f2(va);
+                      vv[u][0] = x2.x, vv[u][1] = x2.y;
+                    }
+                    pk[u] = __shfl_sync(0xffffffffu, pr[i], (lane & 28) | u);
+                  }
+#pragma unroll
+                  for (int u = 0; u < 4; ++u)
+                    if (b + 4 * i + u < cnt) {
+                      lsum = __fadd_rn(lsum, pk[u]);
+#pragma unroll
+                      for (int f = 0; f < VF; ++f) num[f] = __fmaf_rn(pk[u], vv[u][f], num[f]);
+                    }
+                }
+              }
+            };
+            auto row_max4 = [&]() {
+              mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+              mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+            };
+            uint4 w[2];
+            float sg[4];
+            entries(0, w);
+            // this head's rows have landed
+            if (lane == 0) wait_bar(ctl, bar_skv + ((e & 1) ? 8u : 0u), static_cast<uint32_t>((e >> 1) & 1), false);
+            __syncwarp();
+            if (nmax <= 16) {  // the lists of this warp's rows are one block each: scores stay in registers
+              score4(0, w, sg);
+              mx = fmaxf(fmaxf(sg[0], sg[1]), fmaxf(sg[2], sg[3]));
+              row_max4();
+              fold16(0, w, sg);
+            } else {
+              // the scores in this thread's own TMEM lane, 4 columns a block from column kSc + 64 sl (at most
+              // 256 keys), in columns whose accumulators are dead (d = 128) or that hold none (d = 64)
+              const uint32_t tsc = tl + L::kRowCacheCol + 64u * static_cast<uint32_t>(sl);
+#pragma unroll 1
+              for (int b = 0; b < nmax; b += 16) {
+                entries(b, w);
+                score4(b, w, sg);
+                mx = fmaxf(mx, fmaxf(fmaxf(sg[0], sg[1]), fmaxf(sg[2], sg[3])));
+                tmem_st4(tsc + (b >> 2), sg[0], sg[1], sg[2], sg[3]);
+              }
+              tmem_wait_st();
+              row_max4();
+#pragma unroll 1
+              for (int b = 0; b < nmax; b += 16) {
+                entries(b, w);
+                tmem_ld<4>(tsc + (b >> 2), sg);
                 tmem_wait_ld();
-                const float2 p01 = exp2_series2(add2(make_float2(sg[0], sg[1]), make_float2(-mx, -mx)));
-                const float2 p23 = exp2_series2(add2(make_float2(sg[2], sg[3]), make_float2(-mx, -mx)));
-                tmem_st4(tl + kSc + k0, p01.x, p01.y, p23.x, p23.y);
+                fold16(b, w, sg);
               }
             }
-            tmem_wait_st();
-            tc_fence_before();
-            named_bar_sync(qbar, 128);
-            tc_fence_after();
-            wait_bar_warp(ctl, bar_of(e, 1), ph, false);  // this head's V rows have landed
-            // l = sum p and num = sum p v over the row's keys in ascending order, features [4 sl, 4 sl + 4)
-            float lsum = 0.0f, num[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-            for (int b = 0; b < nmax; b += 16) {
-              float pb[16];
-              tmem_ld<16>(tl + kSc + b, pb);
-              tmem_wait_ld();
-              const uint4 w0 = (b < cnt) ? __ldg(lst + (b >> 3)) : make_uint4(0u, 0u, 0u, 0u);
-              const uint4 w1 = (b + 8 < cnt) ? __ldg(lst + (b >> 3) + 1) : make_uint4(0u, 0u, 0u, 0u);
+            const float inv = __fdiv_rn(1.0f, lsum);
 #pragma unroll
-              for (int kk = 0; kk < 16; ++kk) {
-                if (b + kk < cnt) {
-                  const int rho = rowbase + idx_at(kk < 8 ? w0 : w1, kk & 7);
-                  const float4 vv = ld_shared_f4(vbuf + static_cast<uint32_t>(rho) * 64u +
-                                                 static_cast<uint32_t>((sl ^ ((rho >> 1) & 3)) << 4));
-                  lsum = __fadd_rn(lsum, pb[kk]);
-                  num[0] = __fmaf_rn(pb[kk], vv.x, num[0]);
-                  num[1] = __fmaf_rn(pb[kk], vv.y, num[1]);
-                  num[2] = __fmaf_rn(pb[kk], vv.z, num[2]);
-                  num[3] = __fmaf_rn(pb[kk], vv.w, num[3]);
-                }
-              }
-            }
-            {
-              const float inv = __fdiv_rn(1.0f, lsum);
-              float a4[4];
-#pragma unroll
-              for (int f = 0; f < 4; ++f) a4[f] = row_cw ? __fmul_rn(num[f], inv) : 0.0f;
-              // A of (row, head e), features [4 sl, 4 sl + 4), over the head's Q (read by all 4 threads
-              // before the barriers above)
-              tmem_st4(tl + e * DH + 4 * sl, a4[0], a4[1], a4[2], a4[3]);
-            }
-            tmem_wait_st();
-            tc_fence_before();
-            // the row's four threads (the quadrant's warps) are past this head's reads of the
-            // score columns, which the next head's pass 1 rewrites; after the last head every
-            // attention output in TMEM is ordered before Quant(A)
-            if (e == kHeads - 1) named_bar_sync(5, kEpiThreads);
-            else named_bar_sync(qbar, 128);
-            tc_fence_after();
+            for (int f = 0; f < VF; ++f) av[e * VF + f] = row2 ? __fmul_rn(num[f], inv) : 0.0f;
             if (e + 2 < kHeads) {
-              // this warp is past its reads of this head's buffers; the last warp of the CTA to get
-              // here fetches the next-but-one head's K and V into them (no quadrant waits for the
-              // slowest one between heads; a warp that runs ahead waits for those rows to land)
+              // this warp is past its reads of this head's buffers; the last warp of the CTA to get here
+              // fetches the next-but-one head's K and V into them
+              __syncwarp();
               if (lane == 0) {
                 __threadfence_block();
                 if (atomicAdd(s_headdone + (e & 1), 1u) == static_cast<uint32_t>(kEpiWarps - 1)) {
                   s_headdone[e & 1] = 0u;
                   __threadfence_block();
                   fence_proxy_async_smem();
-                  fetch(e + 2, 0), fetch(e + 2, 1);
+                  fetch(e + 2);
                 }
               }
               __syncwarp();
             }
           }
-          // Quant(A) -> O operand: columns [sl XS, sl XS + XS) = heads 2 sl and 2 sl + 1, from TMEM
-          float av[XS];
-          tmem_ld<XS>(tl + sl * XS, av);
-          tmem_wait_ld();
+          named_bar_sync(5, kEpiThreads);  // the buffers (operand tile) are no longer read
+          // Quant(A) -> O operand: this lane has features [VF s, VF s + VF) of every head of row r2
           if constexpr (LIN == 1) {
-            store_bf16<XS>(aop, r, sl * XS, D, av);
-          } else {
-            float amax = 0.0f;
 #pragma unroll
-            for (int j = 0; j < XS; ++j) amax = fmaxf(amax, fabsf(av[j]));
-            float a = word_alpha(row_max(amax));
+            for (int e = 0; e < kHeads; ++e) store_bf16<VF>(aop, r2, e * DH + VF * s, D, av + e * VF);
+          } else {
+            float a = 0.0f;
+#pragma unroll
+            for (int j = 0; j < XS; ++j) a = fmaxf(a, fabsf(av[j]));
+            a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, 1));
+            a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, 2));
+            if (p.alpha_mode != 0) a = word_max(a, s == 0, r2, g2);
             a = (a > p.alpha_floor) ? a : p.alpha_floor;
-            alpha_in = a;
+            if (s == 0) rowmax_s[r2] = a;  // the row's owner reads it after the O GEMM
             const float rr = __fdiv_rn(127.0f, a);
             float qv[XS];
             codes<XS>(av, rr, qv);
-            store_codes<XS>(aop, r, sl * XS, D, qv);
-            if (cap) capture_q(l, 1, qv, sl * XS, XS, alpha_in);
+#pragma unroll
+            for (int e = 0; e < kHeads; ++e) store_codes<VF>(aop, r2, e * DH + VF * s, D, qv + e * VF);
+            const int64_t b2 = gi * p.G + g2;
+            if (row2 && b2 < p.B && b2 < p.cap_B) {
+              const int64_t row = ((b2 * p.n_layers + l) * 4 + 1) * T + t2;
+              if (p.cap_q)
+                for (int j = 0; j < XS; ++j)
+                  p.cap_q[row * W4 + (j / VF) * DH + VF * s + j % VF] = static_cast<int8_t>(qv[j]);
+              if (p.cap_alpha && s == 0) p.cap_alpha[row] = a;
+            }
           }
         }
         // this CTA no longer reads any K/V of this block (arrived before the O GEMM is issued: the
@@ -1875,10 +1912,14 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
 
         // ---------------- S6: O projection + residual + LayerNorm (Sec. 5, Post-LN)
         {
-          const float fo = dq_factor(sw + 3);
+          float fo = STAGED ? 0.0f : dq_factor(sw + 3);
           float ac[XS], bb[XS];
           if constexpr (kEarlyBias) ldg_vec<XS>(lp + LP::bo(D) + sl * XS, bb);
           wait_acc();
+          if constexpr (STAGED) {  // the row's alpha comes from the lanes that computed its attention
+            if constexpr (LIN == 0) alpha_in = rowmax_s[r];
+            fo = dq_factor(sw + 3);
+          }
           tmem_ld<XS>(tl + sl * XS, ac);
           tmem_ld<XS>(tl + 3 * D + sl * XS, x);
           tmem_wait_ld();
@@ -2113,9 +2154,8 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
       wait_bar_drain(ctl, bar_fin, 0);
       issuer.drain();
       if constexpr (STAGED)  // the staged attention's bulk copies of K and V rows (two buffer sets)
-        for (int i = 0; i < 4; ++i)
-          if (s_issued[6 + i] > 0)
-            wait_bar_drain(ctl, ((i & 1) ? bar_sv : bar_sk) + (i >= 2 ? 16u : 0u), (s_issued[6 + i] - 1u) & 1u);
+        for (int i = 0; i < 2; ++i)
+          if (s_issued[6 + i] > 0) wait_bar_drain(ctl, bar_skv + 8u * i, (s_issued[6 + i] - 1u) & 1u);
     }
     __syncwarp();
   }

@@ -82,3 +82,37 @@ def test_warp_tasks_keep_an_infinite_value_with_its_queries(d):
     assert (np.isfinite(caps[0]["alpha"][:, 0, 1]) == finite).all()
     assert (caps[0]["alpha"][:, 0, 1][finite] == caps[1]["alpha"][:, 0, 1][finite]).all()
     assert (caps[0]["acc"][:, 0, 1][finite] == caps[1]["acc"][:, 0, 1][finite]).all()
+
+
+# LDPC codes of 129 to 639 tokens (staged over a cluster) at both widths, lists of one block (HPSA) and
+# more (the code-aware mask), an odd token count, several words to a group, a batch that ends inside one
+STAGED = [(86, 64, 3), (100, 50, 6), (128, 64, 3), (131, 60, 5), (200, 57, 8), (426, 213, 3)]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("mask_mode", [0, 1])
+@pytest.mark.parametrize("n,m,weight", STAGED, ids=lambda v: str(v))
+def test_staged_attention_equals_per_row_walk(n, m, weight, mask_mode, d):
+    if weight == 3 and n == 2 * m:
+        code = I.ldpc_regular_code(n, m, 3, 6, seed=n)
+    else:
+        code = random_code(n, m, weight, n + d)
+    model = I.random_model(code, d, 2, seed=n, spe_noise=True, activation=1 if weight == 5 else 0)
+    model.mask_mode = mask_mode
+    got = both(model, 2 * 152 // 3 + 5 if n <= 128 else 3, seed=m)
+    assert got[0][3] == 3 and got[1][3] == 1
+    same(got)
+
+
+@pytest.mark.gpu
+def test_staged_attention_takes_what_the_buffers_hold():
+    # 642 tokens: past the rows of the staged buffers, the per-row walk stays; and an explicit request for
+    # staged attention at d = 64 is refused as before
+    code = I.ldpc_regular_code(428, 214, 3, 6, seed=1)
+    for d in (64, 128):
+        dec = A.Decoder(I.random_model(code, d, 1, seed=1, spe_noise=True))
+        assert dec.query()["attention_mode"] == 1
+        dec.close()
+    st, h = A.create_handle(I.random_model(I.make_code("ldpc128_64"), 64, 1, seed=1), attention_mode=3)
+    assert st == A.AECCT_ERR_UNSUPPORTED and h is None
