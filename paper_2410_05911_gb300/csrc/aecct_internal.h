@@ -274,8 +274,7 @@ constexpr int kSpeMaxHeads = 8;
 constexpr int kSpeMaxTokens = 1024;
 cudaError_t run_spe_table(const uint8_t *H, int n, int m, int d_spe, int heads, const double *w_pe, const double *wq,
                           const double *wk, const double *wv, const double *wo, double cluster_tol, double vanish_tol,
-                          float *spe_host, double *lam_host, double *U_host, double *spe64_host, int *sweeps,
-                          int *status_host);
+                          float *spe_host, double *lam_host, double *U_host, double *spe64_host, int *status_host);
 
 // api.cu diagnostics kernels live in selftest.cu
 cudaError_t run_selftest_mma(const int8_t *a_host, const int8_t *b_host, int K, int N, float *out_host);

@@ -1132,9 +1132,9 @@ int aecct_spe_table(const uint8_t *H, int32_t n, int32_t k, int32_t d_spe, int32
   const int m = n - k;
   for (size_t i = 0; i < static_cast<size_t>(m) * n; ++i)
     if (H[i] > 1) return AECCT_ERR_INVALID_ARG;
-  int sweeps = 0, status = 0;
+  int status = 0;
   const cudaError_t e = run_spe_table(H, n, m, d_spe, heads, w_pe, wq, wk, wv, wo, 1e-8, 1e-6, spe_out, lam_out, U_out,
-                                      spe64_out, &sweeps, &status);
+                                      spe64_out, &status);
   if (e != cudaSuccess) return cuda_fail(e, "spe table");
   if (status) {
     g_last_error = "spe table: a cluster of equal eigenvalues did not yield a full canonical basis";

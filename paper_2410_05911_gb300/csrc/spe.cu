@@ -1,24 +1,35 @@
 // spe.cu -- the spectral positional encoding of Sec. 4.3 computed on the GPU (aecct_spe_table), in
-// double precision:
+// double precision (GB300 executes two double FMAs per cycle and SM, so operations are counted here):
 //
-//   jacobi_kernel     eigenpairs of the Tanner-graph Laplacian L = D - A by the parallel (two-sided)
-//                     Jacobi method: every step rotates n/2 disjoint index pairs (p, q) of a
-//                     round-robin tournament, each rotation chosen from the current 2 x 2 block so
-//                     that A[p][q] becomes 0, applied to the rows, then the columns of A and of the
-//                     eigenvector matrix V; a sweep is n - 1 steps; sweeps repeat until the
-//                     off-diagonal sum of squares is below 1e-30 of the Frobenius norm squared.  One
-//                     cooperative launch, grid-wide barriers between the phases.
-//   sort_kernel       eigenpairs in ascending order (rank by counting, ties by index).
-//   canonical_kernel  per cluster of equal eigenvalues (consecutive gaps <= cluster_tol x
-//                     max(1, |lambda|max)), the canonical basis: Gram-Schmidt of P e_0, P e_1, ...
-//                     in node order, P = U_c U_c^T the cluster's projector, skipping residuals of
-//                     norm <= vanish_tol (projections removed twice, "twice is enough").
+//   tridiag_kernel    the Tanner-graph Laplacian L = D - A reduced to tridiagonal form by Householder
+//                     reflections (4/3 T^3 operations, where Jacobi rotations take about 10 sweeps of
+//                     6 T^3).  One cooperative launch; the rows stay in shared memory and a step
+//                     takes one grid-wide barrier.
+//   bisect_kernel     the eigenvalues of the tridiagonal matrix by bisection on Sturm counts.
+//   group_kernel      clusters of equal eigenvalues (consecutive gaps <= cluster_tol x
+//                     max(1, |lambda|max)).
+//   invit_kernel      eigenvectors of the tridiagonal matrix by inverse iteration from random vectors
+//                     (for a cluster: vectors that span its invariant subspace).
+//   gram_kernel, chol_kernel, trsm_kernel
+//                     an orthonormal basis of each cluster's subspace: V <- L^-1 V with V V^T = L L^T,
+//                     twice (Cholesky QR, whose second round leaves the orthogonality of a Householder
+//                     factorisation).
+//   back_kernel       the reflections applied to the eigenvectors.
+//   canonical_kernel  per cluster, the canonical basis: Gram-Schmidt of P e_0, P e_1, ... in node
+//                     order, P the cluster's projector, skipping residuals of norm <= vanish_tol; in the
+//                     coordinates of the cluster's basis, where P e_j is row j of it.  For a large cluster
+//                     select_kernel finds the nodes whose residual does not vanish, and their rows take the
+//                     same Cholesky QR.
+//   basis_kernel      the canonical basis vectors in node coordinates.
 //   mhsa_kernel       SPE_j = mean over rows of MHSA(Phi_j W_pe), Phi_j row i = (lambda_i, phi_i[j]):
 //                     every projection of row i is lambda_i (w0 W) + phi_i[j] (w1 W) for the rows
 //                     w0, w1 of W_pe, so each head's scores are a 2 x 2 bilinear form and
 //                     softmax(S) V_j = (P lambda)(w0 Wv) + (P phi[j])(w1 Wv); two passes per query
 //                     row (maximum, then the sums).
-#include <cooperative_groups.h>
+//
+// The long code of 576 nodes (LDPC(384,192)), where Jacobi rotations (about 10 sweeps of 575 steps with
+// three grid-wide barriers each) and Gram-Schmidt in node coordinates took 327 ms: tridiagonal form 4.9 ms,
+// eigenvalues 1.2, inverse iteration 0.8, the clusters' bases 2.3, reflections 1.4, canonical basis 3.9.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -27,115 +38,14 @@
 
 #include "aecct_internal.h"
 
-namespace cg = cooperative_groups;
-
 namespace aecct {
 
 namespace {
 
-constexpr int kJacobiThreads = 256;
-constexpr int kMaxSweeps = 100;
-
-// index of player k at step s of the round-robin tournament on n players (player 0 stays put)
-__device__ __forceinline__ int rr_player(int k, int s, int n) { return k == 0 ? 0 : ((k - 1 + s) % (n - 1)) + 1; }
-
-__global__ void __launch_bounds__(kJacobiThreads) jacobi_kernel(double *A, double *V, int T, int n, double *cs,
-                                                               double *acc, int *sweeps_out) {
-  cg::grid_group grid = cg::this_grid();
-  const int64_t tid = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  const int64_t nthreads = static_cast<int64_t>(gridDim.x) * blockDim.x;
-  __shared__ double red[kJacobiThreads / 32];
-  auto block_sum_atomic = [&](double v, double *dst) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double s = 0.0;
-      for (int w = 0; w < kJacobiThreads / 32; ++w) s += red[w];
-      atomicAdd(dst, s);
-    }
-    __syncthreads();
-  };
-  // acc[0]: Frobenius norm squared; acc[1 + s]: off-diagonal sum of squares before sweep s
-  {
-    double f = 0.0;
-    for (int64_t i = tid; i < static_cast<int64_t>(T) * T; i += nthreads) f += A[i] * A[i];
-    block_sum_atomic(f, acc);
-  }
-  int sweep = 0;
-  for (; sweep < kMaxSweeps; ++sweep) {
-    grid.sync();
-    double off = 0.0;
-    for (int64_t i = tid; i < static_cast<int64_t>(T) * T; i += nthreads) {
-      const int r = static_cast<int>(i / T), c = static_cast<int>(i % T);
-      if (r != c) off += A[i] * A[i];
-    }
-    block_sum_atomic(off, acc + 1 + sweep);
-    grid.sync();
-    if (acc[1 + sweep] <= 1e-30 * acc[0]) break;
-    for (int s = 0; s < n - 1; ++s) {
-      // the rotations of this step (a pair with the padding player n - 1 >= T does nothing)
-      for (int64_t k = tid; k < n / 2; k += nthreads) {
-        int p = rr_player(static_cast<int>(k), s, n), q = rr_player(n - 1 - static_cast<int>(k), s, n);
-        double c = 1.0, sn = 0.0;
-        if (p < T && q < T) {
-          const double apq = A[static_cast<int64_t>(p) * T + q];
-          if (apq != 0.0) {
-            const double app = A[static_cast<int64_t>(p) * T + p], aqq = A[static_cast<int64_t>(q) * T + q];
-            const double tau = (aqq - app) / (2.0 * apq);
-            const double t = (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau));
-            c = 1.0 / sqrt(1.0 + t * t);
-            sn = t * c;
-          }
-        }
-        cs[2 * k] = c;
-        cs[2 * k + 1] = sn;
-      }
-      grid.sync();
-      // rows p and q of A
-      for (int64_t it = tid; it < static_cast<int64_t>(n / 2) * T; it += nthreads) {
-        const int k = static_cast<int>(it / T), col = static_cast<int>(it % T);
-        const int p = rr_player(k, s, n), q = rr_player(n - 1 - k, s, n);
-        if (p >= T || q >= T) continue;
-        const double c = cs[2 * k], sn = cs[2 * k + 1];
-        const double apk = A[static_cast<int64_t>(p) * T + col], aqk = A[static_cast<int64_t>(q) * T + col];
-        A[static_cast<int64_t>(p) * T + col] = c * apk - sn * aqk;
-        A[static_cast<int64_t>(q) * T + col] = sn * apk + c * aqk;
-      }
-      grid.sync();
-      // columns p and q of A and of V
-      for (int64_t it = tid; it < static_cast<int64_t>(n / 2) * T; it += nthreads) {
-        const int k = static_cast<int>(it / T), row = static_cast<int>(it % T);
-        const int p = rr_player(k, s, n), q = rr_player(n - 1 - k, s, n);
-        if (p >= T || q >= T) continue;
-        const double c = cs[2 * k], sn = cs[2 * k + 1];
-        const int64_t rp = static_cast<int64_t>(row) * T + p, rq = static_cast<int64_t>(row) * T + q;
-        const double akp = A[rp], akq = A[rq];
-        A[rp] = c * akp - sn * akq;
-        A[rq] = sn * akp + c * akq;
-        const double vkp = V[rp], vkq = V[rq];
-        V[rp] = c * vkp - sn * vkq;
-        V[rq] = sn * vkp + c * vkq;
-      }
-      grid.sync();
-    }
-  }
-  if (tid == 0) *sweeps_out = sweep;
-}
-
-// ascending order: rank of eigenvalue i = #{j : lam_j < lam_i, or lam_j == lam_i and j < i}
-__global__ void sort_kernel(const double *A, const double *V, int T, double *lam, double *U) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= T) return;
-  const double li = A[static_cast<int64_t>(i) * T + i];
-  int rank = 0;
-  for (int j = 0; j < T; ++j) {
-    const double lj = A[static_cast<int64_t>(j) * T + j];
-    rank += (lj < li || (lj == li && j < i)) ? 1 : 0;
-  }
-  lam[rank] = li;
-  for (int r = 0; r < T; ++r) U[static_cast<int64_t>(r) * T + rank] = V[static_cast<int64_t>(r) * T + i];
-}
+constexpr int kTriThreads = 256;
+constexpr int kInvitIters = 3;
+constexpr int kSeqGroup = 24;         // clusters up to this size: Gram-Schmidt by one CTA
+constexpr double kEps = 2.220446049250313e-16;
 
 // block-wide sum of one double per thread (every thread gets the result)
 __device__ double block_sum(double v, double *red) {
@@ -148,56 +58,635 @@ __device__ double block_sum(double v, double *red) {
   return s;
 }
 
-// one CTA per eigenvalue index i; the CTA of a cluster's first index builds its canonical basis
-__global__ void canonical_kernel(const double *lam, const double *U, int T, double cluster_tol, double vanish_tol,
-                                 double *Uc, double *vbuf, double *dots, int *status) {
-  __shared__ double red[32];
-  const int i = blockIdx.x;
-  double amax = 1.0;
-  for (int j = 0; j < T; ++j) amax = fmax(amax, fabs(lam[j]));
-  const double tol = cluster_tol * amax;
-  if (i > 0 && lam[i] - lam[i - 1] <= tol) return;  // not the first index of its cluster
-  int j1 = i + 1;
-  while (j1 < T && lam[j1] - lam[j1 - 1] <= tol) ++j1;
-  const int r = j1 - i;
-  double *v = vbuf + static_cast<int64_t>(i) * T;  // this cluster's working vector
-  double *dt = dots + static_cast<int64_t>(i) * T;  // its projection coefficients (r <= T)
-  int got = 0;
-  for (int node = 0; node < T && got < r; ++node) {
-    // v = P e_node = U_c (U_c^T e_node): column a of the cluster weighted by U[node][a]
-    for (int a = threadIdx.x; a < T; a += blockDim.x) {
-      double s = 0.0;
-      for (int c = i; c < j1; ++c) s += U[static_cast<int64_t>(a) * T + c] * U[static_cast<int64_t>(node) * T + c];
-      v[a] = s;
+// the sum of one double per thread of a 256-thread CTA, through one of two buffers in turn (one barrier)
+__device__ __forceinline__ double block_sum8(double v, double *red) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  return ((red[0] + red[1]) + (red[2] + red[3])) + ((red[4] + red[5]) + (red[6] + red[7]));
+}
+
+// Barrier of a cooperative launch: every CTA adds one to `count` and thread 0 waits until it reaches
+// `target`, with `polls` left for all of a launch's barriers (its CTAs are resident together; past the
+// limit `status` is set and the launch runs on to its end without waiting).
+constexpr int kBarrierPolls = 1 << 25;
+__device__ __forceinline__ void grid_barrier(unsigned *count, unsigned target, int &polls, int *status) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned seen;
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(count) : "memory");
+    do {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(seen) : "l"(count) : "memory");
+    } while (seen < target && --polls > 0);
+    if (seen < target) atomicOr(status, 2);
+  }
+  __syncthreads();
+}
+
+// Householder tridiagonalisation of the Laplacian of H [m][n].  CTA b holds rows b, b + grid, ... in
+// shared memory.  Step k: every CTA forms column k of the matrix as updated by the steps before k, its
+// reflection v (v[k + 1] = 1, zeros up to k; row k of Vh) and tau, applies the update of step k - 1 to
+// its rows and multiplies them by v; after the barrier every CTA forms w = tau A v - (tau/2)(tau v^T A v) v
+// for the rank-2 update A - v w^T - w v^T of this step, which it applies in the next pass.  Column k comes
+// from row k as it was before the update of step k - 1, which its owner left in rowbuf[k & 1].
+// d and e receive the diagonal and the off-diagonal.  Bound by the latency of a step (the barrier, two
+// block sums, a square root and two divisions); the vector work that every CTA repeats costs less than
+// a second barrier would.
+__global__ void __launch_bounds__(kTriThreads) tridiag_kernel(const uint8_t *__restrict__ H, int n, int m, double *Vh,
+                                                             double *tau, double *d, double *e, double *rowbuf,
+                                                             double *pbuf, unsigned *count, int *status) {
+  extern __shared__ double sh[];
+  __shared__ double red[2][kTriThreads / 32], s_col[2];
+  const int T = n + m, G = gridDim.x, b = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  double *v = sh, *w = sh + T, *vn = sh + 2 * T, *rows = sh + 3 * T;
+  const int R = (T + G - 1) / G;
+  unsigned target = G;
+  int polls = kBarrierPolls;
+  for (int rr = warp; rr < R; rr += kTriThreads / 32) {
+    const int i = b + rr * G;
+    if (i >= T) continue;
+    double deg = 0.0;
+    for (int j = lane; j < T; j += 32) {
+      double a = 0.0;
+      if (i < n && j >= n && H[static_cast<size_t>(j - n) * n + i]) a = -1.0;
+      if (i >= n && j < n && H[static_cast<size_t>(i - n) * n + j]) a = -1.0;
+      rows[static_cast<size_t>(rr) * T + j] = a;
+      deg -= a;
+    }
+    for (int o = 16; o > 0; o >>= 1) deg += __shfl_xor_sync(0xffffffffu, deg, o);
+    __syncwarp();
+    if (lane == 0) rows[static_cast<size_t>(rr) * T + i] = deg;
+    __syncwarp();
+    if (i == 0)
+      for (int j = lane; j < T; j += 32) rowbuf[j] = rows[j];
+  }
+  grid_barrier(count, target, polls, status);
+  double wk = 0.0;  // w[k] of step k - 1 (its v[k] is 1)
+  for (int k = 0; k + 2 < T; ++k) {
+    const double *rb = rowbuf + static_cast<size_t>(k & 1) * T;
+    double s = 0.0;
+    for (int j = k + tid; j < T; j += kTriThreads) {
+      double c = __ldcg(rb + j);
+      if (k > 0) c = c - w[j] - wk * v[j];
+      vn[j] = c;
+      if (j <= k + 1) s_col[j - k] = c;
+      else s = fma(c, c, s);
+    }
+    s = block_sum8(s, red[0]);
+    const double dk = s_col[0], alpha = s_col[1];
+    double beta = alpha, tk = 0.0, sc = 0.0;
+    if (s > 0.0) {
+      beta = -copysign(sqrt(fma(alpha, alpha, s)), alpha);
+      tk = (beta - alpha) / beta;
+      sc = 1.0 / (alpha - beta);
+    }
+    if (b == 0 && tid == 0) d[k] = dk, e[k] = beta, tau[k] = tk;
+    for (int j = k + tid; j < T; j += kTriThreads)
+      if (j > k) vn[j] = j == k + 1 ? 1.0 : vn[j] * sc;
+    __syncthreads();
+    for (int rr = warp; rr < R; rr += kTriThreads / 32) {
+      const int i = b + rr * G;
+      if (i <= k || i >= T) continue;
+      double *row = rows + static_cast<size_t>(rr) * T;
+      const double vi = k > 0 ? v[i] : 0.0, wi = k > 0 ? w[i] : 0.0;
+      double *next = i == k + 1 ? rowbuf + static_cast<size_t>((k + 1) & 1) * T : nullptr;
+      double acc = 0.0;
+#pragma unroll 2
+      for (int j = k + 1 + lane; j < T; j += 32) {
+        double a = row[j];
+        if (k > 0) row[j] = a = fma(-vi, w[j], fma(-wi, v[j], a));
+        if (next) next[j] = a;
+        acc = fma(a, vn[j], acc);
+      }
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (lane == 0) pbuf[static_cast<size_t>(k & 1) * T + i] = acc;
+    }
+    target += G;
+    grid_barrier(count, target, polls, status);
+    const double *pb = pbuf + static_cast<size_t>(k & 1) * T;
+    const double p1 = __ldcg(pb + k + 1);
+    s = 0.0;
+    for (int j = k + 1 + tid; j < T; j += kTriThreads) {
+      const double pj = tk * __ldcg(pb + j);
+      w[j] = pj;
+      v[j] = vn[j];
+      s = fma(pj, vn[j], s);
+    }
+    s = block_sum8(s, red[1]);
+    const double kk = -0.5 * tk * s;
+    for (int j = k + 1 + tid; j < T; j += kTriThreads) {
+      w[j] = fma(kk, vn[j], w[j]);
+      if (b == k % G) Vh[static_cast<size_t>(k) * T + j] = vn[j];
+    }
+    wk = tk * p1 + kk;
+  }
+  __syncthreads();
+  // the last 2 x 2 block: row T - 2 as of the step before the last update, and the owner's row T - 1
+  const int q = T - 2;
+  if (b == 0 && tid == 0) {
+    const double *rb = rowbuf + static_cast<size_t>(q & 1) * T;
+    for (int j = q; j < T; ++j) {
+      const double c = fma(-v[q], w[j], fma(-w[q], v[j], __ldcg(rb + j)));
+      if (j == q) d[q] = c;
+      else e[q] = c;
+    }
+  }
+  if (b == (T - 1) % G && tid == 0)
+    d[T - 1] = fma(-2.0 * v[T - 1], w[T - 1], rows[static_cast<size_t>((T - 1) / G) * T + T - 1]);
+}
+
+// Eigenvalue i (ascending) by bisection into 17 parts a round, 16 lanes an eigenvalue (2 to a warp): the
+// number of eigenvalues below x is the number of sign changes in the Sturm sequence
+// p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2} (a zero counts as the sign opposite to its predecessor's),
+// rescaled by a power of two every 8 steps.  The recurrence without divisions takes three double
+// operations a step.  e^2 is kept above (1e-18 |L|)^2, far below rounding, so that a split matrix
+// does not end the sequence in zeros.
+__global__ void __launch_bounds__(32) bisect_kernel(const double *__restrict__ d, const double *__restrict__ e, int T,
+                                                   double *lam) {
+  extern __shared__ double2 de[];  // d_i and e_{i-1}^2
+  const int lane = threadIdx.x, i = blockIdx.x * 2 + (lane >> 4), sub = lane & 15;
+  double lo = INFINITY, hi = -INFINITY;
+  for (int j = lane; j < T; j += 32) {
+    const double r = (j > 0 ? fabs(e[j - 1]) : 0.0) + (j + 1 < T ? fabs(e[j]) : 0.0);
+    lo = fmin(lo, d[j] - r), hi = fmax(hi, d[j] + r);
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+  const double nt = fmax(fabs(lo), fabs(hi));
+  for (int j = lane; j < T; j += 32)
+    de[j] = make_double2(d[j], j > 0 ? fmax(e[j - 1] * e[j - 1], 1e-36 * nt * nt) : 0.0);
+  __syncwarp();
+  lo -= 8.0 * kEps * nt * T, hi += 8.0 * kEps * nt * T;
+  for (int round = 0; round < 15; ++round) {
+    const double h = (hi - lo) / 17.0, x = fma(h, static_cast<double>(sub + 1), lo);
+    double p0 = 1.0, p1 = de[0].x - x;
+    int sign = p1 <= 0.0 ? 1 : 0, cnt = sign;  // sign of the last term: 1 negative
+    auto step = [&](const double2 &c) {
+      const double p2 = fma(c.x - x, p1, -c.y * p0);
+      p0 = p1, p1 = p2;
+      const int hw = __double2hiint(p2);
+      const int now = ((hw << 1) | __double2loint(p2)) == 0 ? 1 - sign : static_cast<int>(static_cast<unsigned>(hw) >> 31);
+      cnt += now ^ sign;
+      sign = now;
+    };
+    auto rescale = [&]() {
+      const int ex = max(__double2hiint(p0) & 0x7FF00000, __double2hiint(p1) & 0x7FF00000);
+      const double f = __hiloint2double(ex == 0 ? 0x5FF00000 : 0x7FE00000 - ex, 0);  // 2^-(exponent)
+      p0 *= f, p1 *= f;
+    };
+    int j = 1;
+#pragma unroll 1
+    for (; j + 8 <= T; j += 8) {
+      double2 c[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) c[u] = de[j + u];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) step(c[u]);
+      rescale();
+    }
+    for (; j < T; ++j) step(de[j]);
+    const uint32_t above = __ballot_sync(0xffffffffu, cnt > i) >> (lane & 16) & 0xFFFFu;
+    const int f = above ? __ffs(above) - 1 : 16;  // the first point with more than i eigenvalues below it
+    const double base = lo;
+    if (f < 16) hi = fma(h, static_cast<double>(f + 1), base);
+    if (f > 0) lo = fma(h, static_cast<double>(f), base);
+  }
+  if (i < T && sub == 0) lam[i] = 0.5 * (lo + hi);
+}
+
+// ascending eigenvalues (equal ones can come out of the bisection a rounding apart in either order) and
+// their clusters: gs[i] the first index of i's cluster, gn[i] its size
+__global__ void __launch_bounds__(kSpeMaxTokens) group_kernel(double *lam, int T, double cluster_tol, int *gs, int *gn) {
+  __shared__ double x[kSpeMaxTokens];
+  __shared__ int first[kSpeMaxTokens + 1];
+  const int i = threadIdx.x;
+  if (i < T) x[i] = lam[i];
+  __syncthreads();
+  for (int o = 1; o < T; o <<= 1) {  // running maximum
+    const double y = i < T && i >= o ? fmax(x[i], x[i - o]) : (i < T ? x[i] : 0.0);
+    __syncthreads();
+    if (i < T) x[i] = y;
+    __syncthreads();
+  }
+  const double tol = cluster_tol * fmax(1.0, fmax(fabs(x[0]), fabs(x[T - 1])));
+  if (i < T) {
+    lam[i] = x[i];
+    first[i] = i == 0 || x[i] - x[i - 1] > tol;
+  }
+  if (i == 0) first[T] = 1;
+  __syncthreads();
+  if (i >= T) return;
+  int a = i, z = i + 1;
+  while (!first[a]) --a;
+  while (!first[z]) ++z;
+  gs[i] = a;
+  gn[i] = z - a;
+}
+
+// Inverse iteration on the tridiagonal matrix, a thread per eigenvector (nv to a CTA, their factors in
+// shared memory): (T - s I) = P L U with row exchanges, then kInvitIters solves from a random vector.  A
+// single eigenvalue is its own shift s; a cluster's shift lies 1e-10 |L| beside it, so that every vector
+// of its subspace is amplified alike and the random starts stay independent.  Row i of Z is vector i.
+__global__ void invit_kernel(const double *__restrict__ d, const double *__restrict__ e, const double *__restrict__ lam,
+                             const int *__restrict__ gn, int T, int nv, uint32_t seed, double *Z) {
+  extern __shared__ double sh[];
+  const int t = threadIdx.x, vec = blockIdx.x * nv + t;
+  if (t >= nv || vec >= T) return;
+  double *u0 = sh, *u1 = u0 + static_cast<size_t>(T) * nv, *u2 = u1 + static_cast<size_t>(T) * nv,
+         *lf = u2 + static_cast<size_t>(T) * nv, *x = lf + static_cast<size_t>(T) * nv;
+  uint8_t *sw = reinterpret_cast<uint8_t *>(x + static_cast<size_t>(T) * nv);
+  const double nt = fmax(fmax(fabs(lam[0]), fabs(lam[T - 1])), 1e-290);
+  const double tiny = 1e-2 * kEps * nt, s = lam[vec] + (gn[vec] > 1 ? 1e-10 * nt : 0.0);
+  double a = d[0] - s, b = e[0];
+  for (int i = 0; i + 1 < T; ++i) {
+    const double c = e[i], dn = d[i + 1] - s, en = i + 2 < T ? e[i + 1] : 0.0;
+    const bool swap = fabs(c) > fabs(a);
+    double piv = swap ? c : a;
+    if (fabs(piv) < tiny) piv = tiny;
+    const double r1 = swap ? dn : b, r2 = swap ? en : 0.0, rp = 1.0 / piv, l = (swap ? a : c) * rp;
+    u0[i * nv + t] = rp, u1[i * nv + t] = r1, u2[i * nv + t] = r2, lf[i * nv + t] = l;
+    sw[i * nv + t] = swap;
+    a = fma(-l, r1, swap ? b : dn);
+    b = fma(-l, r2, swap ? 0.0 : en);
+  }
+  u0[(T - 1) * nv + t] = 1.0 / (fabs(a) < tiny ? tiny : a);
+  uint32_t h = seed + 2654435761u * static_cast<uint32_t>(vec + 1);
+  for (int i = 0; i < T; ++i) {
+    h ^= h << 13, h ^= h >> 17, h ^= h << 5;
+    x[i * nv + t] = static_cast<double>(static_cast<int32_t>(h)) * 4.656612873077393e-10;
+  }
+  double norm = 1.0;
+  for (int it = 0; it < kInvitIters; ++it) {
+    double y = x[t] * norm;
+    for (int i = 0; i + 1 < T; ++i) {
+      const double yn = x[(i + 1) * nv + t] * norm;
+      const bool swap = sw[i * nv + t] != 0;
+      const double p = swap ? yn : y;
+      x[i * nv + t] = p;
+      y = fma(-lf[i * nv + t], p, swap ? y : yn);
+    }
+    double z1 = y * u0[(T - 1) * nv + t], z2 = 0.0, ss = z1 * z1;
+    x[(T - 1) * nv + t] = z1;
+    for (int i = T - 2; i >= 0; --i) {
+      const double z = fma(-u1[i * nv + t], z1, fma(-u2[i * nv + t], z2, x[i * nv + t])) * u0[i * nv + t];
+      x[i * nv + t] = z;
+      ss = fma(z, z, ss);
+      z2 = z1, z1 = z;
+    }
+    norm = 1.0 / sqrt(ss);
+  }
+  for (int i = 0; i < T; ++i) Z[static_cast<size_t>(vec) * T + i] = x[i * nv + t] * norm;
+}
+
+// length of the vectors of a cluster of size r: T (rows of the eigenvector array) or r (coordinates)
+__device__ __forceinline__ int vec_len(int r, int T, int coords) { return coords ? r : T; }
+
+// Gm[a][b] = row a of V . row b of V for a >= b of one cluster larger than rmin (32 x 32 tiles)
+__global__ void __launch_bounds__(256) gram_kernel(const double *__restrict__ V, const int *__restrict__ gs,
+                                                  const int *__restrict__ gn, int T, int rmin, int coords, double *Gm) {
+  __shared__ double sa[32][33], sb[32][33];
+  const int a0 = blockIdx.y * 32, b0 = blockIdx.x * 32;
+  if (b0 > a0) return;
+  int len = 0;
+  for (int a = a0; a < min(a0 + 32, T); ++a)
+    if (gn[a] > rmin && gs[a] <= min(b0 + 31, a)) len = max(len, vec_len(gn[a], T, coords));
+  if (len == 0) return;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+  for (int c0 = 0; c0 < len; c0 += 32) {
+    for (int it = threadIdx.x; it < 1024; it += 256) {
+      const int rr = it >> 5, c = c0 + (it & 31), a = a0 + rr, b = b0 + rr;
+      sa[rr][it & 31] = a < T && c < vec_len(gn[a], T, coords) ? V[static_cast<size_t>(a) * T + c] : 0.0;
+      sb[rr][it & 31] = b < T && c < vec_len(gn[b], T, coords) ? V[static_cast<size_t>(b) * T + c] : 0.0;
     }
     __syncthreads();
-    // remove the projections on the vectors chosen so far, twice (one warp per coefficient)
-    for (int pass = 0; pass < 2 && got > 0; ++pass) {
-      const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-      for (int b = threadIdx.x >> 5; b < got; b += nw) {
-        double s = 0.0;
-        for (int a = lane; a < T; a += 32) s += Uc[static_cast<int64_t>(a) * T + i + b] * v[a];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) dt[b] = s;
+#pragma unroll 8
+    for (int c = 0; c < 32; ++c) {
+      const double x0 = sa[ty][c], x1 = sa[ty + 16][c], y0 = sb[tx][c], y1 = sb[tx + 16][c];
+      acc[0][0] = fma(x0, y0, acc[0][0]), acc[0][1] = fma(x0, y1, acc[0][1]);
+      acc[1][0] = fma(x1, y0, acc[1][0]), acc[1][1] = fma(x1, y1, acc[1][1]);
+    }
+    __syncthreads();
+  }
+  for (int i = 0; i < 2; ++i)
+    for (int j = 0; j < 2; ++j) {
+      const int a = a0 + ty + 16 * i, b = b0 + tx + 16 * j;
+      if (a < T && b <= a && gs[a] <= b) Gm[static_cast<size_t>(a) * T + b] = acc[i][j];
+    }
+}
+
+// In place, L of Gm = L L^T of every cluster larger than rmin (one CTA each, its lower triangle in shared
+// memory where it fits).  A squared pivot of at most `thr` marks the cluster in `bad`.  Columns go in
+// panels of 16: one warp factors the panel's diagonal block, every thread a row of the rest of the
+// panel, and the trailing triangle takes the panel's update in one pass.
+constexpr int kCholThreads = 512;
+constexpr int kCholPanel = 16;
+constexpr int kCholShared = 216;  // rows of a triangle in shared memory: 187,488 bytes
+constexpr size_t kCholSmem = sizeof(double) * kCholShared * (kCholShared + 1) / 2;
+__global__ void __launch_bounds__(kCholThreads) chol_kernel(double *Gm, const int *__restrict__ gs,
+                                                            const int *__restrict__ gn, int T, int rmin, double thr,
+                                                            int *bad) {
+  extern __shared__ double tri[];
+  __shared__ double diag[kCholPanel][kCholPanel + 1], dinv[kCholPanel];
+  const int g0 = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (gs[g0] != g0 || gn[g0] <= rmin) return;
+  const int r = gn[g0];
+  const bool packed = r <= kCholShared;
+  auto glob = [&](int a, int b) -> double * { return Gm + static_cast<size_t>(g0 + a) * T + g0 + b; };
+  auto at = [&](int a, int b) -> double * { return packed ? tri + a * (a + 1) / 2 + b : glob(a, b); };
+  if (packed)
+    for (int a = warp; a < r; a += kCholThreads / 32)
+      for (int b = lane; b <= a; b += 32) *at(a, b) = *glob(a, b);
+  __syncthreads();
+  bool ok = true;
+  for (int j0 = 0; j0 < r; j0 += kCholPanel) {
+    const int nb = min(kCholPanel, r - j0);
+    if (warp == 0) {
+      // lane a holds row j0 + a of the diagonal block
+      double x[kCholPanel];
+#pragma unroll
+      for (int c = 0; c < kCholPanel; ++c) x[c] = lane < nb && c <= lane ? *at(j0 + lane, j0 + c) : (c == lane ? 1.0 : 0.0);
+#pragma unroll
+      for (int c = 0; c < kCholPanel; ++c) {
+        const double piv = __shfl_sync(0xffffffffu, x[c], c);
+        if (c < nb && !(piv > thr)) ok = false;
+        const double root = sqrt(fmax(piv, 1e-300)), inv = 1.0 / root;
+        x[c] = lane == c ? root : x[c] * inv;
+        if (lane == c) dinv[c] = inv;
+#pragma unroll
+        for (int k = c + 1; k < kCholPanel; ++k) {
+          const double lk = __shfl_sync(0xffffffffu, x[c], k);
+          if (lane >= k) x[k] = fma(-x[c], lk, x[k]);
+        }
+      }
+#pragma unroll
+      for (int c = 0; c < kCholPanel; ++c)
+        if (lane < nb && c <= lane) diag[lane][c] = *at(j0 + lane, j0 + c) = x[c];
+    }
+    __syncthreads();
+    for (int a = j0 + kCholPanel + tid; a < r; a += kCholThreads) {  // (a full panel: nb = kCholPanel)
+      double x[kCholPanel];
+#pragma unroll
+      for (int c = 0; c < kCholPanel; ++c) x[c] = *at(a, j0 + c);
+#pragma unroll
+      for (int c = 0; c < kCholPanel; ++c) {
+        x[c] *= dinv[c];
+#pragma unroll
+        for (int k = c + 1; k < kCholPanel; ++k) x[k] = fma(-x[c], diag[k][c], x[k]);
+      }
+#pragma unroll
+      for (int c = 0; c < kCholPanel; ++c) *at(a, j0 + c) = x[c];
+    }
+    __syncthreads();
+    for (int a = j0 + kCholPanel + warp; a < r; a += kCholThreads / 32) {
+      double la[kCholPanel];
+#pragma unroll
+      for (int c = 0; c < kCholPanel; ++c) la[c] = *at(a, j0 + c);
+      for (int b = j0 + kCholPanel + lane; b <= a; b += 32) {
+        double x0 = *at(a, b), x1 = 0.0;
+#pragma unroll
+        for (int c = 0; c < kCholPanel; c += 2) {
+          x0 = fma(-la[c], *at(b, j0 + c), x0);
+          x1 = fma(-la[c + 1], *at(b, j0 + c + 1), x1);
+        }
+        *at(a, b) = x0 + x1;
+      }
+    }
+    __syncthreads();
+  }
+  if (packed)
+    for (int a = warp; a < r; a += kCholThreads / 32)
+      for (int b = lane; b <= a; b += 32) *glob(a, b) = *at(a, b);
+  if (tid == 0 && !ok) bad[g0] = 1;
+}
+
+// The nodes of each cluster larger than kSeqGroup that give its canonical basis: the first r nodes, in
+// order, whose P e_j is independent of those chosen before (codes have exactly dependent ones).  A
+// right-looking Cholesky of P (over the nodes 0 .. S - 1) that leaves a node out where the
+// squared residual is below 1e-14; one between that and 1e-8, where this arithmetic cannot tell, or too few
+// nodes, mark the cluster for the one-by-one kernel.  node[g0 + a]: the a-th node chosen.
+__global__ void __launch_bounds__(kCholThreads) select_kernel(const double *__restrict__ V, const int *__restrict__ gs,
+                                                              const int *__restrict__ gn, int T, int rmin, int *node,
+                                                              int *bad) {
+  extern __shared__ double tri[];
+  __shared__ double col[kCholShared];
+  const int g0 = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (gs[g0] != g0 || gn[g0] <= rmin) return;
+  const int r = gn[g0], S = min(T, kCholShared);
+  if (r > S) {
+    if (tid == 0) bad[g0] = 1;
+    return;
+  }
+  // P[a][b] = sum_c X[g0 + c][a] X[g0 + c][b], 4 x 4 outputs a thread
+  const double *X = V + static_cast<size_t>(g0) * T;
+  const int nt = (S + 3) / 4, ntri = nt * (nt + 1) / 2;
+  for (int t = tid; t < ntri; t += kCholThreads) {
+    int ta = static_cast<int>((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
+    while ((ta + 1) * (ta + 2) / 2 <= t) ++ta;
+    while (ta * (ta + 1) / 2 > t) --ta;
+    const int a0 = 4 * ta, b0 = 4 * (t - ta * (ta + 1) / 2);
+    double acc[4][4] = {};
+    for (int c = 0; c < r; ++c) {
+      double xa[4], xb[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        xa[u] = a0 + u < S ? X[static_cast<size_t>(c) * T + a0 + u] : 0.0;
+        xb[u] = b0 + u < S ? X[static_cast<size_t>(c) * T + b0 + u] : 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[u][q] = fma(xa[u], xb[q], acc[u][q]);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (a0 + u < S && b0 + q <= a0 + u) tri[(a0 + u) * (a0 + u + 1) / 2 + b0 + q] = acc[u][q];
+  }
+  __syncthreads();
+  int got = 0;
+  bool ok = true;
+  for (int j = 0; j < S && got < r; ++j) {
+    const double piv = tri[j * (j + 1) / 2 + j];
+    if (!(piv > 1e-14)) continue;
+    if (!(piv > 1e-8)) ok = false;
+    if (tid == 0) node[g0 + got] = j;
+    ++got;
+    const double inv = 1.0 / sqrt(piv);
+    for (int a = j + 1 + tid; a < S; a += kCholThreads) col[a] = tri[a * (a + 1) / 2 + j] * inv;
+    __syncthreads();
+    for (int a = j + 1 + warp; a < S; a += kCholThreads / 32) {
+      const double ca = col[a];
+      for (int b = j + 1 + lane; b <= a; b += 32) tri[a * (a + 1) / 2 + b] = fma(-ca, col[b], tri[a * (a + 1) / 2 + b]);
+    }
+    __syncthreads();
+  }
+  if (tid == 0 && (!ok || got < r)) bad[g0] = 1;
+}
+
+// V <- L^-1 V for the rows of every cluster larger than rmin: 16 columns of V to a CTA, in blocks of 16
+// rows (the rows before the block subtracted by all threads, one row and column each, then the block's
+// 16 x 16 triangle one row after another)
+__global__ void __launch_bounds__(256) trsm_kernel(const double *__restrict__ Gm, double *V, const int *__restrict__ gs,
+                                                  const int *__restrict__ gn, int T, int rmin, int coords) {
+  __shared__ double lb[16][17], xb[16][17], rhs[16][17];
+  const int g0 = blockIdx.y, i0 = blockIdx.x * 16, c = threadIdx.x & 15, a = threadIdx.x >> 4;
+  if (gs[g0] != g0 || gn[g0] <= rmin) return;
+  const int r = gn[g0], len = vec_len(r, T, coords);
+  if (i0 >= len) return;
+  const bool in = i0 + c < len;
+  double *x = V + static_cast<size_t>(g0) * T + i0 + c;
+  for (int a0 = 0; a0 < r; a0 += 16) {
+    const bool row = a0 + a < r;
+    const double *la = Gm + static_cast<size_t>(g0 + a0 + a) * T + g0;
+    double s0 = row && in ? x[static_cast<size_t>(a0 + a) * T] : 0.0, s1 = 0.0;
+    for (int b0 = 0; b0 < a0; b0 += 16) {
+      lb[a][c] = row ? la[b0 + c] : 0.0;
+      xb[a][c] = in ? x[static_cast<size_t>(b0 + a) * T] : 0.0;
+      __syncthreads();
+#pragma unroll
+      for (int b = 0; b < 16; b += 2) {
+        s0 = fma(-lb[a][b], xb[b][c], s0);
+        s1 = fma(-lb[a][b + 1], xb[b + 1][c], s1);
       }
       __syncthreads();
-      for (int a = threadIdx.x; a < T; a += blockDim.x) {
-        double s = v[a];
-        for (int b = 0; b < got; ++b) s -= dt[b] * Uc[static_cast<int64_t>(a) * T + i + b];
-        v[a] = s;
+    }
+    lb[a][c] = row && a0 + c < r && c <= a ? la[a0 + c] : 0.0;
+    rhs[a][c] = s0 + s1;
+    __syncthreads();
+    if (threadIdx.x < 16) {  // thread c: column c of the block
+      double y[16];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) y[k] = rhs[k][c];
+#pragma unroll
+      for (int k = 0; k < 16; ++k) {
+        y[k] = a0 + k < r ? y[k] / lb[k][k] : 0.0;
+#pragma unroll
+        for (int q = k + 1; q < 16; ++q) y[q] = fma(-lb[q][k], y[k], y[q]);
+      }
+#pragma unroll
+      for (int k = 0; k < 16; ++k) rhs[k][c] = y[k];
+    }
+    __syncthreads();
+    if (row && in) x[static_cast<size_t>(a0 + a) * T] = rhs[a][c];
+    __syncthreads();
+  }
+}
+
+// Z <- (H_0 H_1 ... H_{T-3}) Z for every row of Z: a warp per vector, its elements j = lane + 32 u in
+// registers (NE per lane), the next reflection's vector loaded while the current one is applied
+template <int NE>
+__global__ void __launch_bounds__(128) back_kernel(const double *__restrict__ Vh, const double *__restrict__ tau, int T,
+                                                  double *Z) {
+  const int vec = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (vec >= T) return;
+  double z[NE], v[NE];
+#pragma unroll
+  for (int u = 0; u < NE; ++u) z[u] = lane + 32 * u < T ? Z[static_cast<size_t>(vec) * T + lane + 32 * u] : 0.0;
+  auto load = [&](int k) {
+#pragma unroll
+    for (int u = 0; u < NE; ++u) {
+      const int j = lane + 32 * u;
+      v[u] = k >= 0 && j > k && j < T ? __ldg(Vh + static_cast<size_t>(k) * T + j) : 0.0;
+    }
+  };
+  load(T - 3);
+  double tn = __ldg(tau + T - 3);
+  for (int k = T - 3; k >= 0; --k) {
+    double cur[NE], s[2] = {0.0, 0.0};
+    const double tk = tn;
+#pragma unroll
+    for (int u = 0; u < NE; ++u) cur[u] = v[u];
+    load(k - 1);
+    if (k > 0) tn = __ldg(tau + k - 1);
+    const int u0 = (k + 1) >> 5;
+#pragma unroll
+    for (int u = 0; u < NE; ++u)
+      if (u >= u0) s[u & 1] = fma(cur[u], z[u], s[u & 1]);
+    double t = s[0] + s[1];
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    t *= -tk;
+#pragma unroll
+    for (int u = 0; u < NE; ++u)
+      if (u >= u0) z[u] = fma(t, cur[u], z[u]);
+  }
+#pragma unroll
+  for (int u = 0; u < NE; ++u)
+    if (lane + 32 * u < T) Z[static_cast<size_t>(vec) * T + lane + 32 * u] = z[u];
+}
+
+// The chosen nodes' rows of a large cluster's basis, in its coordinates: Q[g0 + a][c]
+__global__ void coords_kernel(const double *__restrict__ X, const int *__restrict__ gs, const int *__restrict__ gn,
+                              const int *__restrict__ node, const int *__restrict__ bad, int T, int rmin, double *Q) {
+  const int row = blockIdx.x;
+  if (gn[row] <= rmin || bad[gs[row]]) return;
+  const int g0 = gs[row], a = node[row];
+  for (int c = threadIdx.x; c < gn[row]; c += blockDim.x)
+    Q[static_cast<size_t>(row) * T + c] = X[static_cast<size_t>(g0 + c) * T + a];
+}
+
+// Canonical basis in coordinates, Q[g0 + a][c], of every cluster up to kSeqGroup and of the larger ones
+// marked in `bad`: Gram-Schmidt of the rows P e_0, P e_1, ... one by one, each
+// projected twice ("twice is enough"), skipping residuals of norm <= vanish_tol.  One CTA per cluster.
+constexpr int kSeqThreads = 128;
+__global__ void __launch_bounds__(kSeqThreads) canonical_kernel(const double *__restrict__ X, const int *__restrict__ gs,
+                                                                const int *__restrict__ gn, int T, double vanish_tol,
+                                                                const int *__restrict__ bad, double *Q, int *status) {
+  __shared__ double red[kSeqThreads / 32], w[kSpeMaxTokens], dots[kSpeMaxTokens];
+  const int g0 = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (gs[g0] != g0) return;
+  const int r = gn[g0];
+  if (r > kSeqGroup && !bad[g0]) return;
+  int got = 0;
+  for (int node = 0; node < T && got < r; ++node) {
+    for (int c = tid; c < r; c += kSeqThreads) w[c] = X[static_cast<size_t>(g0 + c) * T + node];
+    __syncthreads();
+    for (int pass = 0; pass < 2 && got > 0; ++pass) {
+      for (int b = warp; b < got; b += kSeqThreads / 32) {
+        double s = 0.0;
+        for (int c = lane; c < r; c += 32) s = fma(Q[static_cast<size_t>(g0 + b) * T + c], w[c], s);
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) dots[b] = s;
+      }
+      __syncthreads();
+      for (int c = tid; c < r; c += kSeqThreads) {
+        double s = w[c];
+        for (int b = 0; b < got; ++b) s = fma(-dots[b], Q[static_cast<size_t>(g0 + b) * T + c], s);
+        w[c] = s;
       }
       __syncthreads();
     }
     double nv = 0.0;
-    for (int a = threadIdx.x; a < T; a += blockDim.x) nv += v[a] * v[a];
+    for (int c = tid; c < r; c += kSeqThreads) nv = fma(w[c], w[c], nv);
     nv = sqrt(block_sum(nv, red));
     if (nv > vanish_tol) {
-      for (int a = threadIdx.x; a < T; a += blockDim.x) Uc[static_cast<int64_t>(a) * T + i + got] = v[a] / nv;
+      for (int c = tid; c < r; c += kSeqThreads) Q[static_cast<size_t>(g0 + got) * T + c] = w[c] / nv;
       ++got;
     }
     __syncthreads();
   }
-  if (got != r && threadIdx.x == 0) atomicOr(status, 1);
+  if (got != r && tid == 0) atomicOr(status, 1);
+}
+
+// the canonical vectors in node coordinates: U[node][i] = sum_c X[g0 + c][node] Q[i][c]
+__global__ void __launch_bounds__(256) basis_kernel(const double *__restrict__ X, const double *__restrict__ Q,
+                                                   const int *__restrict__ gs, const int *__restrict__ gn, int T,
+                                                   double *U) {
+  __shared__ double out[32][9];
+  const int node = blockIdx.x * 32 + (threadIdx.x & 31), sub = threadIdx.x >> 5, i = blockIdx.y * 8 + sub;
+  double s = 0.0;
+  if (node < T && i < T) {
+    const int g0 = gs[i], r = gn[i];
+#pragma unroll 4
+    for (int c = 0; c < r; ++c) s = fma(X[static_cast<size_t>(g0 + c) * T + node], Q[static_cast<size_t>(i) * T + c], s);
+  }
+  out[threadIdx.x & 31][sub] = s;
+  __syncthreads();
+  const int rn = blockIdx.x * 32 + (threadIdx.x >> 3), ri = blockIdx.y * 8 + (threadIdx.x & 7);
+  if (rn < T && ri < T) U[static_cast<size_t>(rn) * T + ri] = out[threadIdx.x >> 3][threadIdx.x & 7];
 }
 
 struct MhsaCoef {
@@ -252,24 +741,20 @@ __global__ void mhsa_kernel(const double *lam, const double *U, int T, int heads
   }
 }
 
+// one Cholesky QR of the clusters larger than rmin
+void chol_qr(double *V, double *Gm, const int *gs, const int *gn, int T, int rmin, int coords, double thr, int *bad) {
+  const int nt = (T + 31) / 32;
+  gram_kernel<<<dim3(nt, nt), 256>>>(V, gs, gn, T, rmin, coords, Gm);
+  chol_kernel<<<T, kCholThreads, kCholSmem>>>(Gm, gs, gn, T, rmin, thr, bad);
+  trsm_kernel<<<dim3((T + 15) / 16, T), 256>>>(Gm, V, gs, gn, T, rmin, coords);
+}
+
 }  // namespace
 
 cudaError_t run_spe_table(const uint8_t *H, int n, int m, int d_spe, int heads, const double *w_pe, const double *wq,
                           const double *wk, const double *wv, const double *wo, double cluster_tol, double vanish_tol,
-                          float *spe_host, double *lam_host, double *U_host, double *spe64_host, int *sweeps,
-                          int *status_host) {
-  const int T = n + m, np = T + (T & 1);
-  const int d_e = d_spe / heads;
-  // the Laplacian on the host (a T x T 0/1 pattern), everything after it on the device
-  std::vector<double> Lh(static_cast<size_t>(T) * T, 0.0), Vh(static_cast<size_t>(T) * T, 0.0);
-  for (int i = 0; i < m; ++i)
-    for (int j = 0; j < n; ++j)
-      if (H[static_cast<size_t>(i) * n + j]) {
-        const int c = n + i;
-        Lh[static_cast<size_t>(j) * T + c] -= 1.0, Lh[static_cast<size_t>(c) * T + j] -= 1.0;
-        Lh[static_cast<size_t>(j) * T + j] += 1.0, Lh[static_cast<size_t>(c) * T + c] += 1.0;
-      }
-  for (int i = 0; i < T; ++i) Vh[static_cast<size_t>(i) * T + i] = 1.0;
+                          float *spe_host, double *lam_host, double *U_host, double *spe64_host, int *status_host) {
+  const int T = n + m, d_e = d_spe / heads;
   // the projections of the two rows of W_pe and the score forms per head
   MhsaCoef coef = {};
   std::vector<double> vah(static_cast<size_t>(d_spe)), vbh(static_cast<size_t>(d_spe));
@@ -290,55 +775,122 @@ cudaError_t run_spe_table(const uint8_t *H, int n, int m, int d_spe, int heads, 
     const double sc = 1.0 / std::sqrt(static_cast<double>(d_e));
     for (int t = 0; t < 4; ++t) coef.form[e][t] = f[t] * sc;
   }
-  double *A = nullptr, *V = nullptr, *U = nullptr, *Uc = nullptr, *lam = nullptr, *cs = nullptr, *acc = nullptr;
-  double *vbuf = nullptr, *dots = nullptr, *va = nullptr, *vb = nullptr, *wod = nullptr, *spe64 = nullptr;
-  float *spe = nullptr;
-  int *dsweeps = nullptr, *dstatus = nullptr;
-  const size_t TT = static_cast<size_t>(T) * T * sizeof(double);
+  // one allocation for everything
+  size_t bytes = 0;
+  auto part = [&](size_t size) {
+    const size_t off = bytes;
+    bytes += (size + 255) & ~static_cast<size_t>(255);
+    return off;
+  };
+  const size_t TT = static_cast<size_t>(T) * T * sizeof(double), T1 = static_cast<size_t>(T) * sizeof(double);
+  const size_t o_X = part(TT), o_V = part(TT), o_G = part(TT), o_U = part(TT), o_d = part(T1), o_e = part(T1),
+               o_tau = part(T1), o_lam = part(T1), o_row = part(2 * T1), o_p = part(2 * T1),
+               o_va = part(sizeof(double) * d_spe), o_vb = part(sizeof(double) * d_spe),
+               o_wo = part(sizeof(double) * d_spe * d_spe), o_spe64 = part(sizeof(double) * T * d_spe),
+               o_spe = part(sizeof(float) * T * d_spe), o_H = part(static_cast<size_t>(m) * n),
+               o_gs = part(sizeof(int) * T), o_gn = part(sizeof(int) * T), o_bad = part(sizeof(int) * 2 * T),
+               o_node = part(sizeof(int) * T), o_status = part(2 * sizeof(int));
+  uint8_t *base = nullptr;
   cudaError_t e = cudaSuccess;
-  int dev = 0, sms = 0, per_sm = 0;
   auto ok = [&](cudaError_t x) { return (e = x) == cudaSuccess; };
-  if (!ok(cudaMalloc(&A, TT)) || !ok(cudaMalloc(&V, TT)) || !ok(cudaMalloc(&U, TT)) || !ok(cudaMalloc(&Uc, TT)) ||
-      !ok(cudaMalloc(&vbuf, TT)) || !ok(cudaMalloc(&dots, TT)) || !ok(cudaMalloc(&lam, sizeof(double) * T)) ||
-      !ok(cudaMalloc(&cs, sizeof(double) * np)) || !ok(cudaMalloc(&acc, sizeof(double) * (kMaxSweeps + 1))) ||
-      !ok(cudaMalloc(&va, sizeof(double) * d_spe)) || !ok(cudaMalloc(&vb, sizeof(double) * d_spe)) ||
-      !ok(cudaMalloc(&wod, sizeof(double) * d_spe * d_spe)) || !ok(cudaMalloc(&spe, sizeof(float) * T * d_spe)) ||
-      !ok(cudaMalloc(&spe64, sizeof(double) * T * d_spe)) || !ok(cudaMalloc(&dsweeps, sizeof(int))) ||
-      !ok(cudaMalloc(&dstatus, sizeof(int))))
+  int dev = 0, sms = 0, per_sm = 0, R = 1, G = 1;
+  std::vector<int> bad(static_cast<size_t>(T));
+  if (!ok(cudaMalloc(&base, bytes))) return e;
+  auto dp = [&](size_t off) { return reinterpret_cast<double *>(base + off); };
+  double *X = dp(o_X), *V = dp(o_V), *Gm = dp(o_G), *U = dp(o_U), *d = dp(o_d), *ed = dp(o_e), *tau = dp(o_tau),
+         *lam = dp(o_lam), *rowbuf = dp(o_row), *pbuf = dp(o_p);
+  float *spe = reinterpret_cast<float *>(base + o_spe);
+  uint8_t *Hd = base + o_H;
+  int *gs = reinterpret_cast<int *>(base + o_gs), *gn = reinterpret_cast<int *>(base + o_gn),
+      *badd = reinterpret_cast<int *>(base + o_bad), *node = reinterpret_cast<int *>(base + o_node),
+      *dstatus = reinterpret_cast<int *>(base + o_status);
+  unsigned *count = reinterpret_cast<unsigned *>(dstatus + 1);
+  const int nt = (T + 31) / 32;
+  if (!ok(cudaMemcpy(Hd, H, static_cast<size_t>(m) * n, cudaMemcpyHostToDevice)) ||
+      !ok(cudaMemset(dstatus, 0, 2 * sizeof(int))) ||
+      !ok(cudaMemcpy(dp(o_va), vah.data(), sizeof(double) * d_spe, cudaMemcpyHostToDevice)) ||
+      !ok(cudaMemcpy(dp(o_vb), vbh.data(), sizeof(double) * d_spe, cudaMemcpyHostToDevice)) ||
+      !ok(cudaMemcpy(dp(o_wo), wo, sizeof(double) * d_spe * d_spe, cudaMemcpyHostToDevice)))
     goto done;
-  if (!ok(cudaMemcpy(A, Lh.data(), TT, cudaMemcpyHostToDevice)) || !ok(cudaMemcpy(V, Vh.data(), TT, cudaMemcpyHostToDevice)) ||
-      !ok(cudaMemset(acc, 0, sizeof(double) * (kMaxSweeps + 1))) || !ok(cudaMemset(dstatus, 0, sizeof(int))) ||
-      !ok(cudaMemset(Uc, 0, TT)) ||
-      !ok(cudaMemcpy(va, vah.data(), sizeof(double) * d_spe, cudaMemcpyHostToDevice)) ||
-      !ok(cudaMemcpy(vb, vbh.data(), sizeof(double) * d_spe, cudaMemcpyHostToDevice)) ||
-      !ok(cudaMemcpy(wod, wo, sizeof(double) * d_spe * d_spe, cudaMemcpyHostToDevice)))
-    goto done;
-  if (!ok(cudaGetDevice(&dev)) || !ok(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) ||
-      !ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_kernel, kJacobiThreads, 0)))
-    goto done;
+  // the tridiagonal form: one CTA per SM (fewer for a small matrix), each with R rows in shared memory
+  if (!ok(cudaGetDevice(&dev)) || !ok(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev))) goto done;
+  G = T < 2 * sms ? (T + 1) / 2 : sms;
+  R = (T + G - 1) / G;
   {
-    int Targ = T, narg = np;
-    void *args[] = {&A, &V, &Targ, &narg, &cs, &acc, &dsweeps};
-    const int blocks = sms * (per_sm < 2 ? per_sm : 2);
-    if (!ok(cudaLaunchCooperativeKernel(reinterpret_cast<void *>(jacobi_kernel), dim3(blocks), dim3(kJacobiThreads), args,
-                                        0, nullptr)))
+    const size_t smem = sizeof(double) * T * (3 + static_cast<size_t>(R));
+    if (!ok(cudaFuncSetAttribute(tridiag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem))) ||
+        !ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tridiag_kernel, kTriThreads, smem)))
+      goto done;
+    if (per_sm < 1) {
+      e = cudaErrorInvalidConfiguration;
+      goto done;
+    }
+    int narg = n, marg = m;
+    void *args[] = {&Hd, &narg, &marg, &V, &tau, &d, &ed, &rowbuf, &pbuf, &count, &dstatus};
+    if (!ok(cudaLaunchCooperativeKernel(reinterpret_cast<void *>(tridiag_kernel), dim3(G), dim3(kTriThreads), args, smem,
+                                        nullptr)))
       goto done;
   }
-  sort_kernel<<<(T + 127) / 128, 128>>>(A, V, T, lam, U);
-  canonical_kernel<<<T, 256>>>(lam, U, T, cluster_tol, vanish_tol, Uc, vbuf, dots, dstatus);
-  mhsa_kernel<<<T, 256, 2 * sizeof(double) * T>>>(lam, Uc, T, heads, coef, va, vb, wod, d_spe, spe, spe64);
+  bisect_kernel<<<(T + 1) / 2, 32, sizeof(double2) * T>>>(d, ed, T, lam);
+  group_kernel<<<1, kSpeMaxTokens>>>(lam, T, cluster_tol, gs, gn);
+  if (!ok(cudaFuncSetAttribute(chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kCholSmem))) ||
+      !ok(cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kCholSmem))))
+    goto done;
+  {
+    // inverse iteration, vectors of a CTA bounded by the shared memory of their factors; another seed where
+    // a cluster's random vectors came out dependent
+    const size_t per_vec = static_cast<size_t>(T) * (5 * sizeof(double) + 1);
+    int nv = static_cast<int>(220000 / per_vec);
+    nv = nv < 1 ? 1 : (nv > 32 ? 32 : nv);
+    const int want = (T + sms - 1) / sms;  // no more to a CTA than fills the SMs
+    nv = nv > want ? want : nv;
+    const size_t smem = per_vec * nv;
+    if (!ok(cudaFuncSetAttribute(invit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem))))
+      goto done;
+    for (uint32_t attempt = 0;; ++attempt) {
+      if (!ok(cudaMemset(badd, 0, sizeof(int) * 2 * T))) goto done;
+      invit_kernel<<<(T + nv - 1) / nv, 32, smem>>>(d, ed, lam, gn, T, nv, 12345u + 977u * attempt, X);
+      chol_qr(X, Gm, gs, gn, T, 1, 0, 1e-14, badd);
+      chol_qr(X, Gm, gs, gn, T, 1, 0, 1e-14, badd);
+      if (!ok(cudaGetLastError()) ||
+          !ok(cudaMemcpy(bad.data(), badd, sizeof(int) * T, cudaMemcpyDeviceToHost)))
+        goto done;
+      bool again = false;
+      for (int b : bad) again = again || b != 0;
+      if (!again) break;
+      if (attempt == 4) {
+        e = cudaErrorUnknown;
+        goto done;
+      }
+    }
+  }
+  if (T <= 128) back_kernel<4><<<(T + 3) / 4, 128>>>(V, tau, T, X);
+  else if (T <= 320) back_kernel<10><<<(T + 3) / 4, 128>>>(V, tau, T, X);
+  else if (T <= 576) back_kernel<18><<<(T + 3) / 4, 128>>>(V, tau, T, X);
+  else back_kernel<32><<<(T + 3) / 4, 128>>>(V, tau, T, X);
+  // the canonical basis in coordinates (V is free now), then in node coordinates
+  select_kernel<<<T, kCholThreads, kCholSmem>>>(X, gs, gn, T, kSeqGroup, node, badd + T);
+  coords_kernel<<<T, 128>>>(X, gs, gn, node, badd + T, T, kSeqGroup, V);
+  chol_qr(V, Gm, gs, gn, T, kSeqGroup, 1, 1e-8, badd + T);
+  chol_qr(V, Gm, gs, gn, T, kSeqGroup, 1, 1e-8, badd + T);
+  canonical_kernel<<<T, kSeqThreads>>>(X, gs, gn, T, vanish_tol, badd + T, V, dstatus);
+  basis_kernel<<<dim3(nt, (T + 7) / 8), 256>>>(X, V, gs, gn, T, U);
+  mhsa_kernel<<<T, 256, 2 * sizeof(double) * T>>>(lam, U, T, heads, coef, dp(o_va), dp(o_vb), dp(o_wo), d_spe, spe,
+                                                  dp(o_spe64));
   if (!ok(cudaGetLastError()) || !ok(cudaDeviceSynchronize())) goto done;
   if (!ok(cudaMemcpy(spe_host, spe, sizeof(float) * T * d_spe, cudaMemcpyDeviceToHost)) ||
-      !ok(cudaMemcpy(sweeps, dsweeps, sizeof(int), cudaMemcpyDeviceToHost)) ||
       !ok(cudaMemcpy(status_host, dstatus, sizeof(int), cudaMemcpyDeviceToHost)))
     goto done;
-  if (lam_host && !ok(cudaMemcpy(lam_host, lam, sizeof(double) * T, cudaMemcpyDeviceToHost))) goto done;
-  if (U_host && !ok(cudaMemcpy(U_host, Uc, TT, cudaMemcpyDeviceToHost))) goto done;
-  if (spe64_host && !ok(cudaMemcpy(spe64_host, spe64, sizeof(double) * T * d_spe, cudaMemcpyDeviceToHost))) goto done;
+  if (*status_host & 2) {
+    e = cudaErrorLaunchTimeout;
+    goto done;
+  }
+  if (lam_host && !ok(cudaMemcpy(lam_host, lam, T1, cudaMemcpyDeviceToHost))) goto done;
+  if (U_host && !ok(cudaMemcpy(U_host, U, TT, cudaMemcpyDeviceToHost))) goto done;
+  if (spe64_host && !ok(cudaMemcpy(spe64_host, dp(o_spe64), sizeof(double) * T * d_spe, cudaMemcpyDeviceToHost)))
+    goto done;
 done:
-  cudaFree(A), cudaFree(V), cudaFree(U), cudaFree(Uc), cudaFree(vbuf), cudaFree(dots), cudaFree(lam), cudaFree(cs);
-  cudaFree(acc), cudaFree(va), cudaFree(vb), cudaFree(wod), cudaFree(spe), cudaFree(spe64), cudaFree(dsweeps);
-  cudaFree(dstatus);
+  cudaFree(base);
   return e;
 }
 
