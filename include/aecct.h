@@ -214,6 +214,12 @@ int aecct_decode_host_noalloc(aecct_handle *h, const float *y_host, int64_t B, u
 int aecct_aap_ternarize(const float *w_dev, int32_t n_tensors, const int64_t *len_host, const float *delta_host,
                         float eps, uint8_t *packed_dev, float *scale_dev, float *wq_dev, void *cuda_stream);
 
+/* The same for tensors that lie apart: w_dev is a HOST array of n_tensors DEVICE pointers, tensor j at
+ * w_dev[j]; the codes and the weights still go out back to back. */
+int aecct_aap_ternarize_list(const float *const *w_dev, int32_t n_tensors, const int64_t *len_host,
+                             const float *delta_host, float eps, uint8_t *packed_dev, float *scale_dev, float *wq_dev,
+                             void *cuda_stream);
+
 /* The spectral positional encoding of Sec. 4.3 computed on the GPU, in double precision: the table
  * aecct_create takes as `spe`.  Tanner graph of H (variables 0..n-1, checks n..n+m-1, m = n - k,
  * T = n + m <= 1024 nodes), Laplacian L = D - A, its eigenpairs (lambda_i, phi_i) in ascending order

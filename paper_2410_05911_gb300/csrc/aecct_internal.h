@@ -264,7 +264,7 @@ constexpr int kStagedMaxKeys = 256;  // staged attention: keys per row (TMEM col
 
 // aap.cu: the AAP weight quantiser (eq. Ternary) and the GPU expansion of 2-bit weights
 constexpr int kTernarizeMaxTensors = 64;  // tensors per launch (the launcher splits larger calls)
-cudaError_t launch_aap_ternarize(const float *w, int n, const int64_t *len, const float *delta, float eps,
+cudaError_t launch_aap_ternarize(const float *const *w, int n, const int64_t *len, const float *delta, float eps,
                                  uint8_t *packed, float *scale, float *wq, cudaStream_t stream);
 cudaError_t launch_unpack_weights(const uint8_t *packed, int n_layers, int D, const ChunkDesc *chunks, int n_chunks,
                                   uint32_t layer_bytes, uint8_t *wstream, cudaStream_t stream);

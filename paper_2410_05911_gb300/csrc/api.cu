@@ -1143,19 +1143,34 @@ int aecct_spe_table(const uint8_t *H, int32_t n, int32_t k, int32_t d_spe, int32
   return AECCT_OK;
 }
 
-int aecct_aap_ternarize(const float *w_dev, int32_t n_tensors, const int64_t *len_host, const float *delta_host,
-                        float eps, uint8_t *packed_dev, float *scale_dev, float *wq_dev, void *cuda_stream) {
+int aecct_aap_ternarize_list(const float *const *w_dev, int32_t n_tensors, const int64_t *len_host,
+                             const float *delta_host, float eps, uint8_t *packed_dev, float *scale_dev, float *wq_dev,
+                             void *cuda_stream) {
   if (n_tensors < 0 || (n_tensors > 0 && (!w_dev || !len_host || !delta_host || !packed_dev || !scale_dev)))
     return AECCT_ERR_INVALID_ARG;
   if (!(eps > 0.0f) || !std::isfinite(eps)) return AECCT_ERR_INVALID_ARG;
   for (int j = 0; j < n_tensors; ++j) {
     if (len_host[j] < 4 || len_host[j] % 4 != 0 || len_host[j] > (int64_t(1) << 31)) return AECCT_ERR_INVALID_ARG;
     if (!(delta_host[j] > 0.0f) || !std::isfinite(delta_host[j])) return AECCT_ERR_INVALID_ARG;
+    if (!w_dev[j]) return AECCT_ERR_INVALID_ARG;
   }
   if (n_tensors == 0) return AECCT_OK;
   const cudaError_t e = launch_aap_ternarize(w_dev, n_tensors, len_host, delta_host, eps, packed_dev, scale_dev, wq_dev,
                                              static_cast<cudaStream_t>(cuda_stream));
   return e == cudaSuccess ? AECCT_OK : cuda_fail(e, "aap ternarize launch");
+}
+
+int aecct_aap_ternarize(const float *w_dev, int32_t n_tensors, const int64_t *len_host, const float *delta_host,
+                        float eps, uint8_t *packed_dev, float *scale_dev, float *wq_dev, void *cuda_stream) {
+  if (n_tensors < 0 || (n_tensors > 0 && (!w_dev || !len_host))) return AECCT_ERR_INVALID_ARG;
+  // the tensors back to back
+  std::vector<const float *> w(static_cast<size_t>(n_tensors));
+  for (int j = 0; j < n_tensors; ++j) {
+    if (len_host[j] < 4 || len_host[j] % 4 != 0 || len_host[j] > (int64_t(1) << 31)) return AECCT_ERR_INVALID_ARG;
+    w[j] = j == 0 ? w_dev : w[j - 1] + len_host[j - 1];
+  }
+  return aecct_aap_ternarize_list(w.data(), n_tensors, len_host, delta_host, eps, packed_dev, scale_dev, wq_dev,
+                                  cuda_stream);
 }
 
 int aecct_selftest_fma_rate(int32_t paired, double *fma_per_s) {
