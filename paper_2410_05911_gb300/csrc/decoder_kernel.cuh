@@ -1078,7 +1078,7 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
     }
     mbar_init(bar_op, kEpiWarps);
     mbar_init(bar_acc, 1);
-    mbar_init(bar_kvr, p.C);
+    mbar_init(bar_kvr, STAGED ? kEpiWarps * p.C : p.C);  // staged: every warp of every CTA
     mbar_init(bar_kvf, p.C);
     mbar_init(bar_zr, p.C);
     mbar_init(bar_zf, p.C);
@@ -1223,12 +1223,15 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
     };
     // after a CTA-wide barrier: this CTA no longer reads any CTA's K/V of this block (signalled by
     // thread `who`)
+    // The arrivals carry no data: the reads they follow are bulk copies that have landed (a thread saw
+    // their barrier complete before it got here), and nothing a peer writes afterwards can reach a
+    // read that has returned.  They are relaxed, because a release would wait for all of this thread's
+    // memory operations while the whole CTA waits for its warp at the O accumulators (2.1 k to 2.5 k
+    // cycles a block of LDPC(128,64) and LDPC(384,192)).
     auto kvf_signal = [&](int who) {
       if (p.C == 1) return;
-      if (tid == who) {
-        fence_acq_rel_cluster();
-        for (int c = 0; c < p.C; ++c) mbar_arrive_cluster(mapa_cluster(bar_kvf, c));
-      }
+      if (tid == who)
+        for (int c = 0; c < p.C; ++c) mbar_arrive_cluster_relaxed(mapa_cluster(bar_kvf, c));
       __syncwarp();
     };
     // accumulators of the last GEMM are complete once warp 0, which waited for them in its
@@ -1687,24 +1690,35 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
           // 330.8) and LDPC(384,192) 164.5 ms for 16,384 (146.9).  LDPC(128,64) at d = 64, whose rows
           // read keys through distributed shared memory before: 21.57 ms for 10,007 words (17.25).
           //
-          // this CTA's K and V rows, from region U to the cluster's scratch in global memory: 16 bulk
-          // copies (one per head and kind) by thread 0, complete before the cluster learns that they are
-          // there
+          // This warp's K and V (32 rows of two heads) go from region U to the cluster's scratch in global
+          // memory, four bulk copies by lane 0, once every CTA is past its reads of the last block's.  Their
+          // completion is counted on every CTA's barrier, which so also says that region U may be written:
+          // no CTA-wide barrier, and no warp waits but the one that fetches.  Against pushing all 16 slabs
+          // after a CTA barrier, with the relaxed signal below: LDPC(384,192) 146.8 -> 144.1 ms,
+          // LDPC(128,64) 330.4 -> 327.8 ms, at d = 64 17.2 -> 16.3 ms.
           constexpr uint32_t kRowBytes = 4u * DH;
           fence_proxy_async_smem();  // this thread's K / V stores, before the bulk copies read them
-          named_bar_sync(5, kEpiThreads);
-          if (tid == 0 && !*s_abort) {
-            const int R = p.C * kRows;
-            for (int ek = 0; ek < 2 * kHeads; ++ek)
-              bulk_s2g(p.kv_scratch + (static_cast<size_t>(cluster_id) * 2 * kHeads + ek) * R * DH +
-                           static_cast<size_t>(crank) * kRows * DH,
-                       kvl + static_cast<uint32_t>(ek) * kRows * kRowBytes, kRows * kRowBytes);
-            bulk_commit_group();
-            bulk_wait_group_0();
-            fence_proxy_async_global();
+          __syncwarp();
+          if (lane == 0) {
+            const uint32_t blk = blk_base + static_cast<uint32_t>(l);
+            if (p.C > 1 && blk > 0) wait_bar(ctl, bar_kvf, (blk - 1u) & 1u, true);
+            if (!*s_abort) {
+              const int R = p.C * kRows;
+#pragma unroll 1
+              for (int i = 0; i < 4; ++i) {
+                const int ek = 2 * (sl + 4 * (i >> 1)) + (i & 1);
+                bulk_s2g(p.kv_scratch + (static_cast<size_t>(cluster_id) * 2 * kHeads + ek) * R * DH +
+                             (static_cast<size_t>(crank) * kRows + 32 * qd) * DH,
+                         kvl + static_cast<uint32_t>(ek * kRows + 32 * qd) * kRowBytes, 32u * kRowBytes);
+              }
+              bulk_commit_group();
+              bulk_wait_group_0();
+              fence_proxy_async_global();
+            }
+            fence_acq_rel_cluster();
+            for (int c = 0; c < p.C; ++c) mbar_arrive_cluster(mapa_cluster(bar_kvr, c));
           }
-          cluster_arrive(bar_kvr);
-          cluster_wait(bar_kvr, kvr_ph);
+          __syncwarp();
           static_assert(L::kOffU == 0 && L::kOffAop == L::kRegionU && 16u * kRows * kRowBytes <= L::kRegionU &&
                             L::kRegionU + L::kAopBytes >= 4u * kStagedMaxRows * kRowBytes,
                         "two sets of K and V buffers span region U and the operand tile");
@@ -1726,21 +1740,38 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
               bulk_g2s(buf_of(e, kind), kvs + (static_cast<size_t>(e) * 2 + kind) * (p.C * kRows) * DH, fetch_bytes, bar);
             ++s_issued[6 + (e & 1)];
           };
-          if (tid == 0) fetch(0), fetch(1);
+          if (tid == 0) {
+            wait_bar(ctl, bar_kvr, kvr_ph, true);
+            fence_proxy_async_global();
+            fetch(0), fetch(1);
+          }
+          kvr_ph ^= 1u;
+          __syncwarp();
           // this lane's row (row ar of the quadrant: its Q, token and word come from lane ar) and part s
           const int ar = 8 * sl + (lane >> 2), s = lane & 3, r2 = 32 * qd + ar;
           const int t2 = __shfl_sync(0xffffffffu, t, ar), g2 = __shfl_sync(0xffffffffu, g, ar);
           const bool row2 = __shfl_sync(0xffffffffu, row_cw ? 1 : 0, ar) != 0;
+          const uint32_t info0 = row2 ? __ldg(p.mask_info[0] + t2) : 0u, info1 = row2 ? __ldg(p.mask_info[1] + t2) : 0u;
           const uint32_t word_off = row2 ? static_cast<uint32_t>(g2 * Tp) * kRowBytes : 0u;
           constexpr int VF = DH / 4;  // features of a lane
           float av[kHeads * VF];
+          int cnt = 0, nmax = 0;
+          const uint4 *lst = nullptr;
+          uint4 w[2];  // the first 16 list entries, kept over the heads of a ring where they are all
 #pragma unroll 1
           for (int e = 0; e < kHeads; ++e) {
-            const int mk = (e < p.h_first) ? 0 : 1;
-            const uint32_t info = row2 ? __ldg(p.mask_info[mk] + t2) : 0u;
-            const int cnt = static_cast<int>(info & 2047u);
-            const uint4 *lst = p.mask_list[mk] + (info >> 11);
-            const int nmax = __reduce_max_sync(0xffffffffu, cnt);
+            // the 16 list entries of block b (zeros past the row's list: the word's first row)
+            auto entries = [&](int b) {
+              w[0] = b < cnt ? __ldg(lst + (b >> 3)) : make_uint4(0u, 0u, 0u, 0u);
+              w[1] = b + 8 < cnt ? __ldg(lst + (b >> 3) + 1) : make_uint4(0u, 0u, 0u, 0u);
+            };
+            if (e == 0 || e == p.h_first) {
+              const uint32_t info = e < p.h_first ? info0 : info1;
+              cnt = static_cast<int>(info & 2047u);
+              lst = p.mask_list[e < p.h_first ? 0 : 1] + (info >> 11);
+              nmax = __reduce_max_sync(0xffffffffu, cnt);
+              entries(0);
+            }
             float q[DH];
             {
               float qa[DH], bq[DH];
@@ -1753,13 +1784,8 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
               for (int i = 0; i < DH; ++i) q[i] = __shfl_sync(0xffffffffu, q[i], ar);
             }
             const uint32_t kbuf = buf_of(e, 0) + word_off, vbuf = buf_of(e, 1) + word_off;
-            // the 16 list entries of block b (zeros past the row's list: the word's first row)
-            auto entries = [&](int b, uint4 *w) {
-              w[0] = b < cnt ? __ldg(lst + (b >> 3)) : make_uint4(0u, 0u, 0u, 0u);
-              w[1] = b + 8 < cnt ? __ldg(lst + (b >> 3) + 1) : make_uint4(0u, 0u, 0u, 0u);
-            };
             // sigma of this lane's keys b + 4 i + s, -inf past the row's list
-            auto score4 = [&](int b, const uint4 *w, float *sg) {
+            auto score4 = [&](int b, float *sg) {
 #pragma unroll
               for (int i = 0; i < 4; ++i) {
                 if (b + 4 * i < nmax) {
@@ -1785,7 +1811,7 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
             for (int f = 0; f < VF; ++f) num[f] = 0.0f;
             // the exponentials of this lane's four scores, then l = sum p and num = sum p v over the block's
             // keys in ascending order: key 4 i + u has its p in lane part u
-            auto fold16 = [&](int b, const uint4 *w, const float *sg) {
+            auto fold16 = [&](int b, const float *sg) {
               const float2 p01 = exp2_series2(add2(make_float2(sg[0], sg[1]), make_float2(-mx, -mx)));
               const float2 p23 = exp2_series2(add2(make_float2(sg[2], sg[3]), make_float2(-mx, -mx)));
               const float pr[4] = {p01.x, p01.y, p23.x, p23.y};
@@ -1821,25 +1847,23 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
               mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
               mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
             };
-            uint4 w[2];
             float sg[4];
-            entries(0, w);
             // this head's rows have landed
             if (lane == 0) wait_bar(ctl, bar_skv + ((e & 1) ? 8u : 0u), static_cast<uint32_t>((e >> 1) & 1), false);
             __syncwarp();
             if (nmax <= 16) {  // the lists of this warp's rows are one block each: scores stay in registers
-              score4(0, w, sg);
+              score4(0, sg);
               mx = fmaxf(fmaxf(sg[0], sg[1]), fmaxf(sg[2], sg[3]));
               row_max4();
-              fold16(0, w, sg);
+              fold16(0, sg);
             } else {
               // the scores in this thread's own TMEM lane, 4 columns a block from column kSc + 64 sl (at most
               // 256 keys), in columns whose accumulators are dead (d = 128) or that hold none (d = 64)
               const uint32_t tsc = tl + L::kRowCacheCol + 64u * static_cast<uint32_t>(sl);
 #pragma unroll 1
               for (int b = 0; b < nmax; b += 16) {
-                entries(b, w);
-                score4(b, w, sg);
+                entries(b);
+                score4(b, sg);
                 mx = fmaxf(mx, fmaxf(fmaxf(sg[0], sg[1]), fmaxf(sg[2], sg[3])));
                 tmem_st4(tsc + (b >> 2), sg[0], sg[1], sg[2], sg[3]);
               }
@@ -1847,10 +1871,10 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
               row_max4();
 #pragma unroll 1
               for (int b = 0; b < nmax; b += 16) {
-                entries(b, w);
+                entries(b);
                 tmem_ld<4>(tsc + (b >> 2), sg);
                 tmem_wait_ld();
-                fold16(b, w, sg);
+                fold16(b, sg);
               }
             }
             const float inv = __fdiv_rn(1.0f, lsum);
@@ -1988,7 +2012,7 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
           };
           if constexpr (LIN == 1) {
             // peers have finished reading this CTA's K/V: the shared region may now take u
-            if constexpr (!TASKS) cluster_wait(bar_kvf, kvf_ph);
+            if constexpr (ATT == 0) cluster_wait(bar_kvf, kvf_ph);
 #pragma unroll
             for (int ch = 0; ch < NCH; ++ch) {
               wait_chunk(ch);
@@ -2021,8 +2045,7 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
             alpha_in = a;
             const float rr = __fdiv_rn(127.0f, a);
             // peers have finished reading this CTA's K/V: the shared region may now take u codes
-            // (d <= 64; at d = 128 the staged attention's scratch is free for the next block's K/V)
-            if constexpr (!TASKS) cluster_wait(bar_kvf, kvf_ph);
+            if constexpr (ATT == 0) cluster_wait(bar_kvf, kvf_ph);
 #pragma unroll
             for (int ch = 0; ch < NCH; ++ch) {
               const int c0 = sl * D + 32 * ch;
