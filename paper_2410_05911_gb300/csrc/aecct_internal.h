@@ -212,7 +212,7 @@ __host__ __device__ constexpr inline uint32_t kv_piece(int dh, uint32_t off) {
 // operand.  Row mode, and task mode at d = 128: per token row 8 heads x (K | V) x d_h fp32 (Q and
 // the attention output stay in TMEM).  Task mode at d <= 64: 8 heads x (Q | K | V) x d_h fp32;
 // the attention output of a (row, head) then replaces its Q.
-template <int D, bool TASKS = false>
+template <int D, bool TASKS = false, int CTAS = 1>
 struct SmemLayout {
   static constexpr bool kQInSmem = TASKS && D != 128;
   static constexpr uint32_t kSlot = (kQInSmem ? 12u : 8u) * (D / 8u);  // bytes of one head of one row
@@ -242,16 +242,26 @@ struct SmemLayout {
   // around the parked residual, d = 32 [128, 512).  Row mode: kRowCache columns per column slice
   // from kRowCacheCol, each thread in its own row's lane (d = 128: [128, 384); d <= 64:
   // [256, 512)).
-  static constexpr uint32_t kTmemCols = 512u;
-  static constexpr int kTaskCache = D == 128 ? 64 : 96;
+  // Two CTAs per SM (d = 32 tasks) have half the columns each: 48 keys a warp in [0, 96), around the
+  // parked residual, and [128, 224).
+  static constexpr int kCtasPerSm = CTAS;
+  static_assert(CTAS == 1 || (D == 32 && TASKS), "two CTAs per SM: d = 32 tasks");
+  static constexpr uint32_t kTmemCols = 512u / CTAS;
+  static constexpr int kTaskCache = D == 128 ? 64 : CTAS == 1 ? 96 : 48;
   __host__ __device__ static constexpr uint32_t task_cache_col(uint32_t slice) {
-    return D == 128 ? 128u + 64u * slice : D == 32 ? 128u + 96u * slice : slice < 2u ? 96u * slice : 64u + 96u * slice;
+    return D == 128 ? 128u + 64u * slice
+           : CTAS == 2 ? (slice < 2u ? 48u * slice : 32u + 48u * slice)
+           : D == 32 ? 128u + 96u * slice : slice < 2u ? 96u * slice : 64u + 96u * slice;
   }
   static constexpr uint32_t kRowCacheCol = (D == 128) ? 128u : 256u;
 };
 
+// the shared and tensor memory of the kernel with attention path ATT
+template <int D, int ATT>
+using KernelLayout = SmemLayout<D, ATT == 1 || ATT == 3, ATT == 3 ? 2 : 1>;
+
 // decoder_kernel.cuh.  ATT: 0 = per-row neighbour lists, 1 = warp tasks, 2 = per-row lists over
-// per-head staged rows (d >= 64); ACT: 0 = ReLU, 1 = GELU; LIN: 0 = AAP linears, 1 = full-precision
+// per-head staged rows (d >= 64), 3 = warp tasks at two CTAs per SM (d = 32); ACT: 0 = ReLU, 1 = GELU; LIN: 0 = AAP linears, 1 = full-precision
 // (bf16) linears.  Instantiated in decoder_kernel.cu (0, 0), decoder_kernel_gelu.cu (1, 0),
 // decoder_kernel_fp.cu (0, 1) and decoder_kernel_fp_gelu.cu (1, 1).
 template <int D, int ATT, int ACT, int LIN>

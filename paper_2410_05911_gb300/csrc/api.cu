@@ -34,6 +34,7 @@ struct aecct_handle {
   int Tp = 0;  // token rows per codeword (T, or T plus padding rows)
   int C = 1, G = 1, max_clusters = 0;
   int att = 0;  // kernel attention path: 0 per-row lists, 1 warp tasks, 2 per-row lists over staged rows
+  bool two_per_sm = false;  // d = 32 tasks: batches of more groups than SMs run two CTAs on each
   int alpha_mode = 0;  // 1 = one alpha per quantised matrix of a word
   int activation = 0;   // 0 = ReLU, 1 = GELU
   int linear_mode = 0;  // 0 = AAP ternary linears, 1 = full-precision (bf16) linears
@@ -277,6 +278,7 @@ cudaError_t prepare_any(int D, int att, int C, uint32_t pb, int *max_clusters) {
     return D == 32   ? prepare_decode_kernel<32, 1, ACT, LIN>(C, pb, max_clusters)
            : D == 64 ? prepare_decode_kernel<64, 1, ACT, LIN>(C, pb, max_clusters)
                      : prepare_decode_kernel<128, 1, ACT, LIN>(C, pb, max_clusters);
+  if (att == 3) return prepare_decode_kernel<32, 3, ACT, LIN>(C, pb, max_clusters);  // d = 32 only
   if (att == 2)
     return D == 64 ? prepare_decode_kernel<64, 2, ACT, LIN>(C, pb, max_clusters)
                    : prepare_decode_kernel<128, 2, ACT, LIN>(C, pb, max_clusters);
@@ -290,6 +292,7 @@ cudaError_t launch_any(int D, int att, const DecodeParams &p, cudaStream_t strea
     return D == 32   ? launch_decode<32, 1, ACT, LIN>(p, stream)
            : D == 64 ? launch_decode<64, 1, ACT, LIN>(p, stream)
                      : launch_decode<128, 1, ACT, LIN>(p, stream);
+  if (att == 3) return launch_decode<32, 3, ACT, LIN>(p, stream);
   if (att == 2) return D == 64 ? launch_decode<64, 2, ACT, LIN>(p, stream) : launch_decode<128, 2, ACT, LIN>(p, stream);
   if (D == 32) return launch_decode<32, 0, ACT, LIN>(p, stream);
   if (D == 64) return launch_decode<64, 0, ACT, LIN>(p, stream);
@@ -502,12 +505,20 @@ int aecct_create(const aecct_model_desc *desc, aecct_handle **out) {
     g_last_error = "no cluster of this size fits on the device";
     return AECCT_ERR_UNSUPPORTED;
   }
+  // d = 32 tasks: also the kernel that fits twice on an SM (decode_params)
+  const bool two_per_sm = D == 32 && att == 1;
+  if (two_per_sm) {
+    int mc = 0;
+    e = prepare_variant(d.activation, d.linear_mode, D, 3, 1, plan_bound, &mc);
+    if (e != cudaSuccess) return cuda_fail(e, "kernel occupancy");
+  }
 
   aecct_handle *h = new aecct_handle();
   h->n = n, h->k = k, h->T = T, h->m = m, h->d = D, h->n_layers = d.n_layers, h->h_first = d.h_first;
   h->Tp = (tasks && D == 128) ? Tp128 : T;
   h->d_spe = d.d_spe, h->C = best_C, h->G = best_G, h->max_clusters = max_clusters, h->att = att;
   h->ln_eps = d.ln_eps, h->alpha_floor = d.alpha_floor, h->b_d1 = d.b_d1, h->device = dev;
+  h->two_per_sm = two_per_sm;
   h->alpha_mode = d.alpha_mode;
   h->activation = d.activation;
   h->linear_mode = d.linear_mode;
@@ -866,6 +877,19 @@ int aecct_create(const aecct_model_desc *desc, aecct_handle **out) {
   return AECCT_OK;
 }
 
+// Clusters of a full launch.  d = 32 tasks: two CTAs on every SM, which hide each other's barriers and
+// latencies (BCH(31,16): 1,024 words 121 -> 100 us, 65,536 words 5.66 -> 4.77 ms).  (The occupancy query
+// answers one CTA per SM for any kernel that allocates tensor memory; the two fit in registers, shared
+// and tensor memory, and the decode does not depend on how many are resident.)
+static int64_t resident_clusters(const aecct_handle *h) { return h->two_per_sm ? 2 * h->max_clusters : h->max_clusters; }
+
+// The attention path of a launch: two CTAs per SM only where there are more groups than SMs.  With fewer
+// a CTA has its SM to itself, and the kernel with twice the registers is faster (one word: 40.0 against
+// 41.7 us).
+static int launch_att(const aecct_handle *h, const DecodeParams &p) {
+  return h->two_per_sm && p.n_clusters > h->max_clusters ? 3 : h->att;
+}
+
 // the kernel arguments of one decode call: the handle's model and plan, this call's buffers
 static DecodeParams decode_params(const aecct_handle *h, int64_t B, const float *y_dev, uint8_t *bits_dev,
                                   uint8_t *syn_dev, float *logits_dev, int *err_dev) {
@@ -875,7 +899,8 @@ static DecodeParams decode_params(const aecct_handle *h, int64_t B, const float 
   p.d_spe = h->d_spe, p.C = h->C, p.G = h->G;
   p.B = B;
   p.n_groups = (B + h->G - 1) / h->G;
-  p.n_clusters = static_cast<int>(p.n_groups < h->max_clusters ? p.n_groups : h->max_clusters);
+  const int64_t most = resident_clusters(h);
+  p.n_clusters = static_cast<int>(p.n_groups < most ? p.n_groups : most);
   p.y = y_dev, p.bits = bits_dev, p.syn = syn_dev, p.logits = logits_dev;
   p.wstream = h->wstream, p.layer_bytes = h->layer_bytes;
   p.lparams = h->lparams, p.xtab = reinterpret_cast<const float4 *>(h->xtab), p.w_d1 = h->w_d1, p.b_d1 = h->b_d1;
@@ -938,7 +963,7 @@ int aecct_decode(aecct_handle *h, const float *y_dev, int64_t B, uint8_t *bits_d
   if (prev != AECCT_OK) return prev;
   const DecodeParams p = decode_params(h, B, y_dev, bits_dev, syndrome_dev, logits_dev, h->d_err);
   cudaError_t e;
-  e = launch_variant(h->activation, h->linear_mode, h->d, h->att, p, stream);
+  e = launch_variant(h->activation, h->linear_mode, h->d, launch_att(h, p), p, stream);
   if (e != cudaSuccess) return cuda_fail(e, "decode launch");
   if ((e = cudaMemcpyAsync(h->h_err, h->d_err, sizeof(int), cudaMemcpyDeviceToHost, stream)) != cudaSuccess)
     return cuda_fail(e, "status copy");
@@ -1051,7 +1076,7 @@ int aecct_decode_host_noalloc(aecct_handle *h, const float *y_host, int64_t B, u
   if ((e = cudaMemcpyAsync(y_dev, y_host, sizeof(float) * b * n, cudaMemcpyHostToDevice, stream)) != cudaSuccess)
     return cuda_fail(e, "copy y");
   const DecodeParams p = decode_params(h, B, y_dev, bits_dev, syn_dev, logits_dev, err);
-  e = launch_variant(h->activation, h->linear_mode, h->d, h->att, p, stream);
+  e = launch_variant(h->activation, h->linear_mode, h->d, launch_att(h, p), p, stream);
   if (e != cudaSuccess) return cuda_fail(e, "decode launch");
   if ((e = cudaMemcpyAsync(bits_host, bits_dev, b * n, cudaMemcpyDeviceToHost, stream)) != cudaSuccess)
     return cuda_fail(e, "copy bits");
@@ -1087,7 +1112,7 @@ int aecct_query(const aecct_handle *h, int32_t *cluster_ctas, int32_t *words_per
   if (!h) return AECCT_ERR_INVALID_ARG;
   if (cluster_ctas) *cluster_ctas = h->C;
   if (words_per_group) *words_per_group = h->G;
-  if (max_clusters) *max_clusters = h->max_clusters;
+  if (max_clusters) *max_clusters = static_cast<int32_t>(resident_clusters(h));
   if (threads_per_cta) *threads_per_cta = kThreads;
   int sm;
   const bool tasks = h->att == 1;

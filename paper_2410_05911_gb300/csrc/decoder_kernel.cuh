@@ -667,7 +667,7 @@ struct BlockCtx {
 
 template <int D, int ATT>
 struct Issuer {
-  using L = SmemLayout<D, ATT == 1>;
+  using L = KernelLayout<D, ATT>;
   using W = WeightSchedule<D>;
   static constexpr int S = W::kStages;
   static constexpr int CPL = W::kCPL;
@@ -799,7 +799,7 @@ struct Issuer {
 template <int ATT>
 struct Issuer<128, ATT> {
   static constexpr int D = 128;
-  using L = SmemLayout<D, ATT == 1>;
+  using L = KernelLayout<D, ATT>;
   using W = WeightSchedule<D>;
   static constexpr uint32_t kChunk = W::kStageBytes;
   static_assert(W::kCPL == 24 && W::kStages == 3 && kChunk == 16384, "d = 128 schedule");
@@ -1033,11 +1033,12 @@ struct Issuer<128, ATT> {
 // the kernel
 // ------------------------------------------------------------------------------------------
 template <int D, int ATT, int ACT, int LIN>
-__global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid_constant__ DecodeParams p) {
-  // ATT: 0 = per-row neighbour lists, 1 = warp tasks, 2 = per-row lists over per-head staged rows
-  constexpr bool TASKS = ATT == 1, STAGED = ATT == 2;
+__global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) aecct_decoder_kernel(const __grid_constant__ DecodeParams p) {
+  // ATT: 0 = per-row neighbour lists, 1 = warp tasks, 2 = per-row lists over per-head staged rows, 3 = warp
+  // tasks at two CTAs per SM (d = 32)
+  constexpr bool TASKS = ATT == 1 || ATT == 3, STAGED = ATT == 2;
   static_assert(!STAGED || D == 64 || D == 128, "staged attention is built for d = 64 and 128");
-  using L = SmemLayout<D, TASKS>;
+  using L = KernelLayout<D, ATT>;
   using LP = LayerParamLayout;
   constexpr int DH = D / kHeads;  // head width
   constexpr int XS = D / 4;       // x columns per thread
@@ -1964,13 +1965,14 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
         // ---------------- S7: FFN1 + ReLU (Sec. 4 item 4) or GELU, Quant(u) -> FFN2 operand
         {
           const float f1 = dq_factor(sw + 4);
-          constexpr int NCH = D / 32;
-          // accumulator column of this thread's chunk ch of 32 hidden units (units sl D + 32 ch +
-          // [0, 32)).  d = 128 (ffn1_unit_of_column): chunks 0 and 1 in [64 sl, 64 sl + 64), done
+          constexpr int CH = ATT == 3 ? 16 : 32;  // hidden units of a chunk (64 registers at two CTAs per SM)
+          constexpr int NCH = D / CH;
+          // accumulator column of this thread's chunk ch of CH hidden units (units sl D + CH ch +
+          // [0, CH)).  d = 128 (ffn1_unit_of_column): chunks 0 and 1 in [64 sl, 64 sl + 64), done
           // with FFN1's first N-tile pair, chunks 2 and 3 in [256 + 64 sl, 256 + 64 sl + 64).
           auto acc_col = [&](int ch) -> int {
             if constexpr (D == 128) return ch < 2 ? 64 * sl + 32 * ch : 256 + 64 * sl + 32 * (ch - 2);
-            else return sl * D + 32 * ch;
+            else return sl * D + CH * ch;
           };
           // before chunk ch.  d = 128: chunks 0 and 1 wait for the first half of FFN1's MMAs, 2 and 3
           // for all of them (the block's third accumulator phase); then warp 0 stages FFN2's
@@ -1988,20 +1990,20 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
               if (ch == 0) wait_acc();
             }
           };
-          // ACT 0 = ReLU, 1 = GELU.  u = act(acc f1 + b1) in 32-column chunks of this thread's D
+          // ACT 0 = ReLU, 1 = GELU.  u = act(acc f1 + b1) in CH-column chunks of this thread's D
           // hidden units.  AAP: u is stored over its own accumulators in TMEM (this thread's lane
           // and columns) between the row maximum and the codes, which leaves the registers to the
           // rest of the kernel.  Full-precision linears: one pass, u rounded to bf16.
           auto hidden = [&](int ch, float *u, bool capture) {
-            const int c0 = sl * D + 32 * ch;
-            float ac[32], bb[32];
-            tmem_ld<32>(tl + acc_col(ch), ac);
+            const int c0 = sl * D + CH * ch;
+            float ac[CH], bb[CH];
+            tmem_ld<CH>(tl + acc_col(ch), ac);
             tmem_wait_ld();
-            if (capture) capture_acc(l, 2, ac, c0, 32);
-            ldg_vec<32>(lp + LP::b1(D) + c0, bb);
-            dequant<32>(ac, f1, bb, u);
+            if (capture) capture_acc(l, 2, ac, c0, CH);
+            ldg_vec<CH>(lp + LP::b1(D) + c0, bb);
+            dequant<CH>(ac, f1, bb, u);
 #pragma unroll
-            for (int j = 0; j < 32; ++j) u[j] = ACT == 0 ? (u[j] > 0.0f ? u[j] : 0.0f) : gelu_as(u[j]);
+            for (int j = 0; j < CH; ++j) u[j] = ACT == 0 ? (u[j] > 0.0f ? u[j] : 0.0f) : gelu_as(u[j]);
           };
           // d = 128: FFN2's operand goes to TMEM, the 32 values of chunk ch packed two to a column
           // into the 16 columns [64 sl + 16 ch, 64 sl + 16 ch + 16) of this thread's lane (hidden
@@ -2016,7 +2018,7 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
 #pragma unroll
             for (int ch = 0; ch < NCH; ++ch) {
               wait_chunk(ch);
-              float u[32];
+              float u[CH];
               hidden(ch, u, cap);
               if constexpr (D == 128) {
                 uint32_t w[16];
@@ -2024,7 +2026,7 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
                 for (int i = 0; i < 16; ++i) w[i] = pack_bf16x2_rn(u[2 * i], u[2 * i + 1]);
                 put_operand(ch, w);
               } else {
-                store_bf16<32>(uqt, r, sl * D + 32 * ch, 4 * D, u);
+                store_bf16<CH>(uqt, r, sl * D + CH * ch, 4 * D, u);
               }
             }
             if constexpr (D == 128) tmem_wait_st();
@@ -2033,11 +2035,11 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
 #pragma unroll
             for (int ch = 0; ch < NCH; ++ch) {
               wait_chunk(ch);
-              float u[32];
+              float u[CH];
               hidden(ch, u, cap);
 #pragma unroll
-              for (int j = 0; j < 32; ++j) umax = fmaxf(umax, fabsf(u[j]));
-              tmem_st<32>(tl + acc_col(ch), u);
+              for (int j = 0; j < CH; ++j) umax = fmaxf(umax, fabsf(u[j]));
+              tmem_st<CH>(tl + acc_col(ch), u);
             }
             tmem_wait_st();
             float a = word_alpha(row_max(umax));
@@ -2048,21 +2050,21 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
             if constexpr (ATT == 0) cluster_wait(bar_kvf, kvf_ph);
 #pragma unroll
             for (int ch = 0; ch < NCH; ++ch) {
-              const int c0 = sl * D + 32 * ch;
-              float u[32];
-              tmem_ld<32>(tl + acc_col(ch), u);
+              const int c0 = sl * D + CH * ch;
+              float u[CH];
+              tmem_ld<CH>(tl + acc_col(ch), u);
               tmem_wait_ld();
-              float qv[32];
-              codes<32>(u, rr, qv);
+              float qv[CH];
+              codes<CH>(u, rr, qv);
               if constexpr (D == 128) {
                 uint32_t w[16];
 #pragma unroll
                 for (int i = 0; i < 16; ++i) w[i] = pack_bf16x2(qv[2 * i], qv[2 * i + 1]);
                 put_operand(ch, w);
               } else {
-                store_codes<32>(uqt, r, c0, 4 * D, qv);
+                store_codes<CH>(uqt, r, c0, 4 * D, qv);
               }
-              if (cap) capture_q(l, 3, qv, c0, 32, alpha_in);
+              if (cap) capture_q(l, 3, qv, c0, CH, alpha_in);
             }
             if constexpr (D == 128) tmem_wait_st();
           }
@@ -2193,19 +2195,19 @@ __global__ void __launch_bounds__(kThreads, 1) aecct_decoder_kernel(const __grid
 
 template <int D, int ATT, int ACT, int LIN>
 cudaError_t prepare_decode_kernel(int cluster_ctas, uint32_t plan_bytes, int *max_active_clusters) {
-  using L = SmemLayout<D, ATT == 1>;
+  using L = KernelLayout<D, ATT>;
   const uint32_t total = L::kTotal + plan_bytes;
   cudaError_t e = cudaFuncSetAttribute(aecct_decoder_kernel<D, ATT, ACT, LIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(total));
   if (e != cudaSuccess) return e;
-  // ask for the smallest shared-memory carve-out that holds one CTA (1 KB of it is reserved by
-  // the system): the rest of the 256 KB unified array stays L1 for spills and parameter loads
+  // ask for the smallest shared-memory carve-out that holds the SM's CTAs (1 KB for each is
+  // reserved by the system): the rest of the 256 KB unified array stays L1 for spills and parameter loads
   int dev = 0, smem_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess)
     return e;
   if (smem_sm > 0) {
-    const int pct = static_cast<int>((100ll * (total + 1024) + smem_sm - 1) / smem_sm);
+    const int pct = static_cast<int>((100ll * L::kCtasPerSm * (total + 1024) + smem_sm - 1) / smem_sm);
     e = cudaFuncSetAttribute(aecct_decoder_kernel<D, ATT, ACT, LIN>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              pct > 100 ? 100 : pct);
     if (e != cudaSuccess) return e;
@@ -2226,7 +2228,7 @@ cudaError_t prepare_decode_kernel(int cluster_ctas, uint32_t plan_bytes, int *ma
 
 template <int D, int ATT, int ACT, int LIN>
 cudaError_t launch_decode(const DecodeParams &p, cudaStream_t stream) {
-  using L = SmemLayout<D, ATT == 1>;
+  using L = KernelLayout<D, ATT>;
   cudaLaunchConfig_t cfg = {};
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;

@@ -116,3 +116,36 @@ def test_staged_attention_takes_what_the_buffers_hold():
         dec.close()
     st, h = A.create_handle(I.random_model(I.make_code("ldpc128_64"), 64, 1, seed=1), attention_mode=3)
     assert st == A.AECCT_ERR_UNSUPPORTED and h is None
+
+
+# d = 32: more groups than SMs run two CTAs on each SM, with half the score cache (48 keys)
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,m,weight,variant", [(31, 15, 3, "relu"), (16, 14, 2, "alpha"), (33, 15, 3, "gelu"),
+                                                (34, 15, 4, "full"), (64, 32, 4, "relu"), (110, 18, 3, "relu")])
+def test_two_ctas_per_sm_equal_one(n, m, weight, variant):
+    model = I.random_model(random_code(n, m, weight, n), 32, 2, seed=n, spe_noise=True,
+                           activation=1 if variant == "gelu" else 0, full_precision=variant == "full")
+    model.alpha_mode = 1 if variant == "alpha" else 0
+    dec = A.Decoder(model)
+    q = dec.query()
+    assert q["attention_mode"] == 2
+    B = q["words_per_group"] * (q["max_clusters"] + q["max_clusters"] // 2) + 1  # some CTAs take a second group
+    rng = np.random.Generator(np.random.PCG64(n))
+    y = torch.from_numpy(rng.standard_normal((B, n)).astype(np.float32)).cuda()
+    cap = {k: v for k, v in dec.set_capture(3).items()}
+    many = [t.clone() for t in dec.decode(y)]
+    torch.cuda.synchronize()
+    first = {k: v.clone() for k, v in cap.items()}
+    # the same words a few at a time: one CTA per SM
+    step = 100 * q["words_per_group"]
+    few = [[t.clone() for t in dec.decode(y[s:s + step].contiguous())] for s in range(0, B, step)]
+    torch.cuda.synchronize()
+    assert dec.synchronize() == A.AECCT_OK
+    for i in range(3):
+        got = torch.cat([f[i] for f in few])
+        assert torch.equal(many[i].view(torch.uint8), got.view(torch.uint8))
+    again = dec.set_capture(3)
+    dec.decode(y[:3].contiguous())
+    torch.cuda.synchronize()
+    assert all(torch.equal(first[k].view(torch.uint8), again[k].view(torch.uint8)) for k in first)
+    dec.close()
