@@ -28,12 +28,13 @@
 //                     row (maximum, then the sums).
 //
 // The long code of 576 nodes (LDPC(384,192)), where Jacobi rotations (about 10 sweeps of 575 steps with
-// three grid-wide barriers each) and Gram-Schmidt in node coordinates took 327 ms: tridiagonal form 4.9 ms,
-// eigenvalues 1.2, inverse iteration 0.8, the clusters' bases 2.3, reflections 1.4, canonical basis 3.9.
-#include <cuda_runtime.h>
-
+// three grid-wide barriers each) and Gram-Schmidt in node coordinates took 327 ms: tridiagonal form 3.9 ms,
+// eigenvalues 0.9, inverse iteration 0.8, the clusters' bases 2.2, reflections 1.4, canonical basis 2.6;
+// the attention 3.8 (41 with double operations).
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 #include <vector>
 
 #include "aecct_internal.h"
@@ -42,7 +43,7 @@ namespace aecct {
 
 namespace {
 
-constexpr int kTriThreads = 256;
+constexpr int kTriThreads = 128;
 constexpr int kInvitIters = 3;
 constexpr int kSeqGroup = 24;         // clusters up to this size: Gram-Schmidt by one CTA
 constexpr double kEps = 2.220446049250313e-16;
@@ -58,12 +59,16 @@ __device__ double block_sum(double v, double *red) {
   return s;
 }
 
-// the sum of one double per thread of a 256-thread CTA, through one of two buffers in turn (one barrier)
-__device__ __forceinline__ double block_sum8(double v, double *red) {
+// The sums of a 128-thread CTA: every warp's part, then all of them (after a barrier).  A warp's double
+// operation occupies its scheduler's pipe for 64 cycles, so there is one warp to a scheduler, and scalar work
+// is done by one warp and handed on through shared memory.
+__device__ __forceinline__ void warp_part(double v, double *red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-  __syncthreads();
-  return ((red[0] + red[1]) + (red[2] + red[3])) + ((red[4] + red[5]) + (red[6] + red[7]));
+}
+__device__ __forceinline__ double all_parts(const double *red) {
+  static_assert(kTriThreads == 128, "four parts");
+  return (red[0] + red[1]) + (red[2] + red[3]);
 }
 
 // Barrier of a cooperative launch: every CTA adds one to `count` and thread 0 waits until it reaches
@@ -96,7 +101,7 @@ __global__ void __launch_bounds__(kTriThreads) tridiag_kernel(const uint8_t *__r
                                                              double *tau, double *d, double *e, double *rowbuf,
                                                              double *pbuf, unsigned *count, int *status) {
   extern __shared__ double sh[];
-  __shared__ double red[2][kTriThreads / 32], s_col[2];
+  __shared__ double red[2][kTriThreads / 32], s_col[2], s_scal[4];
   const int T = n + m, G = gridDim.x, b = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   double *v = sh, *w = sh + T, *vn = sh + 2 * T, *rows = sh + 3 * T;
   const int R = (T + G - 1) / G;
@@ -132,15 +137,25 @@ __global__ void __launch_bounds__(kTriThreads) tridiag_kernel(const uint8_t *__r
       if (j <= k + 1) s_col[j - k] = c;
       else s = fma(c, c, s);
     }
-    s = block_sum8(s, red[0]);
-    const double dk = s_col[0], alpha = s_col[1];
-    double beta = alpha, tk = 0.0, sc = 0.0;
-    if (s > 0.0) {
-      beta = -copysign(sqrt(fma(alpha, alpha, s)), alpha);
-      tk = (beta - alpha) / beta;
-      sc = 1.0 / (alpha - beta);
+    warp_part(s, red[0]);
+    __syncthreads();
+    if (warp == 0) {
+      const double ss = all_parts(red[0]), alpha = s_col[1];
+      double beta = alpha, tk = 0.0, sc = 0.0;
+      if (ss > 0.0) {
+        // tau = (beta - alpha) / beta and 1 / (alpha - beta) with one division
+        beta = -copysign(sqrt(fma(alpha, alpha, ss)), alpha);
+        const double diff = alpha - beta, inv = 1.0 / (beta * diff);
+        tk = -diff * diff * inv;
+        sc = beta * inv;
+      }
+      if (lane == 0) {
+        s_scal[0] = tk, s_scal[1] = sc;
+        if (b == 0) d[k] = s_col[0], e[k] = beta, tau[k] = tk;
+      }
     }
-    if (b == 0 && tid == 0) d[k] = dk, e[k] = beta, tau[k] = tk;
+    __syncthreads();
+    const double tk = s_scal[0], sc = s_scal[1];
     for (int j = k + tid; j < T; j += kTriThreads)
       if (j > k) vn[j] = j == k + 1 ? 1.0 : vn[j] * sc;
     __syncthreads();
@@ -172,8 +187,11 @@ __global__ void __launch_bounds__(kTriThreads) tridiag_kernel(const uint8_t *__r
       v[j] = vn[j];
       s = fma(pj, vn[j], s);
     }
-    s = block_sum8(s, red[1]);
-    const double kk = -0.5 * tk * s;
+    warp_part(s, red[1]);
+    __syncthreads();
+    if (tid == 0) s_scal[2] = -0.5 * tk * all_parts(red[1]);
+    __syncthreads();
+    const double kk = s_scal[2];
     for (int j = k + 1 + tid; j < T; j += kTriThreads) {
       w[j] = fma(kk, vn[j], w[j]);
       if (b == k % G) Vh[static_cast<size_t>(k) * T + j] = vn[j];
@@ -195,16 +213,18 @@ __global__ void __launch_bounds__(kTriThreads) tridiag_kernel(const uint8_t *__r
     d[T - 1] = fma(-2.0 * v[T - 1], w[T - 1], rows[static_cast<size_t>((T - 1) / G) * T + T - 1]);
 }
 
-// Eigenvalue i (ascending) by bisection into 17 parts a round, 16 lanes an eigenvalue (2 to a warp): the
-// number of eigenvalues below x is the number of sign changes in the Sturm sequence
+// Eigenvalue i (ascending) by bisection into 33 parts a round, a warp an eigenvalue: the number of
+// eigenvalues below x is the number of sign changes in the Sturm sequence
 // p_i = (d_i - x) p_{i-1} - e_{i-1}^2 p_{i-2} (a zero counts as the sign opposite to its predecessor's),
 // rescaled by a power of two every 8 steps.  The recurrence without divisions takes three double
-// operations a step.  e^2 is kept above (1e-18 |L|)^2, far below rounding, so that a split matrix
-// does not end the sequence in zeros.
+// operations a step; a warp's double operation occupies its scheduler's pipe for 64 cycles whatever its
+// lanes do, so more parts a round on more warps (up to four to an SM) mean fewer rounds for nothing.
+// e^2 is kept above (1e-18 |L|)^2, far below rounding, so that a split matrix does not end the sequence in
+// zeros.
 __global__ void __launch_bounds__(32) bisect_kernel(const double *__restrict__ d, const double *__restrict__ e, int T,
                                                    double *lam) {
   extern __shared__ double2 de[];  // d_i and e_{i-1}^2
-  const int lane = threadIdx.x, i = blockIdx.x * 2 + (lane >> 4), sub = lane & 15;
+  const int lane = threadIdx.x, i = blockIdx.x;
   double lo = INFINITY, hi = -INFINITY;
   for (int j = lane; j < T; j += 32) {
     const double r = (j > 0 ? fabs(e[j - 1]) : 0.0) + (j + 1 < T ? fabs(e[j]) : 0.0);
@@ -219,8 +239,8 @@ __global__ void __launch_bounds__(32) bisect_kernel(const double *__restrict__ d
     de[j] = make_double2(d[j], j > 0 ? fmax(e[j - 1] * e[j - 1], 1e-36 * nt * nt) : 0.0);
   __syncwarp();
   lo -= 8.0 * kEps * nt * T, hi += 8.0 * kEps * nt * T;
-  for (int round = 0; round < 15; ++round) {
-    const double h = (hi - lo) / 17.0, x = fma(h, static_cast<double>(sub + 1), lo);
+  for (int round = 0; round < 12; ++round) {  // 33^12 > 2^60
+    const double h = (hi - lo) / 33.0, x = fma(h, static_cast<double>(lane + 1), lo);
     double p0 = 1.0, p1 = de[0].x - x;
     int sign = p1 <= 0.0 ? 1 : 0, cnt = sign;  // sign of the last term: 1 negative
     auto step = [&](const double2 &c) {
@@ -231,11 +251,6 @@ __global__ void __launch_bounds__(32) bisect_kernel(const double *__restrict__ d
       cnt += now ^ sign;
       sign = now;
     };
-    auto rescale = [&]() {
-      const int ex = max(__double2hiint(p0) & 0x7FF00000, __double2hiint(p1) & 0x7FF00000);
-      const double f = __hiloint2double(ex == 0 ? 0x5FF00000 : 0x7FE00000 - ex, 0);  // 2^-(exponent)
-      p0 *= f, p1 *= f;
-    };
     int j = 1;
 #pragma unroll 1
     for (; j + 8 <= T; j += 8) {
@@ -244,16 +259,18 @@ __global__ void __launch_bounds__(32) bisect_kernel(const double *__restrict__ d
       for (int u = 0; u < 8; ++u) c[u] = de[j + u];
 #pragma unroll
       for (int u = 0; u < 8; ++u) step(c[u]);
-      rescale();
+      const int ex = max(__double2hiint(p0) & 0x7FF00000, __double2hiint(p1) & 0x7FF00000);
+      const double f = __hiloint2double(ex == 0 ? 0x5FF00000 : 0x7FE00000 - ex, 0);  // 2^-(exponent)
+      p0 *= f, p1 *= f;
     }
     for (; j < T; ++j) step(de[j]);
-    const uint32_t above = __ballot_sync(0xffffffffu, cnt > i) >> (lane & 16) & 0xFFFFu;
-    const int f = above ? __ffs(above) - 1 : 16;  // the first point with more than i eigenvalues below it
+    const uint32_t above = __ballot_sync(0xffffffffu, cnt > i);
+    const int f = above ? __ffs(above) - 1 : 32;  // the first point with more than i eigenvalues below it
     const double base = lo;
-    if (f < 16) hi = fma(h, static_cast<double>(f + 1), base);
+    if (f < 32) hi = fma(h, static_cast<double>(f + 1), base);
     if (f > 0) lo = fma(h, static_cast<double>(f), base);
   }
-  if (i < T && sub == 0) lam[i] = 0.5 * (lo + hi);
+  if (lane == 0) lam[i] = 0.5 * (lo + hi);
 }
 
 // ascending eigenvalues (equal ones can come out of the bisection a rounding apart in either order) and
@@ -412,7 +429,7 @@ __global__ void __launch_bounds__(kCholThreads) chol_kernel(double *Gm, const in
       for (int c = 0; c < kCholPanel; ++c) {
         const double piv = __shfl_sync(0xffffffffu, x[c], c);
         if (c < nb && !(piv > thr)) ok = false;
-        const double root = sqrt(fmax(piv, 1e-300)), inv = 1.0 / root;
+        const double inv = rsqrt(fmax(piv, 1e-300)), root = fmax(piv, 1e-300) * inv;
         x[c] = lane == c ? root : x[c] * inv;
         if (lane == c) dinv[c] = inv;
 #pragma unroll
@@ -462,27 +479,71 @@ __global__ void __launch_bounds__(kCholThreads) chol_kernel(double *Gm, const in
   if (tid == 0 && !ok) bad[g0] = 1;
 }
 
+// P[a][b] = sum_c X[g0 + c][a] X[g0 + c][b] of every cluster larger than rmin over its first S nodes (32 x 32
+// tiles, a >= b), stored S to a row at the cluster's rows of Pm
+__host__ __device__ __forceinline__ int select_nodes(int r, int T) {
+  const int s = r + r / 8 + 24;
+  return s < T ? (s < kCholShared ? s : kCholShared) : (T < kCholShared ? T : kCholShared);
+}
+__global__ void __launch_bounds__(256) proj_kernel(const double *__restrict__ X, const int *__restrict__ gs,
+                                                  const int *__restrict__ gn, int T, int rmin, double *Pm) {
+  const int g0 = blockIdx.z, a0 = blockIdx.y * 32, b0 = blockIdx.x * 32;
+  if (gs[g0] != g0 || gn[g0] <= rmin || b0 > a0) return;
+  const int r = gn[g0], S = select_nodes(r, T);
+  if (r > S || S * S > r * T || a0 >= S) return;
+  __shared__ double sa[32][33], sb[32][33];
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+  for (int c0 = 0; c0 < r; c0 += 32) {
+    for (int it = threadIdx.x; it < 1024; it += 256) {
+      const int c = c0 + (it >> 5), u = it & 31;
+      sa[it >> 5][u] = c < r && a0 + u < S ? X[static_cast<size_t>(g0 + c) * T + a0 + u] : 0.0;
+      sb[it >> 5][u] = c < r && b0 + u < S ? X[static_cast<size_t>(g0 + c) * T + b0 + u] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int c = 0; c < 32; ++c) {
+      const double x0 = sa[c][ty], x1 = sa[c][ty + 16], y0 = sb[c][tx], y1 = sb[c][tx + 16];
+      acc[0][0] = fma(x0, y0, acc[0][0]), acc[0][1] = fma(x0, y1, acc[0][1]);
+      acc[1][0] = fma(x1, y0, acc[1][0]), acc[1][1] = fma(x1, y1, acc[1][1]);
+    }
+    __syncthreads();
+  }
+  double *P = Pm + static_cast<size_t>(g0) * T;
+  for (int i = 0; i < 2; ++i)
+    for (int j = 0; j < 2; ++j) {
+      const int a = a0 + ty + 16 * i, b = b0 + tx + 16 * j;
+      if (a < S && b <= a) P[static_cast<size_t>(a) * S + b] = acc[i][j];
+    }
+}
+
 // The nodes of each cluster larger than kSeqGroup that give its canonical basis: the first r nodes, in
 // order, whose P e_j is independent of those chosen before (codes have exactly dependent ones).  A
 // right-looking Cholesky of P (over the nodes 0 .. S - 1) that leaves a node out where the
 // squared residual is below 1e-14; one between that and 1e-8, where this arithmetic cannot tell, or too few
 // nodes, mark the cluster for the one-by-one kernel.  node[g0 + a]: the a-th node chosen.
-__global__ void __launch_bounds__(kCholThreads) select_kernel(const double *__restrict__ V, const int *__restrict__ gs,
+__global__ void __launch_bounds__(kCholThreads) select_kernel(const double *__restrict__ V, const double *__restrict__ Pm, const int *__restrict__ gs,
                                                               const int *__restrict__ gn, int T, int rmin, int *node,
                                                               int *bad) {
   extern __shared__ double tri[];
   __shared__ double col[kCholShared];
   const int g0 = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (gs[g0] != g0 || gn[g0] <= rmin) return;
-  const int r = gn[g0], S = min(T, kCholShared);
+  const int r = gn[g0], S = select_nodes(r, T);
   if (r > S) {
     if (tid == 0) bad[g0] = 1;
     return;
   }
-  // P[a][b] = sum_c X[g0 + c][a] X[g0 + c][b], 4 x 4 outputs a thread
+  const bool ready = S * S <= r * T;  // proj_kernel has formed P
+  if (ready) {
+    const double *P = Pm + static_cast<size_t>(g0) * T;
+    for (int a = warp; a < S; a += kCholThreads / 32)
+      for (int b = lane; b <= a; b += 32) tri[a * (a + 1) / 2 + b] = P[static_cast<size_t>(a) * S + b];
+  }
+  // else here, 4 x 4 outputs a thread
   const double *X = V + static_cast<size_t>(g0) * T;
   const int nt = (S + 3) / 4, ntri = nt * (nt + 1) / 2;
-  for (int t = tid; t < ntri; t += kCholThreads) {
+  for (int t = ready ? ntri : tid; t < ntri; t += kCholThreads) {
     int ta = static_cast<int>((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
     while ((ta + 1) * (ta + 2) / 2 <= t) ++ta;
     while (ta * (ta + 1) / 2 > t) --ta;
@@ -515,7 +576,7 @@ __global__ void __launch_bounds__(kCholThreads) select_kernel(const double *__re
     if (!(piv > 1e-8)) ok = false;
     if (tid == 0) node[g0 + got] = j;
     ++got;
-    const double inv = 1.0 / sqrt(piv);
+    const double inv = rsqrt(piv);
     for (int a = j + 1 + tid; a < S; a += kCholThreads) col[a] = tri[a * (a + 1) / 2 + j] * inv;
     __syncthreads();
     for (int a = j + 1 + warp; a < S; a += kCholThreads / 32) {
@@ -576,42 +637,59 @@ __global__ void __launch_bounds__(256) trsm_kernel(const double *__restrict__ Gm
   }
 }
 
+// g[k] = v_k . v_{k-1} for the pairs of reflections that back_kernel applies together
+__global__ void __launch_bounds__(32) pair_kernel(const double *__restrict__ Vh, int T, double *g) {
+  const int k = blockIdx.x + 1;
+  double s = 0.0;
+  for (int j = k + 1 + threadIdx.x; j < T; j += 32)
+    s = fma(Vh[static_cast<size_t>(k) * T + j], Vh[static_cast<size_t>(k - 1) * T + j], s);
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (threadIdx.x == 0) g[k] = s;
+}
+
 // Z <- (H_0 H_1 ... H_{T-3}) Z for every row of Z: a warp per vector, its elements j = lane + 32 u in
-// registers (NE per lane), the next reflection's vector loaded while the current one is applied
+// registers (NE per lane), two reflections at a time: z + t_k v_k + t_{k-1} v_{k-1} with
+// t_k = -tau_k (v_k . z) and t_{k-1} = -tau_{k-1} (v_{k-1} . z + t_k g_k).  Bound by the latency of the
+// sums; the vectors of the next two reflections are loaded while the current ones are applied.
 template <int NE>
-__global__ void __launch_bounds__(128) back_kernel(const double *__restrict__ Vh, const double *__restrict__ tau, int T,
-                                                  double *Z) {
+__global__ void __launch_bounds__(64) back_kernel(const double *__restrict__ Vh, const double *__restrict__ tau,
+                                                 const double *__restrict__ g, int T, double *Z) {
   const int vec = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (vec >= T) return;
-  double z[NE], v[NE];
+  double z[NE], va[NE], vb[NE], ta = 0.0, tb = 0.0, gg = 0.0;
 #pragma unroll
   for (int u = 0; u < NE; ++u) z[u] = lane + 32 * u < T ? Z[static_cast<size_t>(vec) * T + lane + 32 * u] : 0.0;
-  auto load = [&](int k) {
+  auto load = [&](int k) {  // reflections k and k - 1 (none below 0)
 #pragma unroll
     for (int u = 0; u < NE; ++u) {
       const int j = lane + 32 * u;
-      v[u] = k >= 0 && j > k && j < T ? __ldg(Vh + static_cast<size_t>(k) * T + j) : 0.0;
+      va[u] = k >= 0 && j > k && j < T ? __ldg(Vh + static_cast<size_t>(k) * T + j) : 0.0;
+      vb[u] = k >= 1 && j > k - 1 && j < T ? __ldg(Vh + static_cast<size_t>(k - 1) * T + j) : 0.0;
     }
+    ta = k >= 0 ? -__ldg(tau + k) : 0.0;
+    tb = k >= 1 ? -__ldg(tau + k - 1) : 0.0;
+    gg = k >= 1 ? __ldg(g + k) : 0.0;
   };
   load(T - 3);
-  double tn = __ldg(tau + T - 3);
-  for (int k = T - 3; k >= 0; --k) {
-    double cur[NE], s[2] = {0.0, 0.0};
-    const double tk = tn;
+  for (int k = T - 3; k >= 0; k -= 2) {
+    double ca[NE], cb[NE], sa[3] = {0.0, 0.0, 0.0}, sb[3] = {0.0, 0.0, 0.0};
+    const double tak = ta, tbk = tb, gk = gg;
 #pragma unroll
-    for (int u = 0; u < NE; ++u) cur[u] = v[u];
-    load(k - 1);
-    if (k > 0) tn = __ldg(tau + k - 1);
-    const int u0 = (k + 1) >> 5;
+    for (int u = 0; u < NE; ++u) ca[u] = va[u], cb[u] = vb[u];
+    load(k - 2);
+    const int u0 = k >> 5;  // elements up to k - 1 of both vectors are zero
 #pragma unroll
     for (int u = 0; u < NE; ++u)
-      if (u >= u0) s[u & 1] = fma(cur[u], z[u], s[u & 1]);
-    double t = s[0] + s[1];
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    t *= -tk;
+      if (u >= u0) sa[u % 3] = fma(ca[u], z[u], sa[u % 3]), sb[u % 3] = fma(cb[u], z[u], sb[u % 3]);
+    double a = (sa[0] + sa[1]) + sa[2], c = (sb[0] + sb[1]) + sb[2];
+    for (int o = 16; o > 0; o >>= 1) {
+      a += __shfl_xor_sync(0xffffffffu, a, o);
+      c += __shfl_xor_sync(0xffffffffu, c, o);
+    }
+    const double t0 = tak * a, t1 = tbk * fma(t0, gk, c);
 #pragma unroll
     for (int u = 0; u < NE; ++u)
-      if (u >= u0) z[u] = fma(t, cur[u], z[u]);
+      if (u >= u0) z[u] = fma(t1, cb[u], fma(t0, ca[u], z[u]));
   }
 #pragma unroll
   for (int u = 0; u < NE; ++u)
@@ -697,11 +775,13 @@ struct MhsaCoef {
 // The fixed-point form of a node's attention.  Double operations are 64 times scarcer than integer ones on
 // this GPU, and the T^2 exponentials of a node and head take about 27 of them each, so the softmax runs on
 // 64-bit integers, with no less precision: scores in base 2 to 2^-52 (a double score of magnitude 8 or
-// more is rounded to 2^-50), exponentials and their products to 2^-64 of the row's largest one, sums
+// more is rounded to 2^-50; 2^-48 past +-1024, where doubles keep 2^-43), exponentials and their products to 2^-64 of the row's largest one, sums
 // exact in 96 bits.  With l = lambda / 2^el and v = u / 2^eu in (-1, 1), a row's scores are
 // A (l_k - l_min) / 2 + B (v_k + 1) / 2 up to a constant, which a softmax does not see; |A| and |B| are
 // scaled by 2^(63 - er) to fill 63 bits.
-constexpr int kFixMaxExp = 8;  // |A|, |B| < 2^8: scores within +-512 (a wider row takes doubles)
+// |A|, |B| < 2^9 (scores within +-1024): 52 fraction bits; < 2^13: 48, still more than a double of that size
+// holds; a wider row takes doubles, whose warp then takes 20 times as long as the others
+constexpr int kFixNarrow = 9, kFixWide = 13;
 struct FixKey {
   uint64_t l, v;  // (l - l_min) / 2 and (v + 1) / 2, 64 fraction bits
 };
@@ -748,7 +828,8 @@ __global__ void exp_table_kernel(uint64_t *table) {
 }
 
 // one CTA per node j: SPE_j[c] = sum_e sum_k (mean_i PL_i va_e[k] + mean_i PU_i vb_e[k]) Wo[e d_e + k][c]
-// T = 576, 4 heads, 576 nodes: 41 ms with double operations, now 6.1 ms.
+// T = 576, 4 heads, 576 nodes: 41 ms with double operations, now 3.8 ms (6.1 while rows with scores past
+// +-512, 4% of the warps, took doubles).
 __global__ void __launch_bounds__(576) mhsa_kernel(const double *lam, const double *U, int T, int heads,
                                                    const MhsaCoef coef, const double *va, const double *vb,
                                                    const double *wo, const uint64_t *exp_table, int d_spe, float *spe,
@@ -758,7 +839,7 @@ __global__ void __launch_bounds__(576) mhsa_kernel(const double *lam, const doub
   FixKey *key = reinterpret_cast<FixKey *>(sh + 2 * T);
   uint64_t *table = reinterpret_cast<uint64_t *>(key + T);
   float2 *key32 = reinterpret_cast<float2 *>(table + kFixTable);
-  __shared__ double red[32], mean[2 * kSpeMaxHeads];
+  __shared__ double red[32], mean[2 * kSpeMaxHeads], part[kSpeMaxHeads][18][2];  // at most 18 warps
   const int j = blockIdx.x;
   double um = 0.0;
   for (int a = threadIdx.x; a < T; a += blockDim.x) {
@@ -790,28 +871,34 @@ __global__ void __launch_bounds__(576) mhsa_kernel(const double *lam, const doub
       const double A1 = L[i] * al + u[i] * ga, B1 = L[i] * be + u[i] * de;
       const double log2e = 1.4426950408889634074;
       const double A = scalbn(A1 * log2e, el + 1), B = scalbn(B1 * log2e, eu + 1), top = fmax(fabs(A), fabs(B));
-      if (top < static_cast<double>(1 << kFixMaxExp)) {
+      if (top < static_cast<double>(1 << kFixWide)) {
         int er = top > 0.0 ? ilogb(top) + 1 : 0;
         if (er < -40) er = -40;
         const uint64_t Ai = static_cast<uint64_t>(scalbn(fabs(A), 63 - er)), Bi = static_cast<uint64_t>(scalbn(fabs(B), 63 - er));
         // the score's negative from magnitudes: flip the bits where a coefficient is positive (-x - 1 = ~x)
         const uint64_t na = A > 0.0 ? ~0ull : 0ull, nb = B > 0.0 ? ~0ull : 0ull;
-        const int shift = 11 - er;  // the products have 63 - er fraction bits
         const float Af = static_cast<float>(A), Bf = static_cast<float>(B);
         float m32 = -INFINITY;
         for (int k = 0; k < T; ++k) m32 = fmaxf(m32, __fmaf_rn(Af, key32[k].x, __fmul_rn(Bf, key32[k].y)));
-        // any shift near the maximum serves: the single-precision one, raised above its own error (2^-13)
-        const uint64_t m = static_cast<uint64_t>(static_cast<int64_t>((static_cast<double>(m32) + 0.015625) * 4503599627370496.0));
         FixSum l = {0, 0}, pl = {0, 0}, pu = {0, 0};
+        auto row = [&](auto wide_tag) {
+          constexpr int F = decltype(wide_tag)::value ? 48 : 52;  // fraction bits of a score
+          const int shift = 63 - F - er;                          // the products have 63 - er
+          // any shift near the maximum serves: the single-precision one, raised above its own error (2^-11, 2^-7)
+          const uint64_t m = static_cast<uint64_t>(static_cast<int64_t>((static_cast<double>(m32) + 0.015625) * static_cast<double>(1ll << F)));
 #pragma unroll 2
-        for (int k = 0; k < T; ++k) {
-          const FixKey f = key[k];
-          const uint64_t y = m + ((mulhi3(Ai, f.l) >> shift) ^ na) + ((mulhi3(Bi, f.v) >> shift) ^ nb);
-          const uint64_t p = fix_exp2(y, table);
-          l.add(p);
-          pl.add(mulhi3(p, f.l));
-          pu.add(mulhi3(p, f.v));
-        }
+          for (int k = 0; k < T; ++k) {
+            const FixKey f = key[k];
+            uint64_t y = m + ((mulhi3(Ai, f.l) >> shift) ^ na) + ((mulhi3(Bi, f.v) >> shift) ^ nb);
+            if (F == 48) y = (y < (64ull << F) ? y : 64ull << F) << 4;
+            const uint64_t p = fix_exp2(y, table);
+            l.add(p);
+            pl.add(mulhi3(p, f.l));
+            pu.add(mulhi3(p, f.v));
+          }
+        };
+        if (er <= kFixNarrow) row(std::false_type{});
+        else row(std::true_type{});
         // sum p v = 2 sum p (v + 1) / 2 - sum p, formed before it is rounded
         const uint64_t tl = pu.lo << 1;
         const uint32_t th = (pu.hi << 1) | static_cast<uint32_t>(pu.lo >> 63);
@@ -834,9 +921,17 @@ __global__ void __launch_bounds__(576) mhsa_kernel(const double *lam, const doub
         spu += pu / l;
       }
     }
-    spl = block_sum(spl, red);
-    spu = block_sum(spu, red);
-    if (threadIdx.x == 0) mean[2 * e] = spl / T, mean[2 * e + 1] = spu / T;
+    for (int o = 16; o > 0; o >>= 1) {
+      spl += __shfl_xor_sync(0xffffffffu, spl, o);
+      spu += __shfl_xor_sync(0xffffffffu, spu, o);
+    }
+    if ((threadIdx.x & 31) == 0) part[e][threadIdx.x >> 5][0] = spl, part[e][threadIdx.x >> 5][1] = spu;
+  }
+  __syncthreads();
+  if (threadIdx.x < 2 * heads) {
+    double s = 0.0;
+    for (int w = 0; w < static_cast<int>(blockDim.x >> 5); ++w) s += part[threadIdx.x >> 1][w][threadIdx.x & 1];
+    mean[threadIdx.x] = s / T;
   }
   __syncthreads();
   const int d_e = d_spe / heads;
@@ -940,7 +1035,7 @@ cudaError_t run_spe_table(const uint8_t *H, int n, int m, int d_spe, int heads, 
                                         nullptr)))
       goto done;
   }
-  bisect_kernel<<<(T + 1) / 2, 32, sizeof(double2) * T>>>(d, ed, T, lam);
+  bisect_kernel<<<T, 32, sizeof(double2) * T>>>(d, ed, T, lam);
   group_kernel<<<1, kSpeMaxTokens>>>(lam, T, cluster_tol, gs, gn);
   if (!ok(cudaFuncSetAttribute(chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kCholSmem))) ||
       !ok(cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kCholSmem))))
@@ -973,12 +1068,17 @@ cudaError_t run_spe_table(const uint8_t *H, int n, int m, int d_spe, int heads, 
       }
     }
   }
-  if (T <= 128) back_kernel<4><<<(T + 3) / 4, 128>>>(V, tau, T, X);
-  else if (T <= 320) back_kernel<10><<<(T + 3) / 4, 128>>>(V, tau, T, X);
-  else if (T <= 576) back_kernel<18><<<(T + 3) / 4, 128>>>(V, tau, T, X);
-  else back_kernel<32><<<(T + 3) / 4, 128>>>(V, tau, T, X);
+  if (T > 3) pair_kernel<<<T - 3, 32>>>(V, T, pbuf);  // (pbuf: the reduction is done with it)
+  if (T <= 128) back_kernel<4><<<(T + 1) / 2, 64>>>(V, tau, pbuf, T, X);
+  else if (T <= 320) back_kernel<10><<<(T + 1) / 2, 64>>>(V, tau, pbuf, T, X);
+  else if (T <= 576) back_kernel<18><<<(T + 1) / 2, 64>>>(V, tau, pbuf, T, X);
+  else back_kernel<32><<<(T + 1) / 2, 64>>>(V, tau, pbuf, T, X);
   // the canonical basis in coordinates (V is free now), then in node coordinates
-  select_kernel<<<T, kCholThreads, kCholSmem>>>(X, gs, gn, T, kSeqGroup, node, badd + T);
+  {
+    const int st = (std::min(T, kCholShared) + 31) / 32;
+    proj_kernel<<<dim3(st, st, T), 256>>>(X, gs, gn, T, kSeqGroup, Gm);
+  }
+  select_kernel<<<T, kCholThreads, kCholSmem>>>(X, Gm, gs, gn, T, kSeqGroup, node, badd + T);
   coords_kernel<<<T, 128>>>(X, gs, gn, node, badd + T, T, kSeqGroup, V);
   chol_qr(V, Gm, gs, gn, T, kSeqGroup, 1, 1e-8, badd + T);
   chol_qr(V, Gm, gs, gn, T, kSeqGroup, 1, 1e-8, badd + T);

@@ -62,9 +62,9 @@ def test_eigenpairs_of_graph(name):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("scale", [1e-3, 1.0, 4.0, 40.0, 1e3])
+@pytest.mark.parametrize("scale", [1e-3, 1.0, 4.0, 8.0, 20.0, 40.0, 1e3])
 def test_table_over_score_ranges(scale):
-    # scores from about 1e-6 to past the fixed-point range (512 in base 2), where rows take doubles; the
+    # scores from about 1e-6 over both fixed-point ranges (1024 and 16384 in base 2) to where rows take doubles; the
     # error of a row's probabilities is that of its scores, 2^-52 of their size or more
     H = I.make_code("bch31_16").H
     p = I.spe_params(H, 16, seed=3)
