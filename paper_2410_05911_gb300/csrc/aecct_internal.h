@@ -261,12 +261,14 @@ template <int D, int ATT>
 using KernelLayout = SmemLayout<D, ATT == 1 || ATT == 3, ATT == 3 ? 2 : 1>;
 
 // decoder_kernel.cuh.  ATT: 0 = per-row neighbour lists, 1 = warp tasks, 2 = per-row lists over
-// per-head staged rows (d >= 64), 3 = warp tasks at two CTAs per SM (d = 32); ACT: 0 = ReLU, 1 = GELU; LIN: 0 = AAP linears, 1 = full-precision
-// (bf16) linears.  Instantiated in decoder_kernel.cu (0, 0), decoder_kernel_gelu.cu (1, 0),
-// decoder_kernel_fp.cu (0, 1) and decoder_kernel_fp_gelu.cu (1, 1).
-template <int D, int ATT, int ACT, int LIN>
+// per-head staged rows (d >= 64), 3 = warp tasks at two CTAs per SM (d = 32); ACT: 0 = ReLU, 1 = GELU;
+// LIN: 0 = AAP linears, 1 = full-precision (bf16) linears.  Instantiated in decoder_kernel.cu (0, 0), decoder_kernel_gelu.cu (1, 0),
+// decoder_kernel_fp.cu (0, 1) and decoder_kernel_fp_gelu.cu (1, 1).  CAP: 1 = with the integer-core capture,
+// 0 = without (warp tasks, ATT 1 and 3, whose kernels with it are instantiated in decoder_kernel_cap.cu and
+// decoder_kernel_cap_fp.cu).
+template <int D, int ATT, int ACT, int LIN, int CAP>
 cudaError_t launch_decode(const DecodeParams &p, cudaStream_t stream);
-template <int D, int ATT, int ACT, int LIN>
+template <int D, int ATT, int ACT, int LIN, int CAP>
 cudaError_t prepare_decode_kernel(int cluster_ctas, uint32_t plan_bytes, int *max_active_clusters);
 constexpr uint32_t kMaxDynSmem = 232448;  // the largest dynamic shared memory a CTA may opt into (227 KB)
 constexpr int kStagedMaxRows = 640;  // staged attention: rows of a group (64 bytes of K and of V each, 40 KB + 40 KB)

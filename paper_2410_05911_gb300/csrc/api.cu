@@ -271,32 +271,46 @@ bool assign_scheduler(const std::vector<int> &cost, int cap, std::vector<int> &o
   return best < 1e300;
 }
 
-// the compiled kernel for (d, attention path ATT, activation ACT, linear mode LIN)
+// the compiled kernel for (d, attention path ATT, activation ACT, linear mode LIN, capture CAP); only the warp
+// tasks (ATT 1 and 3) come without the capture code too
+template <int D, int ATT, int ACT, int LIN>
+cudaError_t prepare_cap(int C, uint32_t pb, int *max_clusters) {
+  if constexpr (ATT == 1 || ATT == 3) {
+    const cudaError_t e = prepare_decode_kernel<D, ATT, ACT, LIN, 0>(C, pb, max_clusters);
+    if (e != cudaSuccess) return e;
+  }
+  return prepare_decode_kernel<D, ATT, ACT, LIN, 1>(C, pb, max_clusters);
+}
+template <int D, int ATT, int ACT, int LIN>
+cudaError_t launch_cap(const DecodeParams &p, cudaStream_t stream) {
+  if constexpr (ATT == 1 || ATT == 3)
+    if (p.cap_B == 0) return launch_decode<D, ATT, ACT, LIN, 0>(p, stream);
+  return launch_decode<D, ATT, ACT, LIN, 1>(p, stream);
+}
 template <int ACT, int LIN>
 cudaError_t prepare_any(int D, int att, int C, uint32_t pb, int *max_clusters) {
   if (att == 1)
-    return D == 32   ? prepare_decode_kernel<32, 1, ACT, LIN>(C, pb, max_clusters)
-           : D == 64 ? prepare_decode_kernel<64, 1, ACT, LIN>(C, pb, max_clusters)
-                     : prepare_decode_kernel<128, 1, ACT, LIN>(C, pb, max_clusters);
-  if (att == 3) return prepare_decode_kernel<32, 3, ACT, LIN>(C, pb, max_clusters);  // d = 32 only
+    return D == 32   ? prepare_cap<32, 1, ACT, LIN>(C, pb, max_clusters)
+           : D == 64 ? prepare_cap<64, 1, ACT, LIN>(C, pb, max_clusters)
+                     : prepare_cap<128, 1, ACT, LIN>(C, pb, max_clusters);
+  if (att == 3) return prepare_cap<32, 3, ACT, LIN>(C, pb, max_clusters);  // d = 32 only
   if (att == 2)
-    return D == 64 ? prepare_decode_kernel<64, 2, ACT, LIN>(C, pb, max_clusters)
-                   : prepare_decode_kernel<128, 2, ACT, LIN>(C, pb, max_clusters);
-  if (D == 32) return prepare_decode_kernel<32, 0, ACT, LIN>(C, pb, max_clusters);
-  if (D == 64) return prepare_decode_kernel<64, 0, ACT, LIN>(C, pb, max_clusters);
-  return prepare_decode_kernel<128, 0, ACT, LIN>(C, pb, max_clusters);
+    return D == 64 ? prepare_cap<64, 2, ACT, LIN>(C, pb, max_clusters) : prepare_cap<128, 2, ACT, LIN>(C, pb, max_clusters);
+  if (D == 32) return prepare_cap<32, 0, ACT, LIN>(C, pb, max_clusters);
+  if (D == 64) return prepare_cap<64, 0, ACT, LIN>(C, pb, max_clusters);
+  return prepare_cap<128, 0, ACT, LIN>(C, pb, max_clusters);
 }
 template <int ACT, int LIN>
 cudaError_t launch_any(int D, int att, const DecodeParams &p, cudaStream_t stream) {
   if (att == 1)
-    return D == 32   ? launch_decode<32, 1, ACT, LIN>(p, stream)
-           : D == 64 ? launch_decode<64, 1, ACT, LIN>(p, stream)
-                     : launch_decode<128, 1, ACT, LIN>(p, stream);
-  if (att == 3) return launch_decode<32, 3, ACT, LIN>(p, stream);
-  if (att == 2) return D == 64 ? launch_decode<64, 2, ACT, LIN>(p, stream) : launch_decode<128, 2, ACT, LIN>(p, stream);
-  if (D == 32) return launch_decode<32, 0, ACT, LIN>(p, stream);
-  if (D == 64) return launch_decode<64, 0, ACT, LIN>(p, stream);
-  return launch_decode<128, 0, ACT, LIN>(p, stream);
+    return D == 32   ? launch_cap<32, 1, ACT, LIN>(p, stream)
+           : D == 64 ? launch_cap<64, 1, ACT, LIN>(p, stream)
+                     : launch_cap<128, 1, ACT, LIN>(p, stream);
+  if (att == 3) return launch_cap<32, 3, ACT, LIN>(p, stream);
+  if (att == 2) return D == 64 ? launch_cap<64, 2, ACT, LIN>(p, stream) : launch_cap<128, 2, ACT, LIN>(p, stream);
+  if (D == 32) return launch_cap<32, 0, ACT, LIN>(p, stream);
+  if (D == 64) return launch_cap<64, 0, ACT, LIN>(p, stream);
+  return launch_cap<128, 0, ACT, LIN>(p, stream);
 }
 cudaError_t prepare_variant(int act, int lin, int D, int att, int C, uint32_t pb, int *max_clusters) {
   if (lin == 0)

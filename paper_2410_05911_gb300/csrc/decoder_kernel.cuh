@@ -1032,8 +1032,12 @@ struct Issuer<128, ATT> {
 // ------------------------------------------------------------------------------------------
 // the kernel
 // ------------------------------------------------------------------------------------------
-template <int D, int ATT, int ACT, int LIN>
+template <int D, int ATT, int ACT, int LIN, int CAP>
 __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) aecct_decoder_kernel(const __grid_constant__ DecodeParams p) {
+  // CAP: 1 = records the integer core where p.cap_B asks for it; 0 = compiled without that code, so that the
+  // capture's pointers and tests hold no registers in the epilogues.  Only the warp tasks have it (BCH(63,36)
+  // 496.2 -> 488.5 ms, Polar(64,32) 45.6 -> 45.0 ms, one word of BCH(31,16) 38.0 -> 37.1 us); staged attention
+  // spills more without the capture and was 0.3% slower
   // ATT: 0 = per-row neighbour lists, 1 = warp tasks, 2 = per-row lists over per-head staged rows, 3 = warp
   // tasks at two CTAs per SM (d = 32)
   constexpr bool TASKS = ATT == 1 || ATT == 3, STAGED = ATT == 2;
@@ -1274,7 +1278,8 @@ __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) ae
       named_bar_sync(5, kEpiThreads);
       const int64_t b = gi * p.G + g;
       const bool valid = row_cw && b < p.B;
-      const bool cap = valid && b < p.cap_B;
+      bool cap = false;
+      if constexpr (CAP == 1) cap = valid && b < p.cap_B;
       const float *yrow = ybuf + (valid ? g : 0) * n;
       // rows of the group's words that the batch holds: the tasks of the others are skipped (one word of
       // BCH(31,16), whose groups hold two: 40.1 -> 37.8 us).  Only where groups of several words and short
@@ -2200,11 +2205,11 @@ __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) ae
   }
 }
 
-template <int D, int ATT, int ACT, int LIN>
+template <int D, int ATT, int ACT, int LIN, int CAP>
 cudaError_t prepare_decode_kernel(int cluster_ctas, uint32_t plan_bytes, int *max_active_clusters) {
   using L = KernelLayout<D, ATT>;
   const uint32_t total = L::kTotal + plan_bytes;
-  cudaError_t e = cudaFuncSetAttribute(aecct_decoder_kernel<D, ATT, ACT, LIN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  cudaError_t e = cudaFuncSetAttribute(aecct_decoder_kernel<D, ATT, ACT, LIN, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(total));
   if (e != cudaSuccess) return e;
   // ask for the smallest shared-memory carve-out that holds the SM's CTAs (1 KB for each is
@@ -2215,7 +2220,7 @@ cudaError_t prepare_decode_kernel(int cluster_ctas, uint32_t plan_bytes, int *ma
     return e;
   if (smem_sm > 0) {
     const int pct = static_cast<int>((100ll * L::kCtasPerSm * (total + 1024) + smem_sm - 1) / smem_sm);
-    e = cudaFuncSetAttribute(aecct_decoder_kernel<D, ATT, ACT, LIN>, cudaFuncAttributePreferredSharedMemoryCarveout,
+    e = cudaFuncSetAttribute(aecct_decoder_kernel<D, ATT, ACT, LIN, CAP>, cudaFuncAttributePreferredSharedMemoryCarveout,
                              pct > 100 ? 100 : pct);
     if (e != cudaSuccess) return e;
   }
@@ -2230,10 +2235,10 @@ cudaError_t prepare_decode_kernel(int cluster_ctas, uint32_t plan_bytes, int *ma
   cfg.dynamicSmemBytes = total;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaOccupancyMaxActiveClusters(max_active_clusters, aecct_decoder_kernel<D, ATT, ACT, LIN>, &cfg);
+  return cudaOccupancyMaxActiveClusters(max_active_clusters, aecct_decoder_kernel<D, ATT, ACT, LIN, CAP>, &cfg);
 }
 
-template <int D, int ATT, int ACT, int LIN>
+template <int D, int ATT, int ACT, int LIN, int CAP>
 cudaError_t launch_decode(const DecodeParams &p, cudaStream_t stream) {
   using L = KernelLayout<D, ATT>;
   cudaLaunchConfig_t cfg = {};
@@ -2248,7 +2253,7 @@ cudaError_t launch_decode(const DecodeParams &p, cudaStream_t stream) {
   cfg.stream = stream;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, aecct_decoder_kernel<D, ATT, ACT, LIN>, p);
+  return cudaLaunchKernelEx(&cfg, aecct_decoder_kernel<D, ATT, ACT, LIN, CAP>, p);
 }
 
 }  // namespace aecct

@@ -149,3 +149,28 @@ def test_two_ctas_per_sm_equal_one(n, m, weight, variant):
     torch.cuda.synchronize()
     assert all(torch.equal(first[k].view(torch.uint8), again[k].view(torch.uint8)) for k in first)
     dec.close()
+
+
+# the warp tasks are compiled with and without the capture: same outputs, also where only part of the batch is
+# recorded and after the capture is off again
+@pytest.mark.gpu
+@pytest.mark.parametrize("d,many", [(32, False), (32, True), (64, False), (128, False)])
+@pytest.mark.parametrize("variant", ["relu", "gelu", "full", "full-gelu"])
+def test_plain_decode_equals_decode_with_capture(d, many, variant):
+    model = I.random_model(random_code(31, 15, 3, d), d, 2, seed=d, spe_noise=True,
+                           activation=1 if "gelu" in variant else 0, full_precision="full" in variant)
+    dec = A.Decoder(model, attention_mode=2)
+    q = dec.query()
+    assert q["attention_mode"] == 2
+    B = q["words_per_group"] * (q["max_clusters"] + 3) + 1 if many else q["words_per_group"] + 1
+    rng = np.random.Generator(np.random.PCG64(d))
+    y = torch.from_numpy(rng.standard_normal((B, model.n)).astype(np.float32)).cuda()
+    got = []
+    for cap_B in (0, 1, 0):
+        dec.set_capture(cap_B)
+        got.append([t.clone() for t in dec.decode(y)])
+        torch.cuda.synchronize()
+    assert dec.synchronize() == A.AECCT_OK
+    dec.close()
+    for other in got[1:]:
+        assert all(torch.equal(a.view(torch.uint8), b.view(torch.uint8)) for a, b in zip(got[0], other))
