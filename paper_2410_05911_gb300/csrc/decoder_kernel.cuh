@@ -1175,12 +1175,12 @@ __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) ae
     auto word_max = [&](float a_row, bool publish, int row, int gw) -> float {
       if (publish) rowmax_s[row] = a_row;
       named_bar_sync(5, kEpiThreads);
-      if (warp < p.G) {
+      for (int w = warp; w < p.G; w += kEpiWarps) {
         float a = 0.0f;
-        for (int i = lane; i < p.Tp; i += 32) a = fmaxf(a, rowmax_s[warp * p.Tp + i]);
+        for (int i = lane; i < p.Tp; i += 32) a = fmaxf(a, rowmax_s[w * p.Tp + i]);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
-        if (lane == 0) wordmax_s[warp] = a;
+        if (lane == 0) wordmax_s[w] = a;
       }
       named_bar_sync(5, kEpiThreads);
       return gw < p.G ? wordmax_s[gw] : a_row;

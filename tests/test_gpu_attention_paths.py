@@ -4,6 +4,7 @@ block and the score cache, lists whose rows are not consecutive, more words than
 import numpy as np
 import pytest
 
+from oracle import oracle as O
 from paper_2410_05911_gb300 import aecct as A
 from paper_2410_05911_gb300 import inputs as I
 
@@ -174,3 +175,21 @@ def test_plain_decode_equals_decode_with_capture(d, many, variant):
     dec.close()
     for other in got[1:]:
         assert all(torch.equal(a.view(torch.uint8), b.view(torch.uint8)) for a, b in zip(got[0], other))
+
+
+# one alpha per quantised matrix of a word, in CTAs of more words (18) than warps
+@pytest.mark.gpu
+@pytest.mark.parametrize("mode", [1, 2])
+def test_word_alpha_of_more_words_than_warps(mode):
+    model = I.random_model(random_code(5, 2, 1, 37), 32, 2, seed=5, spe_noise=True)
+    model.alpha_mode = 1
+    dec = A.Decoder(model, attention_mode=mode)
+    assert dec.query()["words_per_group"] == 18
+    y = np.random.Generator(np.random.PCG64(5)).standard_normal((37, 5)).astype(np.float32)
+    r = O.decode(model, y)
+    bits, syn, logits = dec.decode(torch.from_numpy(y).cuda())
+    torch.cuda.synchronize()
+    assert dec.synchronize() == A.AECCT_OK
+    dec.close()
+    assert (logits.cpu().numpy().view(np.int32) == r["logits"].view(np.int32)).all()
+    assert (bits.cpu().numpy() == r["bits"]).all() and (syn.cpu().numpy() == r["syndrome"]).all()
