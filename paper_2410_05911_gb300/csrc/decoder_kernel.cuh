@@ -152,7 +152,7 @@ __device__ __forceinline__ float psum(const float *v) {
 
 struct Ctl {
   volatile int *abort;
-  int *err;
+  volatile int *err;  // the call's status word, in pinned host or device memory: only ever set to 1
   long long limit;
 };
 
@@ -168,7 +168,7 @@ static __device__ __noinline__ bool wait_bar_slow(const Ctl c, uint32_t bar, uin
     if (*c.abort) return false;
     if (clock64() - t0 > c.limit) {
       *c.abort = 1;
-      atomicOr(c.err, 1);
+      *c.err = 1;
       return false;
     }
   }
@@ -194,7 +194,7 @@ static __device__ __noinline__ bool wait_bar_drain(const Ctl c, uint32_t bar, ui
   const long long t0 = clock64();
   while (!mbar_try_wait(bar, parity)) {
     if (clock64() - t0 > kDrainLimitCycles) {
-      atomicOr(c.err, 1);
+      *c.err = 1;
       return false;
     }
   }
