@@ -53,6 +53,7 @@ struct aecct_handle {
   uint16_t *perm = nullptr, *pos = nullptr;
   float *kv_scratch = nullptr;  // staged attention: K and V rows per cluster
   uint8_t *plan_blob = nullptr;  // the attention plan (task mode), copied into shared memory by the kernel
+  int plans = 1;  // plans in the blob, plan_bytes each: for CTAs of G words, then G - 1, ... (d <= 64)
   uint32_t plan_bytes = 0, off_task = 0, off_grp = 0, off_uinfo = 0, off_ulist = 0, off_mask = 0, off_qslot = 0;
   // the status word of asynchronous decodes: pinned host memory that a kernel whose wait gave up writes
   // itself (d_err, the word's device address), so that a decode queues no copy behind its kernel.  A 4-byte
@@ -658,95 +659,103 @@ int aecct_create(const aecct_model_desc *desc, aecct_handle **out) {
     // where its rows' Q and A live (warps w with w % 4 = quadrant: one scheduler); d <= 64: the
     // schedulers by longest first onto the least-loaded one.  Then the warps of each scheduler by
     // assign_scheduler.
-    std::vector<std::pair<int, int>> tl;  // (cost, task)
-    for (int gi = 0; gi < ng; ++gi)
-      for (int e = 0; e < kHeads; ++e) tl.push_back({ucount[gi * 2 + (e < d.h_first ? 0 : 1)] + 4, gi * 8 + e});
-    std::stable_sort(tl.begin(), tl.end(), [](const std::pair<int, int> &x, const std::pair<int, int> &y) {
-      return x.first > y.first;
-    });
-    std::vector<std::pair<int, int>> per_sched[4];
-    long sched_load[4] = {0, 0, 0, 0};
-    for (const auto &tk : tl) {
-      int q = 0;
+    //
+    // d <= 64: one list for every number of words that a launch may give a CTA (1 to G, launch_words), in
+    // turn; each names the tasks of its words only.
+    const int variants = D == 128 ? 1 : G;
+    ptask.assign((size_t)variants * kEpiWarps * kMaxTasks, 0xFFFFu);
+    for (int words = G - variants + 1; words <= G; ++words) {
+      const int ngw = ng / G * words;  // the groups of the first `words` words
+      std::vector<std::pair<int, int>> tl;  // (cost, task)
+      for (int gi = 0; gi < ngw; ++gi)
+        for (int e = 0; e < kHeads; ++e) tl.push_back({ucount[gi * 2 + (e < d.h_first ? 0 : 1)] + 4, gi * 8 + e});
+      std::stable_sort(tl.begin(), tl.end(), [](const std::pair<int, int> &x, const std::pair<int, int> &y) {
+        return x.first > y.first;
+      });
+      std::vector<std::pair<int, int>> per_sched[4];
+      long sched_load[4] = {0, 0, 0, 0};
+      for (const auto &tk : tl) {
+        int q = 0;
+        if (D == 128) {
+          q = (grps[tk.second / 8].row0 / 32) & 3;
+        } else {
+          for (int c = 1; c < 4; ++c)
+            if (sched_load[c] < sched_load[q]) q = c;
+        }
+        per_sched[q].push_back(tk);
+        sched_load[q] += tk.first;
+      }
+      // d = 128: a task may also run on a warp of a scheduler whose lane quadrant holds no token row,
+      // its Q and A then in a 2 KB slot of weight stage W2 (idle from the previous block's FFN2 to this
+      // block's O GEMM) instead of its rows' TMEM lanes.  Every loaded scheduler hands over the subset
+      // of its tasks (at most kQSlots in all) whose cost comes closest to its excess over the mean load
+      // without passing it; each goes to the free scheduler with the least load.  BCH(63,36): the fourth
+      // quadrant holds no token row, and each of the other three hands it a 67 and a 31 (all at 294).
+      std::vector<uint8_t> slot_of((size_t)ng * 8, 0xFFu);
       if (D == 128) {
-        q = (grps[tk.second / 8].row0 / 32) & 3;
-      } else {
-        for (int c = 1; c < 4; ++c)
-          if (sched_load[c] < sched_load[q]) q = c;
+        auto by_cost = [](const std::pair<int, int> &x, const std::pair<int, int> &y) { return x.first > y.first; };
+        std::vector<int> free_q;
+        long total = 0;
+        for (int q = 0; q < 4; ++q) {
+          total += sched_load[q];
+          if (per_sched[q].empty()) free_q.push_back(q);
+        }
+        const long mean = total / 4;
+        int nmoved = 0;
+        for (int pass = 0; pass < 4 && !free_q.empty(); ++pass) {
+          int q = -1;  // the most loaded scheduler not handled yet
+          for (int c = 0; c < 4; ++c)
+            if (!per_sched[c].empty() && std::find(free_q.begin(), free_q.end(), c) == free_q.end() &&
+                sched_load[c] > mean && (q < 0 || sched_load[c] > sched_load[q]))
+              q = c;
+          if (q < 0) break;
+          const long excess = sched_load[q] - mean;
+          const int mt = static_cast<int>(std::min<size_t>(per_sched[q].size(), 12));
+          uint32_t best_set = 0;
+          long best_sum = 0;
+          for (uint32_t set = 1; set < (1u << mt); ++set) {
+            const int k = __builtin_popcount(set);
+            if (nmoved + k > kQSlots) continue;
+            long sum = 0;
+            for (int t = 0; t < mt; ++t)
+              if (set >> t & 1u) sum += per_sched[q][t].first;
+            if (sum <= excess && (sum > best_sum || (sum == best_sum && k < __builtin_popcount(best_set))))
+              best_sum = sum, best_set = set;
+          }
+          for (int t = mt - 1; t >= 0; --t) {
+            if (!(best_set >> t & 1u)) continue;
+            int fq = free_q[0];
+            for (int c : free_q)
+              if (sched_load[c] < sched_load[fq]) fq = c;
+            const std::pair<int, int> tk = per_sched[q][t];
+            per_sched[q].erase(per_sched[q].begin() + t);
+            sched_load[q] -= tk.first;
+            per_sched[fq].push_back(tk);
+            sched_load[fq] += tk.first;
+            slot_of[tk.second] = static_cast<uint8_t>(nmoved++);
+          }
+          sched_load[q] = std::min(sched_load[q], mean);  // handled: not picked again
+        }
+        for (int q = 0; q < 4; ++q) std::stable_sort(per_sched[q].begin(), per_sched[q].end(), by_cost);
+        // the group of each lane quadrant (every group of a d = 128 word starts on one), then the slots
+        pqslot.assign(4 + (size_t)ng * 8, 0xFFu);
+        for (int gi = 0; gi < ng; ++gi) pqslot[(grps[gi].row0 / 32) & 3] = static_cast<uint8_t>(gi);
+        std::copy(slot_of.begin(), slot_of.end(), pqslot.begin() + 4);
       }
-      per_sched[q].push_back(tk);
-      sched_load[q] += tk.first;
-    }
-    // d = 128: a task may also run on a warp of a scheduler whose lane quadrant holds no token row,
-    // its Q and A then in a 2 KB slot of weight stage W2 (idle from the previous block's FFN2 to this
-    // block's O GEMM) instead of its rows' TMEM lanes.  Every loaded scheduler hands over the subset
-    // of its tasks (at most kQSlots in all) whose cost comes closest to its excess over the mean load
-    // without passing it; each goes to the free scheduler with the least load.  BCH(63,36): the fourth
-    // quadrant holds no token row, and each of the other three hands it a 67 and a 31 (all at 294).
-    std::vector<uint8_t> slot_of((size_t)ng * 8, 0xFFu);
-    if (D == 128) {
-      auto by_cost = [](const std::pair<int, int> &x, const std::pair<int, int> &y) { return x.first > y.first; };
-      std::vector<int> free_q;
-      long total = 0;
+      uint16_t *list = ptask.data() + (size_t)(words - (G - variants + 1)) * kEpiWarps * kMaxTasks;
       for (int q = 0; q < 4; ++q) {
-        total += sched_load[q];
-        if (per_sched[q].empty()) free_q.push_back(q);
-      }
-      const long mean = total / 4;
-      int nmoved = 0;
-      for (int pass = 0; pass < 4 && !free_q.empty(); ++pass) {
-        int q = -1;  // the most loaded scheduler not handled yet
-        for (int c = 0; c < 4; ++c)
-          if (!per_sched[c].empty() && std::find(free_q.begin(), free_q.end(), c) == free_q.end() &&
-              sched_load[c] > mean && (q < 0 || sched_load[c] > sched_load[q]))
-            q = c;
-        if (q < 0) break;
-        const long excess = sched_load[q] - mean;
-        const int mt = static_cast<int>(std::min<size_t>(per_sched[q].size(), 12));
-        uint32_t best_set = 0;
-        long best_sum = 0;
-        for (uint32_t set = 1; set < (1u << mt); ++set) {
-          const int k = __builtin_popcount(set);
-          if (nmoved + k > kQSlots) continue;
-          long sum = 0;
-          for (int t = 0; t < mt; ++t)
-            if (set >> t & 1u) sum += per_sched[q][t].first;
-          if (sum <= excess && (sum > best_sum || (sum == best_sum && k < __builtin_popcount(best_set))))
-            best_sum = sum, best_set = set;
+        std::vector<int> cost, slot;
+        for (const auto &tk : per_sched[q]) cost.push_back(tk.first);
+        if (!assign_scheduler(cost, kMaxTasks, slot)) {
+          free_handle(h);
+          g_last_error = "attention plan: too many tasks for a warp";
+          return AECCT_ERR_UNSUPPORTED;
         }
-        for (int t = mt - 1; t >= 0; --t) {
-          if (!(best_set >> t & 1u)) continue;
-          int fq = free_q[0];
-          for (int c : free_q)
-            if (sched_load[c] < sched_load[fq]) fq = c;
-          const std::pair<int, int> tk = per_sched[q][t];
-          per_sched[q].erase(per_sched[q].begin() + t);
-          sched_load[q] -= tk.first;
-          per_sched[fq].push_back(tk);
-          sched_load[fq] += tk.first;
-          slot_of[tk.second] = static_cast<uint8_t>(nmoved++);
+        int cnt[4] = {0, 0, 0, 0};
+        for (size_t i = 0; i < per_sched[q].size(); ++i) {
+          const int w = q + 4 * slot[i];
+          list[(size_t)w * kMaxTasks + cnt[slot[i]]++] = static_cast<uint16_t>(per_sched[q][i].second);
         }
-        sched_load[q] = std::min(sched_load[q], mean);  // handled: not picked again
-      }
-      for (int q = 0; q < 4; ++q) std::stable_sort(per_sched[q].begin(), per_sched[q].end(), by_cost);
-      // the group of each lane quadrant (every group of a d = 128 word starts on one), then the slots
-      pqslot.assign(4 + (size_t)ng * 8, 0xFFu);
-      for (int gi = 0; gi < ng; ++gi) pqslot[(grps[gi].row0 / 32) & 3] = static_cast<uint8_t>(gi);
-      std::copy(slot_of.begin(), slot_of.end(), pqslot.begin() + 4);
-    }
-    ptask.assign((size_t)kEpiWarps * kMaxTasks, 0xFFFFu);
-    for (int q = 0; q < 4; ++q) {
-      std::vector<int> cost, slot;
-      for (const auto &tk : per_sched[q]) cost.push_back(tk.first);
-      if (!assign_scheduler(cost, kMaxTasks, slot)) {
-        free_handle(h);
-        g_last_error = "attention plan: too many tasks for a warp";
-        return AECCT_ERR_UNSUPPORTED;
-      }
-      int cnt[4] = {0, 0, 0, 0};
-      for (size_t i = 0; i < per_sched[q].size(); ++i) {
-        const int w = q + 4 * slot[i];
-        ptask[(size_t)w * kMaxTasks + cnt[slot[i]]++] = static_cast<uint16_t>(per_sched[q][i].second);
       }
     }
   }
@@ -826,7 +835,8 @@ int aecct_create(const aecct_model_desc *desc, aecct_handle **out) {
       while (blob.size() % 16) blob.push_back(0);
       return off;
     };
-    h->off_task = put(ptask.data(), ptask.size() * 2);
+    const size_t list = (size_t)kEpiWarps * kMaxTasks;  // the plan of best_G words first
+    h->off_task = put(ptask.data() + ptask.size() - list, list * 2);
     h->off_grp = put(pgrp.data(), pgrp.size() * 4);
     h->off_uinfo = put(puinfo.data(), puinfo.size() * 4);
     h->off_ulist = put(pulist.data(), pulist.size());
@@ -837,6 +847,13 @@ int aecct_create(const aecct_model_desc *desc, aecct_handle **out) {
       free_handle(h);
       g_last_error = "internal: the task plan exceeds its bound";
       return AECCT_ERR_UNSUPPORTED;
+    }
+    // the plans of best_G - 1, ..., 1 words, which differ in the task list alone
+    h->plans = static_cast<int>(ptask.size() / list);
+    for (int v = h->plans - 2; v >= 0; --v) {
+      const size_t at = blob.size();
+      blob.insert(blob.end(), blob.begin(), blob.begin() + h->plan_bytes);
+      std::memcpy(blob.data() + at + h->off_task, ptask.data() + v * list, list * 2);
     }
   }
   // embedding and positional encoding in one table, [D / 4][Tp][4]: row by row of a codeword (a padding
@@ -906,15 +923,25 @@ static int launch_att(const aecct_handle *h, const DecodeParams &p) {
   return h->two_per_sm && p.n_clusters > h->max_clusters ? 3 : h->att;
 }
 
+// Words per CTA of a launch.  Warp tasks of small codes have room for several words in a CTA; where the
+// batch leaves SMs idle, fewer words a CTA spread it over them, and each CTA has less attention to do.
+// BCH(31,16) (T = 46, two words to a CTA) at d = 32: one word 28.5 -> 26.7 us, 100 words 32.0 -> 27.0 us; at
+// d = 64, six blocks: 100.3 -> 83.0 and 100.5 -> 84.0 us.
+static int launch_words(const aecct_handle *h, int64_t B) {
+  if (h->plans == 1 || B >= static_cast<int64_t>(h->G) * h->max_clusters) return h->G;
+  const int64_t g = (B + h->max_clusters - 1) / h->max_clusters;
+  return static_cast<int>(g < 1 ? 1 : g);
+}
+
 // the kernel arguments of one decode call: the handle's model and plan, this call's buffers
 static DecodeParams decode_params(const aecct_handle *h, int64_t B, const float *y_dev, uint8_t *bits_dev,
                                   uint8_t *syn_dev, float *logits_dev, int *err_dev) {
   DecodeParams p = {};
   p.n = h->n, p.k = h->k, p.T = h->T, p.m = h->m, p.n_layers = h->n_layers, p.h_first = h->h_first;
   p.Tp = h->Tp;
-  p.d_spe = h->d_spe, p.C = h->C, p.G = h->G;
+  p.d_spe = h->d_spe, p.C = h->C, p.G = launch_words(h, B);
   p.B = B;
-  p.n_groups = (B + h->G - 1) / h->G;
+  p.n_groups = (B + p.G - 1) / p.G;
   const int64_t most = resident_clusters(h);
   p.n_clusters = static_cast<int>(p.n_groups < most ? p.n_groups : most);
   p.y = y_dev, p.bits = bits_dev, p.syn = syn_dev, p.logits = logits_dev;
@@ -922,7 +949,8 @@ static DecodeParams decode_params(const aecct_handle *h, int64_t B, const float 
   p.lparams = h->lparams, p.xtab = reinterpret_cast<const float4 *>(h->xtab), p.w_d1 = h->w_d1, p.b_d1 = h->b_d1;
   p.w_out = h->w_out, p.b_out = h->b_out, p.hbits = h->hbits, p.hwords = h->hwords;
   p.perm = h->perm, p.pos = h->pos;
-  p.plan_blob = reinterpret_cast<const uint4 *>(h->plan_blob), p.plan_bytes = h->plan_bytes;
+  p.plan_blob = reinterpret_cast<const uint4 *>(h->plan_blob + static_cast<size_t>(h->G - p.G) * h->plan_bytes);
+  p.plan_bytes = h->plan_bytes;
   p.off_task = h->off_task, p.off_grp = h->off_grp;
   p.off_uinfo = h->off_uinfo, p.off_ulist = h->off_ulist, p.off_mask = h->off_mask, p.off_qslot = h->off_qslot;
   p.mask_info[0] = h->mask_info[0], p.mask_info[1] = h->mask_info[1];

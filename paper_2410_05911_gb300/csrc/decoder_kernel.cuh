@@ -1296,11 +1296,6 @@ __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) ae
       bool cap = false;
       if constexpr (CAP == 1) cap = valid && b < p.cap_B;
       const float *yrow = ybuf + (valid ? g : 0) * n;
-      // rows of the group's words that the batch holds: the tasks of the others are skipped (one word of
-      // BCH(31,16), whose groups hold two: 40.1 -> 37.8 us).  Only where groups of several words and short
-      // launches meet, the single-CTA kernel of d = 32: elsewhere the live register costs more.
-      constexpr bool kSkipDead = ATT == 1 && D == 32;
-      const uint32_t live_rows = kSkipDead ? static_cast<uint32_t>(min(static_cast<int64_t>(p.G), p.B - gi * p.G) * Tp) : 0u;
 
       float x[XS];
       float alpha_in;
@@ -1502,8 +1497,6 @@ __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) ae
             const int grp = static_cast<int>(task >> 3), e = static_cast<int>(task & 7u);
             const int ring = e < p.h_first ? 0 : 1;
             const uint4 gi = reinterpret_cast<const uint4 *>(splan + p.off_grp)[grp];
-            if constexpr (kSkipDead)
-              if (gi.z >= live_rows) continue;  // a word past the batch's end
             const bool act = lane < static_cast<int>(gi.y);
             const int row = static_cast<int>(gi.x) + (act ? lane : 0);
             // a lane past the group's rows computes on row 0 and its result is dropped; an all-ones

@@ -193,3 +193,25 @@ def test_word_alpha_of_more_words_than_warps(mode):
     dec.close()
     assert (logits.cpu().numpy().view(np.int32) == r["logits"].view(np.int32)).all()
     assert (bits.cpu().numpy() == r["bits"]).all() and (syn.cpu().numpy() == r["syndrome"]).all()
+
+
+# batches that leave SMs idle put fewer words into a CTA than it holds: the same outputs as in a batch that
+# fills every CTA, at the counts where the number of words changes
+@pytest.mark.gpu
+@pytest.mark.parametrize("d", [32, 64])
+@pytest.mark.parametrize("n,m,weight,alpha", [(31, 15, 3, 0), (18, 14, 2, 1), (7, 3, 2, 0), (5, 2, 1, 1), (40, 20, 2, 0)])
+def test_fewer_words_per_cta_equal_a_full_batch(n, m, weight, alpha, d):
+    model = I.random_model(random_code(n, m, weight, n + d), d, 2, seed=n, spe_noise=True)
+    model.alpha_mode = alpha
+    dec = A.Decoder(model, attention_mode=2)
+    G, sms = dec.query()["words_per_group"], torch.cuda.get_device_properties(0).multi_processor_count
+    rng = np.random.Generator(np.random.PCG64(n))
+    y = torch.from_numpy(rng.standard_normal((2 * G * sms + 1, n)).astype(np.float32)).cuda()
+    full = [t.clone() for t in dec.decode(y)]
+    for B in sorted({1, 2, sms - 1, sms, sms + 1, 2 * sms + 1, (G - 1) * sms, (G - 1) * sms + 1, G * sms - 1, G * sms}):
+        if B == 0:
+            continue
+        got = dec.decode(y[:B].contiguous())
+        assert all(torch.equal(a[:B].view(torch.uint8), b.view(torch.uint8)) for a, b in zip(full, got)), B
+    assert dec.synchronize() == A.AECCT_OK
+    dec.close()
