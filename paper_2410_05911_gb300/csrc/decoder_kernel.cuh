@@ -1,7 +1,8 @@
 // decoder_kernel.cuh -- the fused AECCT forward pass for sm_103a (kernel template; its
 // instantiations live in decoder_kernel.cu (ReLU, AAP linears), decoder_kernel_gelu.cu (GELU),
-// decoder_kernel_fp.cu and decoder_kernel_fp_gelu.cu (full-precision bf16 linears), translation
-// units that compile in parallel).
+// decoder_kernel_fp.cu and decoder_kernel_fp_gelu.cu (full-precision bf16 linears), and in
+// decoder_kernel_cap.cu and decoder_kernel_cap_fp.cu (warp tasks with the integer-core capture),
+// translation units that compile in parallel).
 //
 // One persistent kernel decodes the whole batch.  A cluster of C CTAs owns a group of G
 // codewords whose T = 2n-k tokens are packed back to back over the cluster's C x 128 token
@@ -12,8 +13,9 @@
 //   S3-S8  (Sec. 4.1, 4.2, 5) per block:
 //          Quant(x) -> tcgen05.mma QKV (bf16 operands holding exact int8 / ternary values,
 //          fp32 accumulators in TMEM, exact integers) -> dequant -> K,V to shared memory
-//          -> HPSA (warp tasks over shared key lists, or per-row neighbour lists with
-//          distributed-shared-memory reads of peer CTAs) -> Quant(A) -> MMA O
+//          -> HPSA (warp tasks over shared key lists, or per-row neighbour lists over K and V
+//          rows staged head by head, or read in place from the CTAs of the cluster) -> Quant(A)
+//          -> MMA O
 //          -> dequant + residual + LayerNorm -> Quant -> MMA FFN1 -> dequant + ReLU/GELU ->
 //          Quant -> MMA FFN2 -> dequant + residual + LayerNorm
 //   S9/S10 (Sec. 3)        output head, hard decisions, syndrome of the decoded word
@@ -2052,7 +2054,10 @@ __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) ae
             if constexpr (D == 128) tmem_wait_st();
           } else {
             float umax = 0.0f;
-#pragma unroll
+            // the d = 64 tasks loop over their two chunks: less code and no spills (Polar(64,32) 44.43 -> 43.83
+            // ms); unrolled elsewhere (BCH(63,36) 483.0 ms, 487.2 in a loop; LDPC(384,192) 139.5, 141.0)
+            constexpr int kUnroll = D == 64 && ATT == 1 ? 1 : NCH;
+#pragma unroll kUnroll
             for (int ch = 0; ch < NCH; ++ch) {
               wait_chunk(ch);
               float u[CH];
