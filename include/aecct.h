@@ -68,7 +68,7 @@ typedef struct aecct_handle aecct_handle; /* opaque */
  *                 rows start on the first 32-row boundary after the variables);
  *                 3 = per-row neighbour lists over per-head staged rows (d = 128, at most 640
  *                 token rows per group and 256 keys per row): head by head, the group's K and V
- *                 rows are gathered from every CTA of the cluster into local shared memory, and
+ *                 rows are brought from every CTA of the cluster into local shared memory, and
  *                 4 lanes of a warp share a row's keys.  The default for d = 64 (where it cannot be
  *                 asked for) and d = 128 when a group spans more than one CTA.  Every mode computes
  *                 the same results bit for bit.
@@ -223,7 +223,7 @@ int aecct_aap_ternarize_list(const float *const *w_dev, int32_t n_tensors, const
 /* The spectral positional encoding of Sec. 4.3 computed on the GPU, in double precision: the table
  * aecct_create takes as `spe`.  Tanner graph of H (variables 0..n-1, checks n..n+m-1, m = n - k,
  * T = n + m <= 1024 nodes), Laplacian L = D - A, its eigenpairs (lambda_i, phi_i) in ascending order
- * (parallel Jacobi rotations) in the canonical basis (per cluster of eigenvalues within 1e-8 max(1,
+ * (tridiagonal form, bisection and inverse iteration) in the canonical basis (per cluster of eigenvalues within 1e-8 max(1,
  * |lambda|max) of each other: Gram-Schmidt of P e_0, P e_1, ... in node order, P the cluster's
  * projector, residuals of norm <= 1e-6 skipped; a simple eigenvalue's vector has a positive first
  * entry above 1e-6 in magnitude), then for every node j:

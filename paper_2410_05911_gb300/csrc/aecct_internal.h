@@ -160,7 +160,7 @@ struct DecodeParams {
   // offsets in place of row offsets, row offset * 4 d_h + kv_piece(row offset).
   const uint32_t *mask_info[2];
   const uint4 *mask_list[2];
-  // Task-mode attention plan (one CTA per group of codewords, d <= 64).  A task is one head for
+  // Task-mode attention plan (one CTA per group of codewords).  A task is one head for
   // a query group: up to 32 consecutive rows of one codeword, one per lane.  It walks the union of
   // its lanes' key sets (ascending token order) with per-lane membership bits.
   // The plan is one blob that every CTA copies into shared memory (after the SmemLayout regions)

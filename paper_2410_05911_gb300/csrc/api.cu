@@ -10,6 +10,7 @@
 #include <cstdlib>
 #include <algorithm>
 #include <cstring>
+#include <new>
 #include <string>
 #include <vector>
 
@@ -202,13 +203,13 @@ int schedule_chunks(int D, ChunkDesc *out) {
 
 // ---- warp-task attention plan: which warp runs which task
 // A task (one head for one query group) costs the length of its union key list + 4 (its fixed
-// part).  Warps w with the same w % 4 issue from one scheduler and share its issue slots.  Measured
-// on the GPU: a warp alone issues at about 0.36 of a scheduler's rate (its own dependency chains
-// limit it) and about three warps saturate a scheduler, so four warps with unequal loads leave a
-// tail where one warp runs alone (Polar(64,32): its tasks on three warps per scheduler decode 2.2%
-// faster than on four; BCH(63,36)'s on two warps per lane quadrant instead of four make the
-// attention 1.38x slower).  A scheduler's time is modelled in phases: while k of its warps have
-// work left, each advances at min(1, k s) / k.  The plan minimises the largest modelled time.
+// part).  Warps w with the same w % 4 issue from one scheduler and share its issue slots.  A scheduler's
+// time is modelled in phases: while k of its warps have work left, each advances at min(1, k s) / k, with
+// s = kWarpIssueShare.  The plan minimises the largest modelled time.  s was measured with a branch per key
+// in the walk (Polar(64,32): its tasks on three warps per scheduler decoded 2.2% faster than on four with
+// unequal loads, whose tail leaves one warp alone).  The branch-free walk of 63 keys at d_h = 16 runs at
+// 0.66, 0.85, 0.97 and 1 of four warps' rate on one, two, three and four warps (117, 90, 79 and 77 cycles a
+// key step); with these rates the plans of Polar(64,32) and BCH(63,36) are still the best or equal to it.
 constexpr double kWarpIssueShare = 0.36;
 
 double scheduler_time(std::vector<long> loads) {
@@ -1230,7 +1231,12 @@ int aecct_aap_ternarize(const float *w_dev, int32_t n_tensors, const int64_t *le
                         float eps, uint8_t *packed_dev, float *scale_dev, float *wq_dev, void *cuda_stream) {
   if (n_tensors < 0 || (n_tensors > 0 && (!w_dev || !len_host))) return AECCT_ERR_INVALID_ARG;
   // the tensors back to back
-  std::vector<const float *> w(static_cast<size_t>(n_tensors));
+  std::vector<const float *> w;
+  try {
+    w.resize(static_cast<size_t>(n_tensors));
+  } catch (const std::bad_alloc &) {
+    return AECCT_ERR_OUT_OF_MEMORY;
+  }
   for (int j = 0; j < n_tensors; ++j) {
     if (len_host[j] < 4 || len_host[j] % 4 != 0 || len_host[j] > (int64_t(1) << 31)) return AECCT_ERR_INVALID_ARG;
     w[j] = j == 0 ? w_dev : w[j - 1] + len_host[j - 1];

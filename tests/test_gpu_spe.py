@@ -1,4 +1,4 @@
-"""The spectral positional encoding of Sec. 4.3 computed on the GPU (aecct_spe_table: parallel Jacobi
+"""The spectral positional encoding of Sec. 4.3 computed on the GPU (aecct_spe_table: tridiagonal
 eigensolver in double precision, canonical eigenbasis, multi-head self-attention over the eigen-tokens,
 average pooling) against the oracle's restatement (oracle/spe_oracle.c: cyclic Jacobi, the
 definition step by step) and the package's host precompute, on every code of the workloads."""
