@@ -271,6 +271,7 @@ cudaError_t launch_decode(const DecodeParams &p, cudaStream_t stream);
 template <int D, int ATT, int ACT, int LIN, int CAP>
 cudaError_t prepare_decode_kernel(int cluster_ctas, uint32_t plan_bytes, int *max_active_clusters);
 constexpr uint32_t kMaxDynSmem = 232448;  // the largest dynamic shared memory a CTA may opt into (227 KB)
+constexpr uint32_t kSmemPerSm = 233472;   // shared memory of an SM (228 KB)
 constexpr int kStagedMaxRows = 640;  // staged attention: rows of a group (64 bytes of K and of V each, 40 KB + 40 KB)
 constexpr int kStagedMaxKeys = 256;  // staged attention: keys per row (TMEM columns [128, 384))
 

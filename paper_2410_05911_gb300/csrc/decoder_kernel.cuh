@@ -2218,55 +2218,46 @@ __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) ae
   }
 }
 
+// A launch of clusters of `ctas` CTAs.  What a launch needs goes with the launch: a kernel's function attributes are
+// shared by every handle of the process that uses it, and their plans differ in size.
+struct ClusterLaunch {
+  cudaLaunchAttribute attr[2];
+  cudaLaunchConfig_t cfg;
+  ClusterLaunch(int clusters, int ctas, uint32_t smem, int ctas_per_sm, cudaStream_t stream) : attr{}, cfg{} {
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = ctas;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    // ask for the smallest shared-memory carve-out that holds the SM's CTAs (1 KB for each is
+    // reserved by the system): the rest of the 256 KB unified array stays L1 for spills and parameter loads
+    const uint32_t pct = (100u * static_cast<uint32_t>(ctas_per_sm) * (smem + 1024u) + kSmemPerSm - 1u) / kSmemPerSm;
+    attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    attr[1].val.sharedMemCarveout = pct > 100u ? 100u : pct;
+    cfg.gridDim = dim3(clusters * ctas, 1, 1);
+    cfg.blockDim = dim3(kThreads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+  }
+};
+
 template <int D, int ATT, int ACT, int LIN, int CAP>
 cudaError_t prepare_decode_kernel(int cluster_ctas, uint32_t plan_bytes, int *max_active_clusters) {
   using L = KernelLayout<D, ATT>;
-  const uint32_t total = L::kTotal + plan_bytes;
-  cudaError_t e = cudaFuncSetAttribute(aecct_decoder_kernel<D, ATT, ACT, LIN, CAP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(total));
+  // the device's limit, whatever this handle needs: a smaller value would stop another handle's launches
+  const cudaError_t e = cudaFuncSetAttribute(aecct_decoder_kernel<D, ATT, ACT, LIN, CAP>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMaxDynSmem));
   if (e != cudaSuccess) return e;
-  // ask for the smallest shared-memory carve-out that holds the SM's CTAs (1 KB for each is
-  // reserved by the system): the rest of the 256 KB unified array stays L1 for spills and parameter loads
-  int dev = 0, smem_sm = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev)) != cudaSuccess)
-    return e;
-  if (smem_sm > 0) {
-    const int pct = static_cast<int>((100ll * L::kCtasPerSm * (total + 1024) + smem_sm - 1) / smem_sm);
-    e = cudaFuncSetAttribute(aecct_decoder_kernel<D, ATT, ACT, LIN, CAP>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             pct > 100 ? 100 : pct);
-    if (e != cudaSuccess) return e;
-  }
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cluster_ctas;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(cluster_ctas, 1, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = total;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaOccupancyMaxActiveClusters(max_active_clusters, aecct_decoder_kernel<D, ATT, ACT, LIN, CAP>, &cfg);
+  const ClusterLaunch l(1, cluster_ctas, L::kTotal + plan_bytes, L::kCtasPerSm, nullptr);
+  return cudaOccupancyMaxActiveClusters(max_active_clusters, aecct_decoder_kernel<D, ATT, ACT, LIN, CAP>, &l.cfg);
 }
 
 template <int D, int ATT, int ACT, int LIN, int CAP>
 cudaError_t launch_decode(const DecodeParams &p, cudaStream_t stream) {
   using L = KernelLayout<D, ATT>;
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = p.C;
-  attr[0].val.clusterDim.y = 1;
-  attr[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3(p.n_clusters * p.C, 1, 1);
-  cfg.blockDim = dim3(kThreads, 1, 1);
-  cfg.dynamicSmemBytes = L::kTotal + p.plan_bytes;
-  cfg.stream = stream;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, aecct_decoder_kernel<D, ATT, ACT, LIN, CAP>, p);
+  const ClusterLaunch l(p.n_clusters, p.C, L::kTotal + p.plan_bytes, L::kCtasPerSm, stream);
+  return cudaLaunchKernelEx(&l.cfg, aecct_decoder_kernel<D, ATT, ACT, LIN, CAP>, p);
 }
 
 }  // namespace aecct
