@@ -945,6 +945,17 @@ __global__ void __launch_bounds__(576) mhsa_kernel(const double *lam, const doub
   }
 }
 
+// Lets launches of `kernel` ask for all the shared memory that the device has.  The attribute belongs to the process: set
+// to one graph's need it would stop the launches of a call with a larger graph on another thread.
+template <typename... Args>
+cudaError_t allow_shared(void (*kernel)(Args...)) {
+  cudaFuncAttributes a;
+  const cudaError_t e = cudaFuncGetAttributes(&a, kernel);
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(kMaxDynSmem - a.sharedSizeBytes));
+}
+
 // one Cholesky QR of the clusters larger than rmin
 void chol_qr(double *V, double *Gm, const int *gs, const int *gn, int T, int rmin, int coords, double thr, int *bad) {
   const int nt = (T + 31) / 32;
@@ -1022,7 +1033,7 @@ cudaError_t run_spe_table(const uint8_t *H, int n, int m, int d_spe, int heads, 
   R = (T + G - 1) / G;
   {
     const size_t smem = sizeof(double) * T * (3 + static_cast<size_t>(R));
-    if (!ok(cudaFuncSetAttribute(tridiag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem))) ||
+    if (!ok(allow_shared(tridiag_kernel)) ||
         !ok(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, tridiag_kernel, kTriThreads, smem)))
       goto done;
     if (per_sm < 1) {
@@ -1037,9 +1048,7 @@ cudaError_t run_spe_table(const uint8_t *H, int n, int m, int d_spe, int heads, 
   }
   bisect_kernel<<<T, 32, sizeof(double2) * T>>>(d, ed, T, lam);
   group_kernel<<<1, kSpeMaxTokens>>>(lam, T, cluster_tol, gs, gn);
-  if (!ok(cudaFuncSetAttribute(chol_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kCholSmem))) ||
-      !ok(cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kCholSmem))))
-    goto done;
+  if (!ok(allow_shared(chol_kernel)) || !ok(allow_shared(select_kernel))) goto done;
   {
     // inverse iteration, vectors of a CTA bounded by the shared memory of their factors; another seed where
     // a cluster's random vectors came out dependent
@@ -1049,8 +1058,7 @@ cudaError_t run_spe_table(const uint8_t *H, int n, int m, int d_spe, int heads, 
     const int want = (T + sms - 1) / sms;  // no more to a CTA than fills the SMs
     nv = nv > want ? want : nv;
     const size_t smem = per_vec * nv;
-    if (!ok(cudaFuncSetAttribute(invit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem))))
-      goto done;
+    if (!ok(allow_shared(invit_kernel))) goto done;
     for (uint32_t attempt = 0;; ++attempt) {
       if (!ok(cudaMemset(badd, 0, sizeof(int) * 2 * T))) goto done;
       invit_kernel<<<(T + nv - 1) / nv, 32, smem>>>(d, ed, lam, gn, T, nv, 12345u + 977u * attempt, X);
@@ -1087,8 +1095,7 @@ cudaError_t run_spe_table(const uint8_t *H, int n, int m, int d_spe, int heads, 
   {
     const size_t smem = static_cast<size_t>(T) * (2 * sizeof(double) + sizeof(FixKey) + sizeof(float2)) + kFixTable * sizeof(uint64_t);
     const int passes = (T + 575) / 576, threads = ((T + passes - 1) / passes + 31) / 32 * 32;  // rows per pass
-    if (!ok(cudaFuncSetAttribute(mhsa_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem))))
-      goto done;
+    if (!ok(allow_shared(mhsa_kernel))) goto done;
     uint64_t *exp_table = reinterpret_cast<uint64_t *>(base + o_exp);
     exp_table_kernel<<<kFixTable / 256, 256>>>(exp_table);
     mhsa_kernel<<<T, threads, smem>>>(lam, U, T, heads, coef, dp(o_va), dp(o_vb), dp(o_wo), exp_table, d_spe, spe,
