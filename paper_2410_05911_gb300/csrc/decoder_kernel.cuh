@@ -460,51 +460,21 @@ __device__ __forceinline__ bool contiguous(const uint4 &w) {
   return w.x == pat && w.y == pat + 0x04040404u && w.z == pat + 0x08080808u && w.w == pat + 0x0C0C0C0Cu;
 }
 
-// The same head where a V row of the CTA is not finite (parameters near the end of the fp32 range): a
-// lane folds in its own keys only, so that an infinity stays with the queries that attend to it.  q
-// comes in and A goes out in `qa`.
-template <int DH, uint32_t STRIDE>
-static __device__ __noinline__ void hpsa_task_any(float *qa, const uint4 mask, int cnt, const uint4 *ul,
-                                                  const uint8_t *rows, uint32_t kslot, float scale) {
-  const uint8_t *row = reinterpret_cast<const uint8_t *>(ul);
-  auto member = [&](int k) {
-    const uint32_t word = k < 64 ? (k < 32 ? mask.x : mask.y) : (k < 96 ? mask.z : mask.w);
-    return ((word >> (k & 31)) & 1u) != 0u;
-  };
-  auto score = [&](int k) {
-    const float *kk = reinterpret_cast<const float *>(rows + row[k] * STRIDE + kslot);
-    float d0 = 0.0f, d1 = 0.0f;
-    for (int i = 0; i < DH; i += 2) d0 = __fmaf_rn(qa[i], kk[i], d0), d1 = __fmaf_rn(qa[i + 1], kk[i + 1], d1);
-    return __fmul_rn(__fadd_rn(d0, d1), scale);
-  };
-  float mx = -INFINITY, lsum = 0.0f, num[DH];
-  for (int i = 0; i < DH; ++i) num[i] = 0.0f;
-  for (int k = 0; k < cnt; ++k)
-    if (member(k)) mx = fmaxf(mx, score(k));
-  for (int k = 0; k < cnt; ++k) {
-    if (!member(k)) continue;
-    const float pr = exp2_series(__fsub_rn(score(k), mx));
-    const float *vv = reinterpret_cast<const float *>(rows + row[k] * STRIDE + kslot) + DH;
-    lsum = __fadd_rn(lsum, pr);
-    for (int i = 0; i < DH; ++i) num[i] = __fmaf_rn(pr, vv[i], num[i]);
-  }
-  const float inv = __fdiv_rn(1.0f, lsum);
-  for (int i = 0; i < DH; ++i) qa[i] = __fmul_rn(num[i], inv);
-}
-
 // One HPSA head for a query group (task mode).  Every lane walks the group's union key list in
 // ascending token order; the loads are warp-uniform (shared-memory broadcasts).  A key that is not
 // in the lane's own set (membership bit) gets the score -inf and so, exactly, the probability 0:
 // it changes neither the maximum nor l nor num (x + 0 and fma(0, v, x) are x for finite v), and for
 // each query the max, the sum l and the weighted sum num see its keys in ascending order, as in
-// the canonical definition, without a branch per key.  V has to be finite (the caller checks).
+// the canonical definition, without a branch per key.  V has to be finite; where a V row of the CTA is not
+// (a word with a NaN, parameters near the end of the fp32 range), OWN = 1: a branch around every fold, so
+// that an infinity stays with the queries that attend to it.
 // Keys go U at a time; the two lanes of a paired instruction are independent computations, and the
 // folds into l and num stay sequential in key order.
 // Bound by issue slots, FMA pipe and shared-memory loads at 50 to 70% each.  With a divergent branch
 // around every maximum and fold, a key step of three warps a scheduler took 93.8 cycles at d_h = 16
 // (63 keys) and 64 at d_h = 4 (15 keys), now 79 and 48; U = 2 in place of 4 at d_h = 16: 82.
 // BCH(63,36) 546.8 -> 496.6 ms for 262,144 words, Polar(64,32) 46.7 -> 45.5 ms for 65,536.
-template <int DH, uint32_t STRIDE, int CACHE>
+template <int DH, uint32_t STRIDE, int CACHE, int OWN>
 __device__ __forceinline__ void hpsa_task(const float *q, const uint4 mask, int cnt, const uint4 *ul,
                                           const uint8_t *rows, uint32_t kslot, float scale, uint32_t tcache,
                                           float *A) {
@@ -597,6 +567,7 @@ __device__ __forceinline__ void hpsa_task(const float *q, const uint4 mask, int 
   for (int jb = 0; jb < cnt; jb += 16) {
     const uint4 w = ul[jb >> 4];
     const int nk = cnt - jb;
+    const uint32_t seg = segment(jb);
     if (jb < CACHE) {
       float sgs[16];
       tmem_ld<16>(tcache + jb, sgs);
@@ -619,14 +590,16 @@ __device__ __forceinline__ void hpsa_task(const float *q, const uint4 mask, int 
               // sigma - m for two keys: one paired add of -m (the cached scores are not products)
               pr[k / 2] = exp2_series2(add2(make_float2(sgs[k0 + k], sgs[k0 + k + 1]), make_float2(-mx, -mx)));
 #pragma unroll
-            for (int k = 0; k < U; k += 2) fold(pr[k / 2].x, vv[k]), fold(pr[k / 2].y, vv[k + 1]);
+            for (int k = 0; k < U; k += 2) {
+              if (!OWN || ((seg >> (k0 + k)) & 1u)) fold(pr[k / 2].x, vv[k]);
+              if (!OWN || ((seg >> (k0 + k + 1)) & 1u)) fold(pr[k / 2].y, vv[k + 1]);
+            }
           }
         }
       };
       if (contiguous(w)) block(std::true_type{});
       else block(std::false_type{});
     } else {
-      const uint32_t seg = segment(jb);
 #pragma unroll
       for (int k0 = 0; k0 < 16; k0 += U) {
         if (k0 < nk) {
@@ -639,7 +612,8 @@ __device__ __forceinline__ void hpsa_task(const float *q, const uint4 mask, int 
             const float4 *pa = kptr(byte_at(w, k0 + k)), *pb = kptr(byte_at(w, k0 + k + 1));
 #pragma unroll
             for (int i = 0; i < DH / 4; ++i) va[i] = pa[DH / 4 + i], vb[i] = pb[DH / 4 + i];
-            fold(pr.x, va), fold(pr.y, vb);
+            if (!OWN || ((seg >> (k0 + k)) & 1u)) fold(pr.x, va);
+            if (!OWN || ((seg >> (k0 + k + 1)) & 1u)) fold(pr.y, vb);
           }
         }
       }
@@ -1492,76 +1466,74 @@ __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) ae
           // a warp of its group's quadrant); Q comes from the QKV accumulators of this thread's row
           // and the output goes back over them
           const uint32_t tcache = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + L::task_cache_col(warp >> 2);
-          const bool vbad = *s_vbad != 0;
-          for (int k = 0; k < kMaxTasks; ++k) {
-            const uint32_t task = reinterpret_cast<const uint16_t *>(splan + p.off_task)[warp * kMaxTasks + k];
-            if (task == 0xFFFFu) break;
-            const int grp = static_cast<int>(task >> 3), e = static_cast<int>(task & 7u);
-            const int ring = e < p.h_first ? 0 : 1;
-            const uint4 gi = reinterpret_cast<const uint4 *>(splan + p.off_grp)[grp];
-            const bool act = lane < static_cast<int>(gi.y);
-            const int row = static_cast<int>(gi.x) + (act ? lane : 0);
-            // a lane past the group's rows computes on row 0 and its result is dropped; an all-ones
-            // mask keeps it from breaking the dense fast path
-            const uint4 mk = act ? reinterpret_cast<const uint4 *>(splan + p.off_mask)[(grp * 2 + ring) * 32 + lane]
-                                 : make_uint4(~0u, ~0u, ~0u, ~0u);
-            const uint32_t ui = reinterpret_cast<const uint32_t *>(splan + p.off_uinfo)[grp * 2 + ring];
-            float q[DH], a[DH];
-            // d = 128: a task off its rows' quadrant has Q and A in a W2 slot (row = lane)
-            const uint32_t qs = L::kQInSmem ? 0xFFu : qtab[4 + grp * 8 + e];
-            if constexpr (L::kQInSmem) {
-              const float4 *qp = reinterpret_cast<const float4 *>(smem + L::kOffU + row * L::kKvStride + e * L::kSlot);
+          auto run_tasks = [&](auto own_tag) {
+            for (int k = 0; k < kMaxTasks; ++k) {
+              const uint32_t task = reinterpret_cast<const uint16_t *>(splan + p.off_task)[warp * kMaxTasks + k];
+              if (task == 0xFFFFu) break;
+              const int grp = static_cast<int>(task >> 3), e = static_cast<int>(task & 7u);
+              const int ring = e < p.h_first ? 0 : 1;
+              const uint4 gi = reinterpret_cast<const uint4 *>(splan + p.off_grp)[grp];
+              const bool act = lane < static_cast<int>(gi.y);
+              const int row = static_cast<int>(gi.x) + (act ? lane : 0);
+              // a lane past the group's rows computes on row 0 and its result is dropped; an all-ones
+              // mask keeps it from breaking the dense fast path
+              const uint4 mk = act ? reinterpret_cast<const uint4 *>(splan + p.off_mask)[(grp * 2 + ring) * 32 + lane]
+                                   : make_uint4(~0u, ~0u, ~0u, ~0u);
+              const uint32_t ui = reinterpret_cast<const uint32_t *>(splan + p.off_uinfo)[grp * 2 + ring];
+              float q[DH], a[DH];
+              // d = 128: a task off its rows' quadrant has Q and A in a W2 slot (row = lane)
+              const uint32_t qs = L::kQInSmem ? 0xFFu : qtab[4 + grp * 8 + e];
+              if constexpr (L::kQInSmem) {
+                const float4 *qp = reinterpret_cast<const float4 *>(smem + L::kOffU + row * L::kKvStride + e * L::kSlot);
 #pragma unroll
-              for (int i = 0; i < DH / 4; ++i) {
-                const float4 v = qp[i];
-                q[4 * i] = v.x, q[4 * i + 1] = v.y, q[4 * i + 2] = v.z, q[4 * i + 3] = v.w;
+                for (int i = 0; i < DH / 4; ++i) {
+                  const float4 v = qp[i];
+                  q[4 * i] = v.x, q[4 * i + 1] = v.y, q[4 * i + 2] = v.z, q[4 * i + 3] = v.w;
+                }
+              } else if (qs != 0xFFu) {
+#pragma unroll
+                for (int f = 0; f < DH / 4; ++f) {
+                  const float4 v = ld_shared_f4(qslot_piece(qs, lane, f));
+                  q[4 * f] = v.x, q[4 * f + 1] = v.y, q[4 * f + 2] = v.z, q[4 * f + 3] = v.w;
+                }
+              } else {
+                float qa[DH], bq[DH];
+                ldg_vec<DH>(lp + LP::bqkv(D) + e * DH, bq);
+                tmem_ld<DH>(tl + e * DH, qa);
+                tmem_wait_ld();
+                if (cap) capture_acc(l, 0, qa, e * DH, DH);
+                dequant<DH>(qa, fq, bq, q);
               }
-            } else if (qs != 0xFFu) {
+              const uint4 *ul = reinterpret_cast<const uint4 *>(splan + p.off_ulist) + (ui >> 8);
+              const uint8_t *krows = smem + L::kOffU + gi.z * L::kKvStride;
+              const uint32_t kslot = e * L::kSlot + (L::kQInSmem ? 4 * DH : 0);
+              hpsa_task<DH, L::kKvStride, L::kTaskCache, decltype(own_tag)::value>(
+                  q, mk, static_cast<int>(ui & 255u), ul, krows, kslot, p.att_scale, tcache, a);
+              if constexpr (L::kQInSmem) {
+                if (act) {
+                  // A of (row, head e) replaces Q of (row, head e): this task was its only reader
+                  float4 *ap = reinterpret_cast<float4 *>(smem + L::kOffU + row * L::kKvStride + e * L::kSlot);
 #pragma unroll
-              for (int f = 0; f < DH / 4; ++f) {
-                const float4 v = ld_shared_f4(qslot_piece(qs, lane, f));
-                q[4 * f] = v.x, q[4 * f + 1] = v.y, q[4 * f + 2] = v.z, q[4 * f + 3] = v.w;
+                  for (int i = 0; i < DH / 4; ++i) ap[i] = make_float4(a[4 * i], a[4 * i + 1], a[4 * i + 2], a[4 * i + 3]);
+                }
+              } else if (qs != 0xFFu) {
+                // A of (row, head e) over its Q in the slot (this task was its only reader)
+#pragma unroll
+                for (int f = 0; f < DH / 4; ++f) st_shared_f4(qslot_piece(qs, lane, f), a[4 * f], a[4 * f + 1], a[4 * f + 2], a[4 * f + 3]);
+              } else {
+                // every lane's own row: A of (row, head e) over the head's Q accumulators (a lane past
+                // the group's rows writes a padding or empty row, which nothing reads)
+                tmem_st<DH>(tl + e * DH, a);
               }
-            } else {
-              float qa[DH], bq[DH];
-              ldg_vec<DH>(lp + LP::bqkv(D) + e * DH, bq);
-              tmem_ld<DH>(tl + e * DH, qa);
-              tmem_wait_ld();
-              if (cap) capture_acc(l, 0, qa, e * DH, DH);
-              dequant<DH>(qa, fq, bq, q);
+              __syncwarp();
             }
-            const uint4 *ul = reinterpret_cast<const uint4 *>(splan + p.off_ulist) + (ui >> 8);
-            const uint8_t *krows = smem + L::kOffU + gi.z * L::kKvStride;
-            const uint32_t kslot = e * L::kSlot + (L::kQInSmem ? 4 * DH : 0);
-            if (!vbad) {
-              hpsa_task<DH, L::kKvStride, L::kTaskCache>(q, mk, static_cast<int>(ui & 255u), ul, krows, kslot,
-                                                         p.att_scale, tcache, a);
-            } else {
-              float qa[DH];
-#pragma unroll
-              for (int i = 0; i < DH; ++i) qa[i] = q[i];
-              hpsa_task_any<DH, L::kKvStride>(qa, mk, static_cast<int>(ui & 255u), ul, krows, kslot, p.att_scale);
-#pragma unroll
-              for (int i = 0; i < DH; ++i) a[i] = qa[i];
-            }
-            if constexpr (L::kQInSmem) {
-              if (act) {
-                // A of (row, head e) replaces Q of (row, head e): this task was its only reader
-                float4 *ap = reinterpret_cast<float4 *>(smem + L::kOffU + row * L::kKvStride + e * L::kSlot);
-#pragma unroll
-                for (int i = 0; i < DH / 4; ++i) ap[i] = make_float4(a[4 * i], a[4 * i + 1], a[4 * i + 2], a[4 * i + 3]);
-              }
-            } else if (qs != 0xFFu) {
-              // A of (row, head e) over its Q in the slot (this task was its only reader)
-#pragma unroll
-              for (int f = 0; f < DH / 4; ++f) st_shared_f4(qslot_piece(qs, lane, f), a[4 * f], a[4 * f + 1], a[4 * f + 2], a[4 * f + 3]);
-            } else {
-              // every lane's own row: A of (row, head e) over the head's Q accumulators (a lane past
-              // the group's rows writes a padding or empty row, which nothing reads)
-              tmem_st<DH>(tl + e * DH, a);
-            }
-            __syncwarp();
-          }
+          };
+          // V rows that are not finite take a second copy of the loop.  4,096 words of Polar(64,32) (three blocks),
+          // a NaN in each: 1.49 ms, 1.44 without the NaN; 2.96 in a walk key by key.  The copy costs the words
+          // of the first one 0.9% at d = 64 (Polar(64,32) 43.8 -> 44.2 ms) and nothing at d = 32 and 128; a
+          // call out of line from the loop 2.1%, a test around the second pass alone 1.2%.
+          if (*s_vbad == 0) run_tasks(std::integral_constant<int, 0>{});
+          else run_tasks(std::integral_constant<int, 1>{});
           if constexpr (!L::kQInSmem) {
             tmem_wait_st();
             tc_fence_before();  // the TMEM stores are ordered before the barrier for the row owners
