@@ -226,7 +226,8 @@ int aecct_aap_ternarize_list(const float *const *w_dev, int32_t n_tensors, const
  * (tridiagonal form, bisection and inverse iteration) in the canonical basis (per cluster of eigenvalues within 1e-8 max(1,
  * |lambda|max) of each other: Gram-Schmidt of P e_0, P e_1, ... in node order, P the cluster's
  * projector, residuals of norm <= 1e-6 skipped; a simple eigenvalue's vector has a positive first
- * entry above 1e-6 in magnitude), then for every node j:
+ * entry above 1e-6 in magnitude; the vectors are orthonormal to rounding also where eigenvalues lie close
+ * without being in a cluster), then for every node j:
  *   X_j = Phi_j W_pe, Phi_j row i = (lambda_i, phi_i[j]);
  *   MHSA(X_j) = [softmax((X_j Wq_e)(X_j Wk_e)^T / sqrt(d_e)) (X_j Wv_e)]_e Wo, d_e = d_spe / heads;
  *   SPE_j = the mean of the T rows of MHSA(X_j) (average pooling as the reduction W_{(2n-k)->1}).

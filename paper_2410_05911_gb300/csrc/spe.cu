@@ -14,6 +14,9 @@
 //                     an orthonormal basis of each cluster's subspace: V <- L^-1 V with V V^T = L L^T,
 //                     twice (Cholesky QR, whose second round leaves the orthogonality of a Householder
 //                     factorisation).
+//   overlap_kernel, polish_kernel
+//                     X <- X - (X X^T - I) X / 2: vectors of neighbouring eigenvalues come out of the
+//                     inverse iteration orthogonal to eps |L| / gap only.
 //   back_kernel       the reflections applied to the eigenvectors.
 //   canonical_kernel  per cluster, the canonical basis: Gram-Schmidt of P e_0, P e_1, ... in node
 //                     order, P the cluster's projector, skipping residuals of norm <= vanish_tol; in the
@@ -29,7 +32,7 @@
 //
 // The long code of 576 nodes (LDPC(384,192)), where Jacobi rotations (about 10 sweeps of 575 steps with
 // three grid-wide barriers each) and Gram-Schmidt in node coordinates took 327 ms: tridiagonal form 3.9 ms,
-// eigenvalues 0.9, inverse iteration 0.8, the clusters' bases 2.2, reflections 1.4, canonical basis 2.6;
+// eigenvalues 0.9, inverse iteration 0.8, the clusters' bases 2.2, polishing 0.6, reflections 1.4, canonical basis 2.6;
 // the attention 3.8 (41 with double operations).
 #include <algorithm>
 #include <cmath>
@@ -637,6 +640,78 @@ __global__ void __launch_bounds__(256) trsm_kernel(const double *__restrict__ Gm
   }
 }
 
+// E = X X^T - I (32 x 32 tiles, the lower ones computed) and, per tile, whether an entry of it exceeds kOverlapSkip.
+// Inverse iteration leaves vectors of eigenvalues a gap apart with a product of about eps |L| / gap (9e-12 for
+// Polar(64,32), whose closest ones are 5e-6 apart), which nothing after it removes.  `again` is set where
+// an entry is so large that its square is not yet rounding; with `go` null or set the tiles are computed.
+constexpr double kOverlapSkip = 4.0 * kEps, kOverlapAgain = 1e-9;
+__global__ void __launch_bounds__(256) overlap_kernel(const double *__restrict__ X, int T, const int *go, double *E, int *busy,
+                                                     int *again) {
+  __shared__ double sa[32][33], sb[32][33];
+  const int a0 = blockIdx.y * 32, b0 = blockIdx.x * 32, tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  if (b0 > a0 || (go && !*go)) return;
+  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+  for (int c0 = 0; c0 < T; c0 += 32) {
+    for (int it = threadIdx.x; it < 1024; it += 256) {
+      const int rr = it >> 5, c = c0 + (it & 31);
+      sa[rr][it & 31] = a0 + rr < T && c < T ? X[static_cast<size_t>(a0 + rr) * T + c] : 0.0;
+      sb[rr][it & 31] = b0 + rr < T && c < T ? X[static_cast<size_t>(b0 + rr) * T + c] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int c = 0; c < 32; ++c) {
+      const double x0 = sa[ty][c], x1 = sa[ty + 16][c], y0 = sb[tx][c], y1 = sb[tx + 16][c];
+      acc[0][0] = fma(x0, y0, acc[0][0]), acc[0][1] = fma(x0, y1, acc[0][1]);
+      acc[1][0] = fma(x1, y0, acc[1][0]), acc[1][1] = fma(x1, y1, acc[1][1]);
+    }
+    __syncthreads();
+  }
+  double top = 0.0;
+  for (int i = 0; i < 2; ++i)
+    for (int j = 0; j < 2; ++j) {
+      const int a = a0 + ty + 16 * i, b = b0 + tx + 16 * j;
+      if (a >= T || b > a) continue;
+      const double e = acc[i][j] - (a == b ? 1.0 : 0.0);
+      E[static_cast<size_t>(a) * T + b] = E[static_cast<size_t>(b) * T + a] = e;
+      top = fmax(top, fabs(e));
+    }
+  const int some = __syncthreads_or(top > kOverlapSkip), much = __syncthreads_or(top > kOverlapAgain);
+  if (threadIdx.x == 0) {
+    busy[blockIdx.y * gridDim.x + blockIdx.x] = busy[blockIdx.x * gridDim.x + blockIdx.y] = some;
+    if (much) *again = 1;
+  }
+}
+
+// Y = X - E X / 2, from the tiles of E that are marked (all of them as they are with `go` unset)
+__global__ void __launch_bounds__(256) polish_kernel(const double *__restrict__ X, const double *__restrict__ E,
+                                                    const int *__restrict__ busy, int T, const int *go, double *Y) {
+  __shared__ double se[32][33], sx[32][33];
+  const int a0 = blockIdx.y * 32, c0 = blockIdx.x * 32, tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+  const bool on = !go || *go;
+  for (int b0 = 0; on && b0 < T; b0 += 32) {
+    if (!busy[blockIdx.y * gridDim.y + b0 / 32]) continue;
+    for (int it = threadIdx.x; it < 1024; it += 256) {
+      const int rr = it >> 5, u = it & 31;
+      se[rr][u] = a0 + rr < T && b0 + u < T ? E[static_cast<size_t>(a0 + rr) * T + b0 + u] : 0.0;
+      sx[rr][u] = b0 + rr < T && c0 + u < T ? X[static_cast<size_t>(b0 + rr) * T + c0 + u] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll 8
+    for (int b = 0; b < 32; ++b) {
+      const double x0 = se[ty][b], x1 = se[ty + 16][b], y0 = sx[b][tx], y1 = sx[b][tx + 16];
+      acc[0][0] = fma(x0, y0, acc[0][0]), acc[0][1] = fma(x0, y1, acc[0][1]);
+      acc[1][0] = fma(x1, y0, acc[1][0]), acc[1][1] = fma(x1, y1, acc[1][1]);
+    }
+    __syncthreads();
+  }
+  for (int i = 0; i < 2; ++i)
+    for (int j = 0; j < 2; ++j) {
+      const int a = a0 + ty + 16 * i, c = c0 + tx + 16 * j;
+      if (a < T && c < T) Y[static_cast<size_t>(a) * T + c] = fma(-0.5, acc[i][j], X[static_cast<size_t>(a) * T + c]);
+    }
+}
+
 // g[k] = v_k . v_{k-1} for the pairs of reflections that back_kernel applies together
 __global__ void __launch_bounds__(32) pair_kernel(const double *__restrict__ Vh, int T, double *g) {
   const int k = blockIdx.x + 1;
@@ -1004,7 +1079,7 @@ cudaError_t run_spe_table(const uint8_t *H, int n, int m, int d_spe, int heads, 
                o_wo = part(sizeof(double) * d_spe * d_spe), o_spe64 = part(sizeof(double) * T * d_spe),
                o_spe = part(sizeof(float) * T * d_spe), o_H = part(static_cast<size_t>(m) * n),
                o_gs = part(sizeof(int) * T), o_gn = part(sizeof(int) * T), o_bad = part(sizeof(int) * 2 * T),
-               o_node = part(sizeof(int) * T), o_exp = part(kFixTable * sizeof(uint64_t)), o_status = part(2 * sizeof(int));
+               o_node = part(sizeof(int) * T), o_busy = part(sizeof(int) * (32 * 32 + 1)), o_exp = part(kFixTable * sizeof(uint64_t)), o_status = part(2 * sizeof(int));
   uint8_t *base = nullptr;
   cudaError_t e = cudaSuccess;
   auto ok = [&](cudaError_t x) { return (e = x) == cudaSuccess; };
@@ -1018,6 +1093,7 @@ cudaError_t run_spe_table(const uint8_t *H, int n, int m, int d_spe, int heads, 
   uint8_t *Hd = base + o_H;
   int *gs = reinterpret_cast<int *>(base + o_gs), *gn = reinterpret_cast<int *>(base + o_gn),
       *badd = reinterpret_cast<int *>(base + o_bad), *node = reinterpret_cast<int *>(base + o_node),
+      *busy = reinterpret_cast<int *>(base + o_busy), *again = busy + 32 * 32,
       *dstatus = reinterpret_cast<int *>(base + o_status);
   unsigned *count = reinterpret_cast<unsigned *>(dstatus + 1);
   const int nt = (T + 31) / 32;
@@ -1076,6 +1152,13 @@ cudaError_t run_spe_table(const uint8_t *H, int n, int m, int d_spe, int heads, 
       }
     }
   }
+  // orthogonal vectors to rounding: one round, and a second where that left more (U is free until the end)
+  static_assert(kSpeMaxTokens <= 32 * 32, "a mark for every tile");
+  if (!ok(cudaMemset(again, 0, sizeof(int)))) goto done;
+  overlap_kernel<<<dim3(nt, nt), 256>>>(X, T, nullptr, Gm, busy, again);
+  polish_kernel<<<dim3(nt, nt), 256>>>(X, Gm, busy, T, nullptr, U);
+  overlap_kernel<<<dim3(nt, nt), 256>>>(U, T, again, Gm, busy, again);
+  polish_kernel<<<dim3(nt, nt), 256>>>(U, Gm, busy, T, again, X);
   if (T > 3) pair_kernel<<<T - 3, 32>>>(V, T, pbuf);  // (pbuf: the reduction is done with it)
   if (T <= 128) back_kernel<4><<<(T + 1) / 2, 64>>>(V, tau, pbuf, T, X);
   else if (T <= 320) back_kernel<10><<<(T + 1) / 2, 64>>>(V, tau, pbuf, T, X);

@@ -61,6 +61,24 @@ def test_eigenpairs_of_graph(name):
         assert np.abs(tab - ref).max() <= 1e-6 * (1 + np.abs(ref).max())
 
 
+# eigenvalues that lie close without being equal (5e-6 apart for Polar(64,32)): their vectors are orthogonal to
+# rounding, a few T eps, whatever the gap
+CLOSE = dict(GRAPHS, **{"polar": I.make_code("polar64_32").H, "bch63": I.make_code("bch63_36").H,
+                        "ldpc 192": I.make_code("ldpc128_64").H,
+                        "ninety hamming": np.kron(np.eye(90, dtype=np.uint8), I.make_code("hamming7_4").H)})
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("name", CLOSE)
+def test_eigenvectors_are_orthonormal(name):
+    H = CLOSE[name]
+    T = sum(H.shape)
+    _, _, lam, U = A.spe_table(H, I.spe_params(H, 8, seed=1), want_eigen=True)
+    assert np.abs(U.T @ U - np.eye(T)).max() <= 2 * EPS * T
+    L = spe.tanner_laplacian(H)
+    assert np.abs(L @ U - U * lam).max() <= 32 * EPS * lam[-1] * T
+
+
 @pytest.mark.gpu
 @pytest.mark.parametrize("scale", [1e-3, 1.0, 4.0, 8.0, 20.0, 40.0, 1e3])
 def test_table_over_score_ranges(scale):
