@@ -188,6 +188,28 @@ def check_outputs(out, B: int, n: int, m: int, device):
     return bits, syn, logits
 
 
+def _stream_of(stream, device, tensors):
+    """The stream that a call launches on: `stream`, or the current one.  The call's tensors belong to the
+    current stream (its work produces the inputs and copies of them, and its allocator hands out the
+    outputs), so another stream waits for what is queued there, and the tensors' memory is not handed out
+    again before that stream is done with them.  A stream under capture and one that is not cannot wait for
+    each other: there the order is the caller's."""
+    import torch
+
+    current = torch.cuda.current_stream(device)
+    if stream is None or stream.cuda_stream == current.cuda_stream:
+        return current
+    capturing = torch.cuda.is_current_stream_capturing()
+    with torch.cuda.stream(stream):
+        same = torch.cuda.is_current_stream_capturing() == capturing
+    if same:
+        stream.wait_stream(current)
+    for t in tensors:
+        if t is not None:
+            t.record_stream(stream)
+    return stream
+
+
 class Decoder:
     """A decoder handle on the current CUDA device.
 
@@ -329,7 +351,7 @@ def selftest_fma_rate(paired: bool) -> float:
 
 def aap_ternarize(tensors, delta=None, eps: float = 1e-8, want_weights: bool = False, stream=None):
     """aecct_aap_ternarize: eq. Ternary on the GPU for a list of float32 CUDA tensors (each with a
-    multiple of 4 elements).  Returns (packed uint8 codes per tensor, scales float32 [n], and the
+    multiple of 4 elements), on `stream` after what is queued on the current one.  Returns (packed uint8 codes per tensor, scales float32 [n], and the
     weights scale * Ternary(W) per tensor when want_weights)."""
     import torch
 
@@ -339,10 +361,10 @@ def aap_ternarize(tensors, delta=None, eps: float = 1e-8, want_weights: bool = F
     f32 = torch.float32
     if dev.type != "cuda":
         raise ValueError("aap_ternarize takes CUDA tensors")
-    # On the current stream the kernel reads contiguous float32 tensors where they are; anything else is
-    # put back to back first.  (60 tensors: 296 us a call, all of it host time, with the flat copy and the
-    # outputs sliced one by one; 114 us without.)
-    apart = stream is None and all(t.dtype is f32 and t.device == dev and t.is_contiguous() for t in tensors)
+    # The kernel reads contiguous float32 tensors where they are; anything else is put back to back first.
+    # (60 tensors: 296 us a call, all of it host time, with the flat copy and the outputs sliced one by one;
+    # 114 us without.)
+    apart = all(t.dtype is f32 and t.device == dev and t.is_contiguous() for t in tensors)
     flat = None if apart else torch.cat([t.reshape(-1).to(f32) for t in tensors]).contiguous()
     sizes = [t.numel() for t in tensors]
     lens = np.array(sizes, np.int64)
@@ -351,7 +373,7 @@ def aap_ternarize(tensors, delta=None, eps: float = 1e-8, want_weights: bool = F
     packed = torch.empty(total // 4, dtype=torch.uint8, device=dev)
     scale = torch.empty(len(tensors), dtype=f32, device=dev)
     wq = torch.empty(total, dtype=f32, device=dev) if want_weights else None
-    s = stream if stream is not None else torch.cuda.current_stream(dev)
+    s = _stream_of(stream, dev, (*(tensors if apart else (flat,)), packed, scale, wq))
     rest = (len(tensors), lens.ctypes.data, deltas.ctypes.data, float(eps), packed.data_ptr(), scale.data_ptr(),
             wq.data_ptr() if wq is not None else None, s.cuda_stream)
     if apart:
