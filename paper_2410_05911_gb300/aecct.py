@@ -215,7 +215,7 @@ class Decoder:
 
     decode(y) takes a float32 CUDA tensor [B, n] and returns (bits uint8 [B, n],
     syndrome uint8 [B, n-k] or None, logits float32 [B, n] or None), computed on
-    torch.cuda.current_stream().
+    torch.cuda.current_stream(), or on `stream` after what is queued there.
     """
 
     def __init__(self, model, cluster_ctas: int = 0, wait_limit_cycles: int = 0, attention_mode: int = 0):
@@ -263,7 +263,7 @@ class Decoder:
             logits = torch.empty((B, self.n), dtype=torch.float32, device=y.device) if want_logits else None
         else:
             bits, syn, logits = check_outputs(out, B, self.n, self.m, y.device)
-        s = stream if stream is not None else torch.cuda.current_stream(y.device)
+        s = _stream_of(stream, y.device, (y, bits, syn, logits))
         st = self._L.aecct_decode(self._h, y.data_ptr(), B, bits.data_ptr(), syn.data_ptr() if syn is not None else None,
                                   logits.data_ptr() if logits is not None else None, s.cuda_stream)
         _check(st, "aecct_decode")

@@ -47,3 +47,60 @@ def test_ternarize_on_another_stream(form):
     assert same([*codes, scale, *wq], want)
     del codes, scale, wq
     assert all(bool((t == 7.0).all()) for t in other)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("strided", [False, True])
+def test_decode_on_another_stream(strided):
+    model = I.random_model(I.make_code("polar64_32"), 64, 2, seed=3, spe_noise=True)
+    dec = A.Decoder(model)
+    host = torch.from_numpy(np.random.Generator(np.random.PCG64(9)).standard_normal((300, 64)).astype(np.float32)).cuda()
+    want = [t.clone() for t in dec.decode(host)]
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+
+    def late(value):
+        y = torch.zeros((300, 128 if strided else 64), device="cuda")
+        torch.cuda._sleep(DELAY)
+        part = y[:, ::2] if strided else y
+        part.copy_(value)
+        return part
+
+    got = dec.decode(late(host), stream=side)
+    side.synchronize()
+    assert same(got, want)
+    # the words go back to the allocator while the other stream has not begun
+    y = late(host)
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(DELAY)
+    got = dec.decode(y, stream=side)
+    del y
+    other = [torch.full((300, 128 if i else 64), 7.0, device="cuda") for i in range(4)]
+    torch.cuda.current_stream().synchronize()
+    side.synchronize()
+    assert same(got, want)
+    del got
+    assert all(bool((t == 7.0).all()) for t in other)
+    assert dec.synchronize() == A.AECCT_OK
+    dec.close()
+
+
+@pytest.mark.gpu
+def test_decode_captured_on_a_stream_that_is_not_current():
+    model = I.random_model(I.make_code("bch31_16"), 32, 2, seed=3, spe_noise=True)
+    dec = A.Decoder(model)
+    y = torch.from_numpy(np.random.Generator(np.random.PCG64(9)).standard_normal((40, 31)).astype(np.float32)).cuda()
+    want = [t.clone() for t in dec.decode(y)]
+    out = [torch.empty_like(t) for t in want]
+    torch.cuda.synchronize()
+    assert dec.synchronize() == A.AECCT_OK  # no status query is left for the captured call
+    side, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.stream(side):
+        graph.capture_begin()
+    dec.decode(y, out=out, stream=side)  # the current stream is not under capture
+    with torch.cuda.stream(side):
+        graph.capture_end()
+    graph.replay()
+    torch.cuda.synchronize()
+    assert same(out, want)
+    dec.close()
