@@ -263,7 +263,7 @@ class Decoder:
             logits = torch.empty((B, self.n), dtype=torch.float32, device=y.device) if want_logits else None
         else:
             bits, syn, logits = check_outputs(out, B, self.n, self.m, y.device)
-        s = _stream_of(stream, y.device, (y, bits, syn, logits))
+        s = torch.cuda.current_stream(y.device) if stream is None else _stream_of(stream, y.device, (y, bits, syn, logits))
         st = self._L.aecct_decode(self._h, y.data_ptr(), B, bits.data_ptr(), syn.data_ptr() if syn is not None else None,
                                   logits.data_ptr() if logits is not None else None, s.cuda_stream)
         _check(st, "aecct_decode")
