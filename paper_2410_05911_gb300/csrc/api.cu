@@ -35,7 +35,7 @@ struct aecct_handle {
   int Tp = 0;  // token rows per codeword (T, or T plus padding rows)
   int C = 1, G = 1, max_clusters = 0;
   int att = 0;  // kernel attention path: 0 per-row lists, 1 warp tasks, 2 per-row lists over staged rows
-  bool two_per_sm = false;  // d = 32 tasks: batches of more groups than SMs run two CTAs on each
+  bool two_per_sm = false;  // d = 32 tasks that fit twice on an SM: batches of more groups than SMs run two CTAs on each
   int alpha_mode = 0;  // 1 = one alpha per quantised matrix of a word
   int activation = 0;   // 0 = ReLU, 1 = GELU
   int linear_mode = 0;  // 0 = AAP ternary linears, 1 = full-precision (bf16) linears
@@ -524,20 +524,11 @@ int aecct_create(const aecct_model_desc *desc, aecct_handle **out) {
     g_last_error = "no cluster of this size fits on the device";
     return AECCT_ERR_UNSUPPORTED;
   }
-  // d = 32 tasks: also the kernel that fits twice on an SM (decode_params)
-  const bool two_per_sm = D == 32 && att == 1;
-  if (two_per_sm) {
-    int mc = 0;
-    e = prepare_variant(d.activation, d.linear_mode, D, 3, 1, plan_bound, &mc);
-    if (e != cudaSuccess) return cuda_fail(e, "kernel occupancy");
-  }
-
   aecct_handle *h = new aecct_handle();
   h->n = n, h->k = k, h->T = T, h->m = m, h->d = D, h->n_layers = d.n_layers, h->h_first = d.h_first;
   h->Tp = (tasks && D == 128) ? Tp128 : T;
   h->d_spe = d.d_spe, h->C = best_C, h->G = best_G, h->max_clusters = max_clusters, h->att = att;
   h->ln_eps = d.ln_eps, h->alpha_floor = d.alpha_floor, h->b_d1 = d.b_d1, h->device = dev;
-  h->two_per_sm = two_per_sm;
   h->alpha_mode = d.alpha_mode;
   h->activation = d.activation;
   h->linear_mode = d.linear_mode;
@@ -848,6 +839,17 @@ int aecct_create(const aecct_model_desc *desc, aecct_handle **out) {
       free_handle(h);
       g_last_error = "internal: the task plan exceeds its bound";
       return AECCT_ERR_UNSUPPORTED;
+    }
+    // d = 32: also the kernel that is compiled to fit twice on an SM, where its shared memory does with this
+    // plan (at four tokens a word, 35 KB of plan, it does not)
+    h->two_per_sm = D == 32 && 2u * (KernelLayout<32, 3>::kTotal + h->plan_bytes + 1024u) <= kSmemPerSm;
+    if (h->two_per_sm) {
+      int mc = 0;
+      e = prepare_variant(d.activation, d.linear_mode, D, 3, 1, h->plan_bytes, &mc);
+      if (e != cudaSuccess) {
+        free_handle(h);
+        return cuda_fail(e, "kernel occupancy");
+      }
     }
     // the plans of best_G - 1, ..., 1 words, which differ in the task list alone
     h->plans = static_cast<int>(ptask.size() / list);

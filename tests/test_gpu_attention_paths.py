@@ -248,3 +248,23 @@ def test_words_with_a_nan_among_others(key, d):
     assert nan <= 1.4 * plain, (plain, nan)
     assert dec.synchronize() == A.AECCT_OK
     dec.close()
+
+
+# two CTAs to an SM only where their shared memory fits: not with the plan of 32 words of four tokens
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,m,weight,per_sm", [(3, 1, 1, 1), (4, 1, 1, 2), (5, 2, 1, 2), (31, 15, 3, 2), (110, 18, 3, 2)])
+def test_two_ctas_per_sm_where_they_fit(n, m, weight, per_sm):
+    model = I.random_model(random_code(n, m, weight, n), 32, 2, seed=n, spe_noise=True)
+    dec = A.Decoder(model)
+    q, props = dec.query(), torch.cuda.get_device_properties(0)
+    sms, smem_sm = props.multi_processor_count, 233472  # 228 KB
+    assert q["max_clusters"] == per_sm * sms
+    assert per_sm * (q["smem_bytes"] + 1024) <= smem_sm
+    B = 2 * q["words_per_group"] * sms + 3  # more groups than SMs
+    y = np.random.Generator(np.random.PCG64(n)).standard_normal((B, n)).astype(np.float32)
+    _, _, logits = dec.decode(torch.from_numpy(y).cuda())
+    torch.cuda.synchronize()
+    assert dec.synchronize() == A.AECCT_OK
+    dec.close()
+    for part in (slice(0, 40), slice(B - 40, B)):
+        assert (logits[part].cpu().numpy().view(np.int32) == O.decode(model, y[part])["logits"].view(np.int32)).all()
