@@ -212,12 +212,17 @@ int schedule_chunks(int D, ChunkDesc *out) {
 // key step); with these rates the plans of Polar(64,32) and BCH(63,36) are still the best or equal to it.
 constexpr double kWarpIssueShare = 0.36;
 
-double scheduler_time(std::vector<long> loads) {
-  loads.erase(std::remove(loads.begin(), loads.end(), 0L), loads.end());
-  std::sort(loads.begin(), loads.end());
+double scheduler_time(const long *warp_loads, int warps) {
+  long loads[4];
+  int n = 0;  // warps with tasks, in ascending order of load (the search below comes here thousands of times)
+  for (int w = 0; w < warps; ++w) {
+    if (warp_loads[w] == 0) continue;
+    int i = n++;
+    for (; i > 0 && loads[i - 1] > warp_loads[w]; --i) loads[i] = loads[i - 1];
+    loads[i] = warp_loads[w];
+  }
   double t = 0.0;
   long done = 0;
-  const int n = static_cast<int>(loads.size());
   for (int i = 0; i < n; ++i) {
     const int k = n - i;  // warps with work left
     const double per_warp = std::min(1.0, k * kWarpIssueShare) / k;
@@ -243,7 +248,7 @@ bool assign_scheduler(const std::vector<int> &cost, int cap, std::vector<int> &o
     int cnt[4] = {0, 0, 0, 0};
     auto rec = [&](auto &&self, int i, int used) -> void {
       if (i == m) {
-        const double t = scheduler_time({load[0], load[1], load[2], load[3]});
+        const double t = scheduler_time(load, 4);
         if (t < best) best = t, out = cur;
         return;
       }
@@ -268,7 +273,7 @@ bool assign_scheduler(const std::vector<int> &cost, int cap, std::vector<int> &o
         else load[b] += cost[i], ++cnt[b], cur[i] = b;
       }
       if (!ok) continue;
-      const double t = scheduler_time(load);
+      const double t = scheduler_time(load.data(), k);
       if (t < best) best = t, out = cur;
     }
   }
@@ -735,14 +740,16 @@ int aecct_create(const aecct_model_desc *desc, aecct_handle **out) {
         std::copy(slot_of.begin(), slot_of.end(), pqslot.begin() + 4);
       }
       uint16_t *list = ptask.data() + (size_t)(words - (G - variants + 1)) * kEpiWarps * kMaxTasks;
+      std::vector<int> last, slot;  // schedulers with the same costs have the same assignment
       for (int q = 0; q < 4; ++q) {
-        std::vector<int> cost, slot;
+        std::vector<int> cost;
         for (const auto &tk : per_sched[q]) cost.push_back(tk.first);
-        if (!assign_scheduler(cost, kMaxTasks, slot)) {
+        if ((q == 0 || cost != last) && !assign_scheduler(cost, kMaxTasks, slot)) {
           free_handle(h);
           g_last_error = "attention plan: too many tasks for a warp";
           return AECCT_ERR_UNSUPPORTED;
         }
+        last = cost;
         int cnt[4] = {0, 0, 0, 0};
         for (size_t i = 0; i < per_sched[q].size(); ++i) {
           const int w = q + 4 * slot[i];

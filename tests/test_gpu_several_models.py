@@ -1,6 +1,8 @@
 """Several decoders alive at once: models of one width share their kernels and differ in the size of the
 attention plan that a launch asks shared memory for.  Creating one must not change what another's launches
 may ask for."""
+import time
+
 import numpy as np
 import pytest
 
@@ -31,3 +33,24 @@ def test_decoders_of_one_width_side_by_side(codes, d):
             assert (logits[:4].cpu().numpy().view(np.int32) == refs[i].view(np.int32)).all(), (codes[i], B)
     for dec in decs:
         dec.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d", [32, 64])
+def test_create_with_a_plan_for_every_word_count(d):
+    # 24 tokens: plans for one to five words to a CTA; a decoder without plans has the same uploads
+    code = I.ldpc_regular_code(16, 8, 3, 6, seed=1)
+    model = I.random_model(code, d, 1, seed=5, spe_noise=True, full_precision=True)
+
+    def fastest(mode):
+        times = []
+        for _ in range(20):
+            t0 = time.perf_counter()
+            st, h = A.create_handle(model, attention_mode=mode)
+            times.append(time.perf_counter() - t0)
+            assert st == A.AECCT_OK
+            A.load().aecct_destroy(h)
+        return min(times)
+
+    plans, none = fastest(2), fastest(1)
+    assert plans <= none + 0.2e-3, (plans, none)
