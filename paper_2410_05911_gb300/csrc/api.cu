@@ -63,7 +63,6 @@ struct aecct_handle {
   int *h_err = nullptr, *d_err = nullptr;
   cudaEvent_t ev = nullptr;
   bool ev_pending = false;
-  int pending_status = AECCT_OK;
   // capture
   int64_t cap_B = 0;
   int8_t *cap_q = nullptr;
@@ -988,11 +987,7 @@ static int check_device(const aecct_handle *h, const char *who) {
 }
 
 static int collect_status(aecct_handle *h, bool block) {
-  if (!h->ev_pending) {
-    const int s = h->pending_status;
-    h->pending_status = AECCT_OK;
-    return s;
-  }
+  if (!h->ev_pending) return AECCT_OK;
   cudaError_t e = block ? cudaEventSynchronize(h->ev) : cudaEventQuery(h->ev);
   if (e == cudaErrorNotReady) return AECCT_OK;
   h->ev_pending = false;

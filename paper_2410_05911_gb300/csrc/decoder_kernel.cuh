@@ -1005,21 +1005,19 @@ struct Issuer<128, ATT> {
   }
 };
 
-// the largest row maximum of word w (a whole warp)
-__device__ __forceinline__ void word_maximum(const float *rowmax, float *wordmax, int w, int rows, int lane) {
-  float a = 0.0f;
-  for (int i = lane; i < rows; i += 32) a = fmaxf(a, rowmax[w * rows + i]);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
-  if (lane == 0) wordmax[w] = a;
-}
-// Every word's, the words in turn over the warps.  Out of line: only one alpha per word (alpha_mode 1) takes
+// The largest row maximum of every word, the words in turn over the warps.  Out of line: only one alpha per word (alpha_mode 1) takes
 // it, and inlined at its four places it cost every block instruction fetches and registers (LDPC(128,64)
 // 327.8 -> 318.9 ms, LDPC(384,192) 143.7 -> 139.2, BCH(63,36) 489.7 -> 482.9, Polar(64,32) 45.04 -> 44.49).
 // The barriers around it as well: Polar(64,32) 0.2% faster, BCH(63,36) 2.7% slower.
 static __device__ __noinline__ void word_maxima(const float *rowmax, float *wordmax, int words, int rows, int warp) {
-  for (int w = warp; w < words; w += kEpiWarps)
-    word_maximum(rowmax, wordmax, w, rows, static_cast<int>(threadIdx.x & 31u));
+  const int lane = static_cast<int>(threadIdx.x & 31u);
+  for (int w = warp; w < words; w += kEpiWarps) {
+    float a = 0.0f;
+    for (int i = lane; i < rows; i += 32) a = fmaxf(a, rowmax[w * rows + i]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
+    if (lane == 0) wordmax[w] = a;
+  }
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1168,15 +1166,14 @@ __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) ae
     auto word_max = [&](float a_row, bool publish, int row, int gw) -> float {
       if (publish) rowmax_s[row] = a_row;
       named_bar_sync(5, kEpiThreads);
-      if constexpr (ATT == 1 && D == 128) {  // one word to a CTA
-        if (warp == 0) word_maximum(rowmax_s, wordmax_s, 0, p.Tp, lane);
-      } else {
-        word_maxima(rowmax_s, wordmax_s, p.G, p.Tp, warp);
-      }
+      word_maxima(rowmax_s, wordmax_s, p.G, p.Tp, warp);
       named_bar_sync(5, kEpiThreads);
       return gw < p.G ? wordmax_s[gw] : a_row;
     };
-    auto word_alpha = [&](float a_row) -> float { return p.alpha_mode == 0 ? a_row : word_max(a_row, sl == 0, r, g); };
+    auto word_alpha = [&](float a_row) -> float {
+      if constexpr (TASKS && D == 128) return a_row;  // (one alpha per row: aecct_create refuses the other)
+      else return p.alpha_mode == 0 ? a_row : word_max(a_row, sl == 0, r, g);
+    };
     auto row_sum = [&](float v) -> float {
       *red.slot(sl, r) = v;
       named_bar_sync(qbar, 128);
