@@ -1690,6 +1690,7 @@ __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) ae
           // LDPC(128,64) 330.4 -> 327.8 ms, at d = 64 17.2 -> 16.3 ms.
           constexpr uint32_t kRowBytes = 4u * DH;
           fence_proxy_async_smem();  // this thread's K / V stores, before the bulk copies read them
+          tc_fence_before();  // and its reads of the K and V accumulators, before scores go over them
           __syncwarp();
           if (lane == 0) {
             const uint32_t blk = blk_base + static_cast<uint32_t>(l);
@@ -1849,8 +1850,10 @@ __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) ae
               row_max4();
               fold16(0, sg);
             } else {
-              // the scores in this thread's own TMEM lane, 4 columns a block from column kSc + 64 sl (at most
-              // 256 keys), in columns whose accumulators are dead (d = 128) or that hold none (d = 64)
+              // the scores in this thread's own TMEM lane, 4 columns a block from column kRowCacheCol + 64 sl (at
+              // most 256 keys), in columns whose accumulators are dead (d = 128) or that hold none (d = 64):
+              // the rows that have landed here were sent after every warp had read its K and V accumulators
+              tc_fence_after();
               const uint32_t tsc = tl + L::kRowCacheCol + 64u * static_cast<uint32_t>(sl);
 #pragma unroll 1
               for (int b = 0; b < nmax; b += 16) {
