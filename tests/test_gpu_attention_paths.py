@@ -268,3 +268,51 @@ def test_two_ctas_per_sm_where_they_fit(n, m, weight, per_sm):
     dec.close()
     for part in (slice(0, 40), slice(B - 40, B)):
         assert (logits[part].cpu().numpy().view(np.int32) == O.decode(model, y[part])["logits"].view(np.int32)).all()
+
+
+# staged attention against the oracle: both widths (d = 64 takes it by default only), short lists and long ones
+@pytest.mark.gpu
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("mask_mode", [0, 1])
+def test_staged_attention_matches_oracle(mask_mode, d):
+    model = I.random_model(I.make_code("ldpc128_64"), d, 2, seed=11, spe_noise=True)
+    model.mask_mode = mask_mode
+    y = np.random.Generator(np.random.PCG64(12)).standard_normal((7, model.n)).astype(np.float32)
+    dec = A.Decoder(model)
+    assert dec.query()["attention_mode"] == 3
+    bits, syn, logits = dec.decode(torch.from_numpy(y).cuda())
+    torch.cuda.synchronize()
+    assert dec.synchronize() == A.AECCT_OK
+    dec.close()
+    r = O.decode(model, y)
+    assert (logits.cpu().numpy().view(np.int32) == r["logits"].view(np.int32)).all()
+    assert (bits.cpu().numpy() == r["bits"]).all() and (syn.cpu().numpy() == r["syndrome"]).all()
+
+
+# full-precision linears: the attention outputs go to the O GEMM as bf16, by another store
+@pytest.mark.gpu
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("mask_mode", [0, 1])
+def test_staged_attention_with_full_precision_linears_equals_per_row_walk(mask_mode, d):
+    model = I.random_model(I.make_code("ldpc128_64"), d, 2, seed=13, spe_noise=True, activation=mask_mode, full_precision=True)
+    model.mask_mode = mask_mode
+    got = both(model, 107, seed=14)
+    assert got[0][3] == 3 and got[1][3] == 1
+    same(got)
+
+
+# one alpha per quantised matrix of a word through the staged path's own exchange, several words to a CTA
+@pytest.mark.gpu
+@pytest.mark.parametrize("key,words", [("hamming7_4", 12), ("bch31_16", 2), ("polar64_32", 1)])
+def test_staged_attention_with_word_alpha_matches_oracle(key, words):
+    model = I.random_model(I.make_code(key), 128, 2, seed=15, spe_noise=True)
+    model.alpha_mode = 1
+    dec = A.Decoder(model, attention_mode=3)
+    q = dec.query()
+    assert (q["attention_mode"], q["words_per_group"]) == (3, words)
+    y = np.random.Generator(np.random.PCG64(16)).standard_normal((2 * words + 1, model.n)).astype(np.float32)
+    _, _, logits = dec.decode(torch.from_numpy(y).cuda())
+    torch.cuda.synchronize()
+    assert dec.synchronize() == A.AECCT_OK
+    dec.close()
+    assert (logits.cpu().numpy().view(np.int32) == O.decode(model, y)["logits"].view(np.int32)).all()

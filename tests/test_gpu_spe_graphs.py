@@ -95,3 +95,37 @@ def test_table_over_score_ranges(scale):
     own = spe.spe_from_eigenpairs(lam_g, U_g, p)
     size = 1 + np.abs(ref).max()
     assert np.abs(t64 - own).max() <= 64 * EPS * size * max(1.0, 16.0 * scale * scale)
+
+
+def _attention(lam, U, p, nodes):
+    """SPE rows of `nodes` by the definition, and the largest score."""
+    heads, d_e = p.wq.shape[0], p.wq.shape[2]
+    rows, top = [], 0.0
+    for j in nodes:
+        X = np.stack([lam, U[j]], 1) @ p.w_pe
+        parts = []
+        for e in range(heads):
+            S = (X @ p.wq[e]) @ (X @ p.wk[e]).T / np.sqrt(d_e)
+            top = max(top, np.abs(S).max())
+            P = np.exp(S - S.max(1, keepdims=True))
+            parts.append((P / P.sum(1, keepdims=True) @ (X @ p.wv[e])).mean(0))
+        rows.append(np.concatenate(parts) @ p.wo)
+    return np.array(rows), top
+
+
+# past 576 nodes a thread takes several rows; the larger scales reach the wide fixed-point rows and the double ones
+@pytest.mark.gpu
+@pytest.mark.parametrize("name", ["random 300", "ldpc 450", "ldpc 690", "wide star", "ldpc 1020"])
+@pytest.mark.parametrize("scale", [1.0, 8.0, 40.0])
+def test_table_of_long_codes_on_sampled_nodes(name, scale):
+    H = GRAPHS[name]
+    T = sum(H.shape)
+    p = I.spe_params(H, 8, seed=4)
+    p.wq, p.wk = p.wq * scale, p.wk * scale
+    tab, t64, lam, U = A.spe_table(H, p, want_eigen=True)
+    nodes = [0, 1, T // 3, T // 2, T - 2, T - 1]
+    ref, top = _attention(lam, U, p, nodes)
+    # the error of a probability is that of its score, 2^-52 of the largest score or more
+    bound = 64 * EPS * (1 + np.abs(ref).max()) * max(1.0, top)
+    assert np.abs(t64[nodes] - ref).max() <= bound
+    assert np.abs(tab - t64).max() <= 1e-7 * (1 + np.abs(t64).max())

@@ -46,3 +46,24 @@ def test_short_wait_limit_reports_timeout_and_context_survives(key, B, cluster_c
     assert (logits.cpu().numpy().view(np.int32) == ref["logits"].view(np.int32)).all()
     assert (bits.cpu().numpy() == ref["bits"]).all() and (syn.cpu().numpy() == ref["syndrome"]).all()
     dec.close()
+
+
+@pytest.mark.gpu
+def test_short_wait_limit_in_staged_attention_at_d_64():
+    # bulk copies of K and V rows and the cluster's signals in flight when the first wait gives up
+    model = I.random_model(I.make_code("ldpc128_64"), 64, 2, seed=17, spe_noise=True)
+    y = np.random.Generator(np.random.PCG64(18)).standard_normal((300, model.n)).astype(np.float32)
+    yt = torch.from_numpy(y).cuda()
+    short = A.Decoder(model, wait_limit_cycles=1)
+    assert short.query()["attention_mode"] == 3
+    short.decode(yt)
+    torch.cuda.synchronize()
+    assert short.synchronize() == A.AECCT_ERR_TIMEOUT
+    assert short.synchronize() == A.AECCT_OK
+    short.close()
+    dec = A.Decoder(model)
+    _, _, logits = dec.decode(yt[:5])
+    torch.cuda.synchronize()
+    assert dec.synchronize() == A.AECCT_OK
+    dec.close()
+    assert (logits.cpu().numpy().view(np.int32) == O.decode(model, y[:5])["logits"].view(np.int32)).all()
