@@ -411,13 +411,18 @@ def run_cuda(args, rank, world, local_rank):
                     "is one op); peak = fp32 FMA rate measured on this GPU by aecct_selftest_fma_rate (the larger "
                     f"of scalar {alu_rates['scalar']:.1f} and paired {alu_rates['paired']:.1f} T FMA/s; nominal "
                     f"152 SMs x 128 lanes x 2070 MHz = {ALU_NOMINAL_TOPS:.1f})")
+    # the kernel's attention path: 0 per-row lists, 1 warp tasks, 2 staged rows, 3 warp tasks at two CTAs per SM
+    path = {1: 0, 2: 1, 3: 2}[q["attention_mode"]]
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    if path == 1 and q["max_clusters"] > sms and B > sms * q["words_per_group"]:
+        path = 3
     # d <= 64: the fp32 work (HPSA, epilogues) binds; d = 128: the linear layers' contraction
     roof = dict(alu if w.d <= 64 else tensor)
     roof.update(traffic=args.traffic if args.traffic is not None else
                 (measured_traffic(args.workload, B) if args.variant == "aecct" else None),
-                kernel=f"aecct_decoder_kernel<{w.d}, {int(q['attention_mode'] == 2)}, {model.activation}, "
-                       f"{model.linear_mode}>",
-                other={k: v for k, v in (("tensor", tensor), ("alu", alu)) if v["bound"] != roof["bound"]})
+                kernel=f"aecct_decoder_kernel<{w.d}, {path}, {model.activation}, {model.linear_mode}, "
+                      f"{int(path in (0, 2))}>",
+               other={k: v for k, v in (("tensor", tensor), ("alu", alu)) if v["bound"] != roof["bound"]})
     cpu = None
     parity = None
     if not args.no_cpu_baseline:

@@ -190,7 +190,7 @@ struct DecodeParams {
   // pieces of a row in the order of kv_piece
   float *kv_scratch;
   // control
-  int *err;  // device word, bit 0 = a bounded wait timed out
+  int *err;  // the call's status word (the handle's pinned host word, or device scratch): 1 = a bounded wait timed out
   long long wait_limit;
 };
 

@@ -208,7 +208,9 @@ int schedule_chunks(int D, ChunkDesc *out) {
 // in the walk (Polar(64,32): its tasks on three warps per scheduler decoded 2.2% faster than on four with
 // unequal loads, whose tail leaves one warp alone).  The branch-free walk of 63 keys at d_h = 16 runs at
 // 0.66, 0.85, 0.97 and 1 of four warps' rate on one, two, three and four warps (117, 90, 79 and 77 cycles a
-// key step); with these rates the plans of Polar(64,32) and BCH(63,36) are still the best or equal to it.
+// key step), where the model says 0.36, 0.72, 1 and 1: it is too hard on schedulers with few warps.  With the
+// measured rates the full plans of Polar(64,32) and BCH(63,36) are the best or equal to it; other codes' plans,
+// and those of fewer words a CTA, were not compared.
 constexpr double kWarpIssueShare = 0.36;
 
 double scheduler_time(const long *warp_loads, int warps) {
@@ -935,7 +937,8 @@ static int launch_att(const aecct_handle *h, const DecodeParams &p) {
 // Words per CTA of a launch.  Warp tasks of small codes have room for several words in a CTA; where the
 // batch leaves SMs idle, fewer words a CTA spread it over them, and each CTA has less attention to do.
 // BCH(31,16) (T = 46, two words to a CTA) at d = 32: one word 28.5 -> 26.7 us, 100 words 32.0 -> 27.0 us; at
-// d = 64, six blocks: 100.3 -> 83.0 and 100.5 -> 84.0 us.
+// d = 64, six blocks: 100.3 -> 83.0 and 100.5 -> 84.0 us.  The smallest number that covers the batch in one wave of
+// one CTA per SM; two of the smaller CTAs on an SM (d = 32, from 153 to 304 words of such a code) were not tried.
 static int launch_words(const aecct_handle *h, int64_t B) {
   if (h->plans == 1 || B >= static_cast<int64_t>(h->G) * h->max_clusters) return h->G;
   const int64_t g = (B + h->max_clusters - 1) / h->max_clusters;
@@ -972,8 +975,8 @@ static DecodeParams decode_params(const aecct_handle *h, int64_t B, const float 
   return p;
 }
 
-// The handle's model, plan and status word live on the device that was current at create; a
-// decode launched while another device is current would read them from the wrong GPU.
+// The handle's model and plan live on the device that was current at create (its status word in pinned host
+// memory); a decode launched while another device is current would read them from the wrong GPU.
 static int check_device(const aecct_handle *h, const char *who) {
   int dev = -1;
   const cudaError_t e = cudaGetDevice(&dev);

@@ -1459,9 +1459,9 @@ __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) ae
           named_bar_sync(5, kEpiThreads);  // every Q, K, V row of this CTA is in shared memory
           tc_fence_after();
           // this warp's score cache: its lane quadrant, kTaskCache columns (SmemLayout).
-          // d = 128: a task's 32 rows are this warp's TMEM lane quadrant (the plan keeps every task on
-          // a warp of its group's quadrant); Q comes from the QKV accumulators of this thread's row
-          // and the output goes back over them
+          // d = 128: where a task's 32 rows are this warp's TMEM lane quadrant, Q comes from the QKV
+          // accumulators of this thread's row and the output goes back over them; a task that the plan
+          // gives to another quadrant's warp has both in a slot of stage W2
           const uint32_t tcache = tmem + (static_cast<uint32_t>(32 * (warp & 3)) << 16) + L::task_cache_col(warp >> 2);
           auto run_tasks = [&](auto own_tag) {
             for (int k = 0; k < kMaxTasks; ++k) {

@@ -403,7 +403,9 @@ __global__ void __launch_bounds__(256) gram_kernel(const double *__restrict__ V,
 // panel, and the trailing triangle takes the panel's update in one pass.
 constexpr int kCholThreads = 512;
 constexpr int kCholPanel = 16;
-constexpr int kCholShared = 216;  // rows of a triangle in shared memory: 187,488 bytes
+// rows of a triangle in shared memory: 187,488 bytes (up to 237 would fit; larger clusters' Cholesky works in global memory
+// and their node choice one by one, 690 nodes with a cluster of 230 take 54 ms, 576 with 192 take 17)
+constexpr int kCholShared = 216;
 constexpr size_t kCholSmem = sizeof(double) * kCholShared * (kCholShared + 1) / 2;
 __global__ void __launch_bounds__(kCholThreads) chol_kernel(double *Gm, const int *__restrict__ gs,
                                                             const int *__restrict__ gn, int T, int rmin, double thr,
@@ -849,13 +851,15 @@ struct MhsaCoef {
 
 // The fixed-point form of a node's attention.  Double operations are 64 times scarcer than integer ones on
 // this GPU, and the T^2 exponentials of a node and head take about 27 of them each, so the softmax runs on
-// 64-bit integers, with no less precision: scores in base 2 to 2^-52 (a double score of magnitude 8 or
-// more is rounded to 2^-50; 2^-48 past +-1024, where doubles keep 2^-43), exponentials and their products to 2^-64 of the row's largest one, sums
-// exact in 96 bits.  With l = lambda / 2^el and v = u / 2^eu in (-1, 1), a row's scores are
+// 64-bit integers: scores in base 2 to 2^-52, 2^-48 in a row whose coefficients pass 2^9 (a double score of magnitude
+// 8 or more is rounded to 2^-50, past 1024 to 2^-43, one near zero more finely than either), exponentials to about 2^-53
+// of the row's largest one (double table entries and the series below), they and their products held with 64
+// fraction bits of it (fewer significant ones the smaller they are), sums exact in 96 bits.  The table's error
+// against 64 bits is that of double operations (2.5e-8 in fp32).  With l = lambda / 2^el and v = u / 2^eu in (-1, 1), a row's scores are
 // A (l_k - l_min) / 2 + B (v_k + 1) / 2 up to a constant, which a softmax does not see; |A| and |B| are
 // scaled by 2^(63 - er) to fill 63 bits.
-// |A|, |B| < 2^9 (scores within +-1024): 52 fraction bits; < 2^13: 48, still more than a double of that size
-// holds; a wider row takes doubles, whose warp then takes 20 times as long as the others
+// |A|, |B| < 2^9 (scores within +-1024): 52 fraction bits; < 2^13: 48, more than a double of that size holds (its
+// scores near zero keep fewer than a double would); a wider row takes doubles, whose warp then takes 20 times as long as the others
 constexpr int kFixNarrow = 9, kFixWide = 13;
 struct FixKey {
   uint64_t l, v;  // (l - l_min) / 2 and (v + 1) / 2, 64 fraction bits
@@ -1160,6 +1164,7 @@ cudaError_t run_spe_table(const uint8_t *H, int n, int m, int d_spe, int heads, 
   overlap_kernel<<<dim3(nt, nt), 256>>>(U, T, again, Gm, busy, again);
   polish_kernel<<<dim3(nt, nt), 256>>>(U, Gm, busy, T, again, X);
   if (T > 3) pair_kernel<<<T - 3, 32>>>(V, T, pbuf);  // (pbuf: the reduction is done with it)
+  // (32 elements a lane spill 812 bytes a thread; they serve every T past 576)
   if (T <= 128) back_kernel<4><<<(T + 1) / 2, 64>>>(V, tau, pbuf, T, X);
   else if (T <= 320) back_kernel<10><<<(T + 1) / 2, 64>>>(V, tau, pbuf, T, X);
   else if (T <= 576) back_kernel<18><<<(T + 1) / 2, 64>>>(V, tau, pbuf, T, X);
