@@ -624,6 +624,12 @@ __device__ __forceinline__ void hpsa_task(const float *q, const uint4 mask, int 
   for (int i = 0; i < DH; ++i) A[i] = __fmul_rn(num[i], inv);
 }
 
+// The named barrier at which the other warps wait for warp 0, which waits for the accumulators itself and only
+// arrives there.  It is not the CTA-wide barrier 5: after QKV warp 0 goes on to that one with nothing in between, and
+// its two arrivals would complete a phase that a late warp had not reached (barriers count arrivals, not
+// warps).  Warp 0's next arrival here follows the next operand, which every warp publishes after this wait.
+constexpr uint32_t kAccBar = 6;
+
 // ------------------------------------------------------------------------------------------
 // weight streaming and tensor-core issue (run by warp 0 of each CTA)
 // ------------------------------------------------------------------------------------------
@@ -667,7 +673,7 @@ struct Issuer {
   __device__ __forceinline__ uint32_t bar_op() const { return sb + L::kOffBar + 16 * S; }
   __device__ __forceinline__ uint32_t bar_acc() const { return sb + L::kOffBar + 16 * S + 8; }
   // the accumulators are complete: let the CTA's other warps (waiting in wait_acc) go
-  __device__ __forceinline__ static void release_acc() { named_bar_arrive(5, kEpiThreads); }
+  __device__ __forceinline__ static void release_acc() { named_bar_arrive(kAccBar, kEpiThreads); }
 
   // whole warp: lane 0 polls (the slow path is bounded and raises the abort flag), then the
   // warp reconverges
@@ -801,7 +807,7 @@ struct Issuer<128, ATT> {
   // FFN1's N tiles 0 and 1 (hidden units [0, 256)) are complete: once per block
   __device__ __forceinline__ uint32_t bar_acc_lo() const { return sb + L::kOffBar + 160; }
   // the accumulators are complete: let the CTA's other warps (waiting in wait_acc) go
-  __device__ __forceinline__ static void release_acc() { named_bar_arrive(5, kEpiThreads); }
+  __device__ __forceinline__ static void release_acc() { named_bar_arrive(kAccBar, kEpiThreads); }
 
   // slot of chunk P: shared-memory offset, barrier id, uses of that barrier per block, use index
   struct Slot {
@@ -1230,7 +1236,7 @@ __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) ae
     // accumulators of the last GEMM are complete once warp 0, which waited for them in its
     // gemm<G> call and then arrived at this barrier, releases it
     auto wait_acc = [&]() {
-      if (warp != 0) named_bar_sync(5, kEpiThreads);
+      if (warp != 0) named_bar_sync(kAccBar, kEpiThreads);
       tc_fence_after();
     };
     // wait for a cluster-wide phase: thread 0 waits on the mbarrier, the others in a named barrier
