@@ -467,7 +467,7 @@ __device__ __forceinline__ bool contiguous(const uint4 &w) {
 // each query the max, the sum l and the weighted sum num see its keys in ascending order, as in
 // the canonical definition, without a branch per key.  V has to be finite; where a V row of the CTA is not
 // (a word with a NaN, parameters near the end of the fp32 range), OWN = 1: a branch around every fold, so
-// that an infinity stays with the queries that attend to it.
+// that an infinity stays with the queries that attend to it, and one form of block to keep that copy small.
 // Keys go U at a time; the two lanes of a paired instruction are independent computations, and the
 // folds into l and num stay sequential in key order.
 // Bound by issue slots, FMA pipe and shared-memory loads at 50 to 70% each.  With a divergent branch
@@ -539,7 +539,7 @@ __device__ __forceinline__ void hpsa_task(const float *q, const uint4 mask, int 
         }
       }
     };
-    if (contiguous(w)) {
+    if (!OWN && contiguous(w)) {
       if (nk >= 16 && __all_sync(0xffffffffu, (seg & 0xFFFFu) == 0xFFFFu)) block(std::true_type{}, std::true_type{});
       else block(std::true_type{}, std::false_type{});
     } else {
@@ -597,7 +597,7 @@ __device__ __forceinline__ void hpsa_task(const float *q, const uint4 mask, int 
           }
         }
       };
-      if (contiguous(w)) block(std::true_type{});
+      if (!OWN && contiguous(w)) block(std::true_type{});
       else block(std::false_type{});
     } else {
 #pragma unroll
@@ -1532,7 +1532,7 @@ __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) ae
             }
           };
           // V rows that are not finite take a second copy of the loop.  4,096 words of Polar(64,32) (three blocks),
-          // a NaN in each: 1.49 ms, 1.44 without the NaN; 2.96 in a walk key by key.  The copy costs the words
+          // a NaN in each: 1.55 ms, 1.44 without the NaN; 2.96 in a walk key by key.  The copy costs the words
           // of the first one 0.9% at d = 64 (Polar(64,32) 43.8 -> 44.2 ms) and nothing at d = 32 and 128; a
           // call out of line from the loop 2.1%, a test around the second pass alone 1.2%.
           if (*s_vbad == 0) run_tasks(std::integral_constant<int, 0>{});
@@ -2012,10 +2012,14 @@ __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) ae
           auto put_operand = [&](int ch, const uint32_t *w) {
             tmem_st_u32<16>(tl + 64 * sl + 16 * ch, w);
           };
+          // the d = 64 tasks loop over their two chunks: less code and no spills (Polar(64,32) 44.43 -> 43.83
+          // ms; with full-precision linears and ReLU 41.11 -> 40.55, with GELU 76.52 -> 77.15: unrolled); unrolled
+          // elsewhere (BCH(63,36) 483.0 ms, 487.2 in a loop; LDPC(384,192) 139.5, 141.0)
+          constexpr int kUnroll = D == 64 && ATT == 1 && (LIN == 0 || ACT == 0) ? 1 : NCH;
           if constexpr (LIN == 1) {
             // peers have finished reading this CTA's K/V: the shared region may now take u
             if constexpr (ATT == 0) cluster_wait(bar_kvf, kvf_ph);
-#pragma unroll
+#pragma unroll kUnroll
             for (int ch = 0; ch < NCH; ++ch) {
               wait_chunk(ch);
               float u[CH];
@@ -2032,9 +2036,6 @@ __global__ void __launch_bounds__(kThreads, KernelLayout<D, ATT>::kCtasPerSm) ae
             if constexpr (D == 128) tmem_wait_st();
           } else {
             float umax = 0.0f;
-            // the d = 64 tasks loop over their two chunks: less code and no spills (Polar(64,32) 44.43 -> 43.83
-            // ms); unrolled elsewhere (BCH(63,36) 483.0 ms, 487.2 in a loop; LDPC(384,192) 139.5, 141.0)
-            constexpr int kUnroll = D == 64 && ATT == 1 ? 1 : NCH;
 #pragma unroll kUnroll
             for (int ch = 0; ch < NCH; ++ch) {
               wait_chunk(ch);
